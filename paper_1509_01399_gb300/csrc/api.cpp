@@ -1296,11 +1296,11 @@ hyb_status misfit_impl(hyb_mesh* m, const T* trace, const T* obs, int weights, d
   g.wt = quad ? m->dt : 1.0;
   for (int s = 0; s < m->nsrc; ++s) g.hh[s] = quad ? face_cell_area(m, m->src[s].face) : 1.0;
   g.halve = quad ? 1 : 0;
-  HYB_TRY(ensure(m, m->part, 2 * (size_t)kReduceBlocks * sizeof(double)));
+  HYB_TRY(ensure(m, m->part, (size_t)misfit_parts(g) * sizeof(double)));
   HYB_TRY(ensure(m, m->scal, 16 * sizeof(double)));
-  launch_misfit<T>(g, trace, obs, cot, (double*)m->part.p, m->st);
+  const int parts = launch_misfit<T>(g, trace, obs, cot, (double*)m->part.p, m->st);
   HYB_LAUNCHED(m);
-  launch_sum((double*)m->part.p, kReduceBlocks, (double*)m->scal.p + 8, m->st);
+  launch_sum((double*)m->part.p, parts, (double*)m->scal.p + 8, m->st);
   HYB_LAUNCHED(m);
   if (J) {
     HYB_CU(cudaMemcpyAsync(m->hscal + 8, (double*)m->scal.p + 8, sizeof(double), cudaMemcpyDeviceToHost, m->st));
@@ -1318,7 +1318,6 @@ hyb_status misfit_batch_impl(hyb_mesh* m, const T* trace, const T* obs, int weig
   if (!m->have_run) return fail(HYB_ERR_STATE, "hyb_misfit_batch needs a preceding forward");
   const int nsrc = m->nsrc;
   const size_t rows = (size_t)(m->nsteps + 1) * m->obs_stride;
-  HYB_TRY(ensure(m, m->part, 2 * (size_t)kReduceBlocks * sizeof(double)));
   HYB_TRY(ensure(m, m->scal, (16 + kMaxSlots) * sizeof(double)));
   double* out = (double*)m->scal.p + 16;
   const bool quad = weights == HYB_WEIGHTS_QUADRATURE;
@@ -1335,9 +1334,11 @@ hyb_status misfit_batch_impl(hyb_mesh* m, const T* trace, const T* obs, int weig
     g.wt = quad ? m->dt : 1.0;
     g.hh[0] = quad ? face_cell_area(m, m->src[s].face) : 1.0;
     g.halve = quad ? 1 : 0;
-    launch_misfit<T>(g, trace + s * rows, obs + s * rows, cot ? cot + s * rows : nullptr, (double*)m->part.p, m->st);
+    HYB_TRY(ensure(m, m->part, (size_t)misfit_parts(g) * sizeof(double)));
+    const int parts =
+        launch_misfit<T>(g, trace + s * rows, obs + s * rows, cot ? cot + s * rows : nullptr, (double*)m->part.p, m->st);
     HYB_LAUNCHED(m);
-    launch_sum((double*)m->part.p, kReduceBlocks, out + s, m->st);
+    launch_sum((double*)m->part.p, parts, out + s, m->st);
     HYB_LAUNCHED(m);
   }
   if (J_host) {
@@ -1364,7 +1365,7 @@ hyb_status cg_impl(hyb_mesh* m, double* a, const T* obs, const hyb_source* src, 
   HYB_TRY(ensure(m, m->cot, tb));
   HYB_TRY(ensure(m, m->g, (size_t)nu * sizeof(double)));
   HYB_TRY(ensure(m, m->atrial, (size_t)nu * sizeof(double)));
-  HYB_TRY(ensure(m, m->part, kCgParts * (size_t)kReduceBlocks * sizeof(double)));
+  HYB_TRY(ensure(m, m->part, (size_t)std::max(kMisfitParts, kCgParts * kReduceBlocks) * sizeof(double)));
   HYB_TRY(ensure(m, m->scal, 16 * sizeof(double)));
   double* part = (double*)m->part.p;
   double* scal = (double*)m->scal.p;

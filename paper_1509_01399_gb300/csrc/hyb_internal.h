@@ -220,9 +220,11 @@ struct MisfitGeom {
   double hh[kMaxSlots];              // face weight scale per source (1, or the in-face cell area)
   int halve;                         // halve the face weight on the face border
 };
+// Returns the number of partials written, at most misfit_parts(g).
+constexpr int kMisfitParts = 4096;
+long long misfit_parts(const MisfitGeom& g);
 template <typename T>
-void launch_misfit(const MisfitGeom& g, const T* trace, const T* obs, T* cot, double* partials,
-                   cudaStream_t st);
+int launch_misfit(const MisfitGeom& g, const T* trace, const T* obs, T* cot, double* partials, cudaStream_t st);
 // out[0] = sum of `n` partials (one block, fixed order).
 void launch_sum(const double* partials, int n, double* out, cudaStream_t st);
 // g = scale * sum_s G_s + gamma * vol * (a - a0), G holding n_src arrays of n

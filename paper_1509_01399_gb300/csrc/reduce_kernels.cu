@@ -50,37 +50,93 @@ __device__ double block_max(double v) {
   return v;
 }
 
+// FP64-pipe operations that the misfit's FP32 traces seldom need, out of line so
+// that the common path does not carry them.
+__device__ __noinline__ double widen_any(float x) { return (double)x; }
+__device__ __noinline__ float product_any(double w, double d) { return (float)(w * d); }
+
+// x in FP64: for normal numbers and zeros by moving its bits (the conversion
+// instruction runs in the FP64 pipe).
+__device__ __forceinline__ double widen(float x) {
+  const unsigned u = __float_as_uint(x), a = u & 0x7fffffffu;
+  if (a - 1u < 0x007fffffu || a >= 0x7f800000u) return widen_any(x);  // subnormal, infinite, NaN
+  const unsigned hi = a == 0u ? 0u : (a >> 3) + 0x38000000u;          // exponent bias 1023 - 127
+  return __hiloint2double((int)(hi | (u & 0x80000000u)), (int)(a << 29));
+}
+__device__ __forceinline__ double widen(double x) { return x; }
+
+// w (a - b) rounded to FP32, w = wh + wl and d = a - b: the difference as s + e
+// and the leading product as p + q exactly, the small terms summed before they
+// meet p (within 2^-46 of the rounded FP64 product); the FP64 product where the
+// error terms would not be exact.
+__device__ __forceinline__ float product(float a, float b, float wh, float wl, double w, double d) {
+  const float s = a - b, v = s - a, e = (a - (s - v)) + (-b - v);
+  const float p = wh * s;
+  if (!(fabsf(p) > 1e-30f && fabsf(p) < 1e30f && fabsf(s) < 1e30f) && s != 0.f) return product_any(w, d);
+  return p + (fmaf(wh, s, -p) + (wl * s + wh * e));
+}
+__device__ __forceinline__ double product(double, double, float, float, double w, double d) { return w * d; }
+
+// Misfit of one block of trace rows (blockIdx.y: `rows` of them, blockIdx.z:
+// source) and kMisfitCols columns per thread, kReduceThreads apart, so that a
+// thread's face weights stay in registers over its rows.  The FP64 pipe (two
+// lanes per SM and clock) bounds it before the three trace-sized streams do, so
+// an entry gives it only the difference and its square's accumulation
+// (weighted once at the end); FP32 traces are widened by integer moves and their
+// cotangent formed from exact FP32 splits.  Eight sources x 601 rows of 16,641
+// entries, FP32, with the cotangent (0.96 GB): 2.09 ms with index divisions and
+// seven FP64-pipe operations an entry, 1.01 ms with six and no divisions,
+// 0.38 ms so (four columns a thread: 0.94 ms, the calls out of line spill).
+constexpr int kMisfitCols = 2;
+
 template <typename T>
-__global__ void __launch_bounds__(kReduceThreads) misfit_kernel(const MisfitGeom g, const T* __restrict__ trace,
+__global__ void __launch_bounds__(kReduceThreads) misfit_kernel(const MisfitGeom g, int rows,
+                                                                const T* __restrict__ trace,
                                                                 const T* __restrict__ obs, T* __restrict__ cot,
                                                                 double* __restrict__ partials) {
-  const long long rows = (long long)g.n_src * (g.nsteps + 1);
-  const long long total = rows * g.stride;
-  double acc = 0.0;
-  for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < total;
-       e += (long long)gridDim.x * blockDim.x) {
-    const int jj = (int)(e % g.stride);
-    const long long r = e / g.stride;
-    const int k = (int)(r % (g.nsteps + 1));
-    const int s = (int)(r / (g.nsteps + 1));
-    const int np = g.np[s], nq = g.nq[s];
-    T cv = T(0);
-    if (k >= 1 && jj < np * nq) {
-      double m = g.hh[s];
-      if (g.halve) {
-        const int cp = jj % np, cq = jj / np;
-        if (cp == 0 || cp == np - 1) m *= 0.5;
-        if (cq == 0 || cq == nq - 1) m *= 0.5;
-      }
-      const double d = (double)trace[e] - (double)obs[e];
-      const double w = g.wt * m;
-      acc += 0.5 * w * d * d;
-      cv = (T)(w * d);
+  const int s = (int)blockIdx.z;
+  const int np = g.np[s], n = np * g.nq[s];
+  const int c0 = (int)blockIdx.x * (kReduceThreads * kMisfitCols) + (int)threadIdx.x;
+  double w[kMisfitCols], sq[kMisfitCols];
+  float wh[kMisfitCols], wl[kMisfitCols];
+#pragma unroll
+  for (int q = 0; q < kMisfitCols; ++q) {
+    const int jj = c0 + q * kReduceThreads;
+    double m = jj < n ? g.hh[s] : 0.0;  // (row padding: weight 0)
+    if (g.halve && jj < n) {
+      const int cp = jj % np, cq = jj / np;
+      if (cp == 0 || cp == np - 1) m *= 0.5;
+      if (cq == 0 || cq == g.nq[s] - 1) m *= 0.5;
     }
-    if (cot) cot[e] = cv;
+    w[q] = g.wt * m;
+    wh[q] = (float)w[q];
+    wl[q] = (float)(w[q] - (double)wh[q]);
+    sq[q] = 0.0;
   }
+  const int k0 = (int)blockIdx.y * rows, k1 = min(k0 + rows, g.nsteps + 1);
+  long long e = ((long long)s * (g.nsteps + 1) + k0) * g.stride + c0;
+  for (int k = k0; k < k1; ++k, e += g.stride) {
+    T tv[kMisfitCols], ov[kMisfitCols];
+#pragma unroll
+    for (int q = 0; q < kMisfitCols; ++q) {
+      const int jj = c0 + q * kReduceThreads;
+      const bool on = k >= 1 && jj < n;
+      tv[q] = on ? trace[e + q * kReduceThreads] : T(0);
+      ov[q] = on ? obs[e + q * kReduceThreads] : T(0);
+    }
+#pragma unroll
+    for (int q = 0; q < kMisfitCols; ++q) {
+      const double d = widen(tv[q]) - widen(ov[q]);
+      sq[q] += d * d;
+      if (cot && c0 + q * kReduceThreads < g.stride)
+        cot[e + q * kReduceThreads] = product(tv[q], ov[q], wh[q], wl[q], w[q], d);
+    }
+  }
+  double acc = 0.0;
+#pragma unroll
+  for (int q = 0; q < kMisfitCols; ++q) acc += w[q] == 0.0 ? 0.0 : 0.5 * w[q] * sq[q];
   acc = block_sum(acc);
-  if (threadIdx.x == 0) partials[blockIdx.x] = acc;
+  if (threadIdx.x == 0) partials[((size_t)s * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x] = acc;
 }
 
 __global__ void sum_kernel(const double* __restrict__ p, int n, double* out) {
@@ -182,15 +238,30 @@ __global__ void __launch_bounds__(kReduceThreads) cg_axpy_clip_kernel(
 
 }  // namespace
 
-template <typename T>
-void launch_misfit(const MisfitGeom& g, const T* trace, const T* obs, T* cot, double* partials,
-                   cudaStream_t st) {
-  misfit_kernel<T><<<kReduceBlocks, kReduceThreads, 0, st>>>(g, trace, obs, cot, partials);
+// Column blocks of one trace row.
+static long long misfit_cols(const MisfitGeom& g) {
+  const int per = kReduceThreads * kMisfitCols;
+  return ((long long)g.stride + per - 1) / per;
 }
-template void launch_misfit<float>(const MisfitGeom&, const float*, const float*, float*, double*,
-                                   cudaStream_t);
-template void launch_misfit<double>(const MisfitGeom&, const double*, const double*, double*, double*,
-                                    cudaStream_t);
+
+long long misfit_parts(const MisfitGeom& g) {
+  const long long least = misfit_cols(g) * g.n_src;
+  return least > kMisfitParts ? least : kMisfitParts;
+}
+
+template <typename T>
+int launch_misfit(const MisfitGeom& g, const T* trace, const T* obs, T* cot, double* partials, cudaStream_t st) {
+  const long long cols = misfit_cols(g);
+  // rows per block: about kMisfitParts / 2 blocks, at most kMisfitParts
+  const long long all = g.nsteps + 1;
+  long long rows = (all * cols * g.n_src + kMisfitParts / 2 - 1) / (kMisfitParts / 2);
+  while (cols * g.n_src * ((all + rows - 1) / rows) > kMisfitParts && rows < all) ++rows;
+  const dim3 grid((unsigned)cols, (unsigned)((all + rows - 1) / rows), (unsigned)g.n_src);
+  misfit_kernel<T><<<grid, kReduceThreads, 0, st>>>(g, (int)rows, trace, obs, cot, partials);
+  return (int)(grid.x * grid.y * grid.z);
+}
+template int launch_misfit<float>(const MisfitGeom&, const float*, const float*, float*, double*, cudaStream_t);
+template int launch_misfit<double>(const MisfitGeom&, const double*, const double*, double*, double*, cudaStream_t);
 
 void launch_sum(const double* partials, int n, double* out, cudaStream_t st) {
   sum_kernel<<<1, 256, 0, st>>>(partials, n, out);
