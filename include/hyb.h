@@ -87,7 +87,8 @@ typedef struct {
                           voxels need every corner at least 2 nodes from the
                           outer faces. */
   int64_t wait_cycles; /* limit, in SM clock cycles, of each bounded wait of
-                          the step kernels for their staged planes (0: the
+                          the step kernels for their staged planes and for
+                          the earlier levels' work they build on (0: the
                           default, 2^29 cycles, about 0.25 s).  A wait that
                           runs out makes the kernel stop and hyb_sync return
                           HYB_ERR_TIMEOUT; the field is then undefined.
@@ -142,11 +143,9 @@ typedef struct {
                           ghost 2 dx g uses that step too, the quadrature
                           weight of a face node is its in-face cell area
                           dx_p dx_q (halved on the face's border), and
-                          dt_max = 1 / sqrt(a_max sum 1 / dx^2).  Every level
-                          then takes two launches (the rows off the faces,
-                          then the face layers by the generic rows; no staged
-                          tiles).  Needs no refinement, the exact adjoint and
-                          the wave model, and no batches (HYB_ERR_ARG). */
+                          dt_max = 1 / sqrt(a_max sum 1 / dx^2).  Needs no
+                          refinement, the exact adjoint and the wave model,
+                          and no batches (HYB_ERR_ARG). */
 } hyb_mesh_desc;
 
 #define HYB_WAIT_NONE (-1)

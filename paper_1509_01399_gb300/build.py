@@ -17,7 +17,7 @@ CSRC = os.path.join(PKG, "csrc")
 BUILD = os.path.join(PKG, "_build")
 LIB = os.path.join(PKG, "libhyb.so")
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
-SOURCES = ["step_kernels.cu", "reduce_kernels.cu", "api.cpp"]
+SOURCES = ["sweep_kernels.cu", "step_kernels.cu", "reduce_kernels.cu", "api.cpp"]
 
 
 def nvcc_path() -> str:

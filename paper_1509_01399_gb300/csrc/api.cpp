@@ -47,7 +47,7 @@ struct SweepKey {
   double dt = 0.0;
   int face[16] = {0};
   double omega[16] = {0.0}, amp[16] = {0.0}, dir[16][3] = {};
-  const void* bufs[10] = {nullptr};
+  const void* bufs[11] = {nullptr};
 };
 
 bool same_key(const SweepKey& a, const SweepKey& b) {
@@ -58,7 +58,7 @@ bool same_key(const SweepKey& a, const SweepKey& b) {
     if (a.face[i] != b.face[i] || a.omega[i] != b.omega[i] || a.amp[i] != b.amp[i] || a.dir[i][0] != b.dir[i][0] ||
         a.dir[i][1] != b.dir[i][1] || a.dir[i][2] != b.dir[i][2])
       return false;
-  for (int i = 0; i < 10; ++i)
+  for (int i = 0; i < 11; ++i)
     if (a.bufs[i] != b.bufs[i]) return false;
   return true;
 }
@@ -70,6 +70,13 @@ struct SweepGraph {
   bool seen = false;
   cudaGraphExec_t exec = nullptr;
   long long launches = 0;
+};
+
+// Work items of one level (sweep kernel) for a slot count.
+struct SweepPlan {
+  DevBuf items, need, rslab, sync;
+  int nitems = 0, nslab = 0, slabz = 0, block = 0, grid = 0;
+  int ns = 0, smem = 0, split = 0, ccen = 0, yo = 0, ncur = 0, nstage = 0;  // ring (StepArgs)
 };
 
 }  // namespace
@@ -114,12 +121,17 @@ struct hyb_mesh {
   bool ani = false;          // the lattice steps differ per axis (every level by the bulk and shell kernels)
   double hv[3] = {0, 0, 0};  // lattice step per axis
   cudaStream_t cap = nullptr;  // private stream used only to capture sweep graphs
-  // interior work items of the forward / transposed step per slot count; built
-  // once and kept (captured sweep graphs refer to them)
+  // work items of a level per slot count; built once and kept (captured sweep
+  // graphs refer to them)
+  SweepPlan plans[kMaxSlots + 1];
+  int nsm = 0;                  // SMs of the device
+  DevBuf table;                 // the sweep launch's slots at every level
+  // tile kernel: interior work items of the forward / transposed step per slot
+  // count; built once and kept
   DevBuf items[2][kMaxSlots + 1];
   int nitems[2][kMaxSlots + 1] = {};
-  int nsm = 0;                 // SMs of the device
-  int bps = 0;                 // resident step-kernel blocks per SM
+  int bps = 0;                  // its resident blocks per SM
+  std::vector<int> rcorner, rcentre;  // refined corner rows / centres below each plane (prefix counts)
   SweepGraph graphs[3];
 };
 
@@ -190,9 +202,9 @@ SweepKey make_key(const hyb_mesh* m, int kind, const void* io, int accumulate, i
     k.amp[i] = src[i].amp;
     for (int a = 0; a < 3; ++a) k.dir[i][a] = src[i].dir[a];
   }
-  const void* b[10] = {m->U.p, m->L.p, m->hist.p, m->ckpt.p, m->G.p, m->W.p, m->CU.p, m->CL.p,
-                       m->have_init ? m->I0.p : nullptr, m->have_init ? m->IC0.p : nullptr};
-  for (int i = 0; i < 10; ++i) k.bufs[i] = b[i];
+  const void* b[11] = {m->U.p, m->L.p, m->hist.p, m->ckpt.p, m->G.p, m->W.p, m->CU.p, m->CL.p,
+                       m->have_init ? m->I0.p : nullptr, m->have_init ? m->IC0.p : nullptr, m->table.p};
+  for (int i = 0; i < 11; ++i) k.bufs[i] = b[i];
   return k;
 }
 
@@ -303,6 +315,16 @@ int mask_at(const hyb_mesh* m, const hyb_source& s, int k, double dt) {
   return mask;
 }
 
+// The entry faces and their switch times (the sweep kernel's phase()).
+template <typename T>
+void set_entry(Slot<T>& S, const Wave& w) {
+  S.entry = 0;
+  for (int f = 0; f < 6; ++f) {
+    S.tsw[f] = w.tsw[f];
+    if (w.fac[f] > 0.0) S.entry |= 1 << f;
+  }
+}
+
 // The slot's plane-wave constants for the step leaving t_k.
 template <typename T>
 void set_wave(const hyb_mesh* m, Slot<T>& S, const hyb_source& src, int k, double dt) {
@@ -313,6 +335,7 @@ void set_wave(const hyb_mesh* m, Slot<T>& S, const hyb_source& src, int k, doubl
   S.src_mask = sm;
   S.st = k * dt;
   const double h = m->d.h;
+  set_entry(S, w);
   for (int f = 0; f < 6; ++f) S.sf[f] = dt * dt * 2.0 / (m->ani ? m->hv[f >> 1] : h) * src.amp * w.fac[f];
   for (int a = 0; a < 3; ++a) {
     S.sd[a] = m->ani ? w.d[a] * m->hv[a] : w.d[a];  // per-axis steps: the delay d . (x - x0) axis by axis
@@ -323,13 +346,11 @@ void set_wave(const hyb_mesh* m, Slot<T>& S, const hyb_source& src, int k, doubl
   S.st1 = 2.0 * M_PI / src.omega;
 }
 
-// Launch geometry of one step: the interior covers nodes 1 .. n-2 on every
+// Launch geometry of one step of the tile kernel: the interior covers nodes 1 .. n-2 on every
 // axis in 32 x 16 tiles (in x from tile_x0: FP32 tiles start at x = 0); the edge tiles cover the nodes within one node of
-// two faces.  Lattices with fewer than 5 nodes on an axis use a single
-// generic kernel instead.
-void step_geometry(const hyb_mesh* m, int* npb, int* ntx, int* small, int* nedge) {
-  *small = (m->n[0] < 5 || m->n[1] < 5 || m->n[2] < 5) ? 1 : 0;
-  *nedge = *small ? 0 : 1 + (m->n[0] - 4 + 7) / 8 + (m->n[1] - 4 + 7) / 8 + (m->n[2] - 4 + 7) / 8;
+// two faces.
+void step_geometry(const hyb_mesh* m, int* npb, int* ntx, int* nedge) {
+  *nedge = 1 + (m->n[0] - 4 + 7) / 8 + (m->n[1] - 4 + 7) / 8 + (m->n[2] - 4 + 7) / 8;
   *ntx = (m->n[0] - 1 - tile_x0(m->d.precision) + kTileX - 1) / kTileX;
   const int nty = (m->n[1] - 2 + kTileY - 1) / kTileY;
   *npb = *ntx * nty;
@@ -411,14 +432,24 @@ std::vector<int> build_items(const hyb_mesh* m, int nslots, bool adjoint) {
   return out;
 }
 
-// One time level on `st`: one launch (two with per-axis steps).
-template <class Launch>
-hyb_status step_launch(hyb_mesh* m, cudaStream_t st, Launch launch) {
-  const int n = launch(st);  // kernels the level took (two with per-axis steps)
-  m->launches += n - 1;
-  HYB_LAUNCHED(m);
-  return HYB_OK;
+// x groups of 16 bytes that hold the nodes 1 .. nx - 2.
+int quads_of_row(const hyb_mesh* m) {
+  return (m->n[0] - 2) / (m->d.precision == HYB_FP32 ? 4 : 2) + 1;
 }
+
+// Bytes behind a field ring that the last item's plane copy may reach into.
+constexpr size_t kFieldPad = 64;
+
+// Planes of a slab at most (the planes at the ends of a march are read twice),
+// and the items a resident block should get per level: enough that blocks of
+// uneven speed even out, FP64 rows with the pairing being several times the
+// others (131 x 118 x 143 FP64, two sources, forward / transposed level:
+// 0.175 / 0.341 ms with one item a block, 0.144 / 0.262 with three, 0.132 /
+// 0.197 with six, 0.133 / 0.189 with ten).
+// Entries a thread of a face or refined item takes at most.
+constexpr int kGatherRounds = 4;
+constexpr int kMaxMarch = 16;
+constexpr double kItemsPerBlock = 8.0;
 
 // P1 element of a tetrahedron (vertex coordinates X[4][3]): volume and
 // stiffness K_ij = |K| grad phi_i . grad phi_j (Sec. 7.2), a = 1.
@@ -686,6 +717,15 @@ hyb_status build_refined(hyb_mesh* m, const uint8_t* mask) {
         rzr[2 * c + 1] = std::max(rzr[2 * c + 1], m->fl[2] + k);
       }
   HYB_TRY(upload(m, m->rzr, rzr));
+  // rows and centres below each plane (both lists run in plane order)
+  m->rcorner.assign(m->n[2] + 1, 0);
+  m->rcentre.assign(m->n[2] + 1, 0);
+  for (long long p : rows) ++m->rcorner[(size_t)(p / ((long long)m->px * m->n[1])) + 1];
+  for (int u : refid) ++m->rcentre[(size_t)(m->fl[2] + u / (m->un[0] * m->un[1])) + 1];
+  for (int k = 0; k < m->n[2]; ++k) {
+    m->rcorner[k + 1] += m->rcorner[k];
+    m->rcentre[k + 1] += m->rcentre[k];
+  }
   HYB_TRY(upload(m, m->refvox, refv));
   HYB_TRY(upload(m, m->refvox_id, refid));
   // the refined voxels' origins packed for the kernel: (x | y << 16, z) in unknown-voxel coordinates
@@ -766,7 +806,6 @@ hyb_status step_maps(const hyb_mesh* m, StepArgs<T>& A, const DevBuf& field, int
 // first time this slot count is used, outside any captured sweep).
 template <typename T>
 hyb_status step_items(hyb_mesh* m, StepArgs<T>& A, int nslots, bool adjoint) {
-  if (A.small) return HYB_OK;
   const int d = adjoint ? 1 : 0;
   DevBuf& buf = m->items[d][nslots];
   if (!buf.p) {
@@ -776,6 +815,89 @@ hyb_status step_items(hyb_mesh* m, StepArgs<T>& A, int nslots, bool adjoint) {
   }
   A.items = (const int*)buf.p;
   A.nitems = m->nitems[d][nslots];
+  return HYB_OK;
+}
+
+// Levels of one sweep launch at most: about this many node-steps, so that
+// sweeps on other streams get their turn.
+constexpr double kLaunchNodeSteps = 5e9;
+
+int launch_levels(const hyb_mesh* m, int nsrc) {
+  return (int)std::min(1e6, std::max(1.0, kLaunchNodeSteps / ((double)m->Np * nsrc)));
+}
+
+// The plan for `nslots` slots (built and uploaded the first time this slot
+// count is used, outside any captured sweep): the ring of plane stages, the
+// slab depth (a march through the planes of a slab) and the items.
+hyb_status build_plan(hyb_mesh* m, int nslots) {
+  SweepPlan& P = m->plans[nslots];
+  if (P.nitems) return HYB_OK;
+  const int nx = m->n[0], ny = m->n[1], nz = m->n[2], px = m->px;
+  const int V = m->d.precision == HYB_FP32 ? 4 : 2;
+  const int nqx = quads_of_row(m);
+  const long long nq = (long long)(ny - 2) * nqx;
+  const double work = (double)nslots * nq * (nz - 2);  // quads of a level
+  const int block = work < (double)m->nsm * kMaxBlock ? 128 : kMaxBlock;
+  // ring: the longest run of memory that holds an item's quads, with the rows
+  // above and below as one run, or (rows longer than the run) apart
+  long long span = 0;
+  for (long long f = 0; f < nq; f += block) {
+    const long long l = std::min(f + block, nq) - 1;
+    span = std::max(span, (long long)px * (l / nqx - f / nqx) + V * (l % nqx - f % nqx + 1));
+  }
+  P.split = px > span ? 1 : 0;
+  P.yo = P.split ? (int)span + 2 * V : px;
+  P.ccen = P.split ? P.yo + V : px;
+  P.ncur = P.split ? 3 * P.yo : (int)span + 2 * px + V;
+  P.nstage = (P.ncur + (int)span + 31) & ~31;
+  const int stage = P.nstage * (int)esize(m);
+  int bps = block == 128 ? kSweepBlocksPerSm + 1 : kSweepBlocksPerSm;
+  while (bps > 1 && kMaxRing / bps / stage < 4) --bps;
+  P.ns = std::min(kMaxStages, kMaxRing / bps / stage);
+  P.smem = P.ns * stage;
+  const int resident = m->nsm * sweep_blocks_per_sm(m->d.precision, block, P.smem);
+  const int B = (int)std::min((double)kMaxMarch, std::max(1.0, std::floor(work / block / (kItemsPerBlock * resident))));
+  const int nslab = (nz - 2 + B - 1) / B;
+  std::vector<int> items, need(nslab, 0), rslab(4 * (size_t)nslab, 0);
+  auto add = [&](int kind, int slab, long long first, long long end, int w) {
+    items.insert(items.end(), {kind | slab << 8, (int)first, (int)end, w});
+    ++need[slab];
+  };
+  const int mx = nx - 4, my = ny - 4, per = block / 128;
+  // entries of a face or refined item: up to kGatherRounds per thread
+  const double gathered = nslots * (2.0 * mx * my + 2.0 * (mx + my) * (nz - 4) + m->nrl + m->nc);
+  const int gather = block * (int)std::min((double)kGatherRounds, std::max(1.0, std::floor(gathered / block / resident)));
+  for (int s = 0; s < nslab; ++s) {
+    const int c0 = 1 + s * B, c1 = std::min(c0 + B, nz - 1);          // planes
+    const int k0 = std::max(c0, 2), k1 = std::min(c1, nz - 2);        // planes off the z faces
+    const int mz = std::max(0, k1 - k0);
+    const int xy = 1 + (ny - 4 + 15) / 16 + (nx - 4 + 15) / 16;       // tiles of one z end
+    for (int end = 0; end < 2; ++end)
+      if (s == (end ? nslab - 1 : 0))
+        for (int e = 0; e < xy; e += per) add(3, s, e, std::min(e + per, xy), end);
+    const int ez = (mz + 7) / 8;
+    for (int e = 0; e < ez; e += per) add(2, s, e, std::min(e + per, ez), 0);
+    const long long nf = ((s == 0 ? 1LL : 0) + (s == nslab - 1 ? 1LL : 0)) * mx * my + 2LL * (mx + my) * mz;
+    for (long long f = 0; f < nf; f += gather) add(1, s, f, std::min(f + gather, nf), 0);
+    if (m->nc > 0) {
+      int* r = &rslab[4 * (size_t)s];
+      r[0] = m->rcorner[c0];
+      r[1] = m->rcorner[c1] - m->rcorner[c0];
+      r[2] = m->rcentre[c0];
+      r[3] = m->rcentre[c1] - m->rcentre[c0];
+      for (int f = 0; f < r[1] + r[3]; f += gather) add(4, s, f, std::min(f + gather, r[1] + r[3]), 0);
+    }
+    for (long long f = 0; f < nq; f += block) add(0, s, f, nq, 0);
+  }
+  HYB_TRY(upload(m, P.items, items));
+  HYB_TRY(upload(m, P.need, need));
+  HYB_TRY(upload(m, P.rslab, rslab));
+  HYB_TRY(upload(m, P.sync, std::vector<unsigned>(2 + (size_t)nslots * nslab, 0u)));
+  P.nslab = nslab;
+  P.slabz = B;
+  P.block = block;
+  P.nitems = (int)(items.size() / 4);
+  P.grid = (int)std::min((double)resident, 2.0 * P.nitems * nslots);
   return HYB_OK;
 }
 
@@ -808,11 +930,14 @@ void base_args(const hyb_mesh* m, StepArgs<T>& A, double dt, int nslots) {
   const double h = m->ani ? m->hv[0] : m->d.h;
   A.c2 = (T)(dt * dt / (h * h));
   A.r = (T)((h - dt) / (h + dt));
-  step_geometry(m, &A.npb, &A.ntx, &A.small, &A.nedge);
-  if (m->ani) {  // every level by the bulk and shell kernels, axis terms weighed by kap
-    A.ani = 1;
+  // the generic kernel: lattices without an interior, and beyond the sweep
+  // kernel's 32-bit item indices
+  A.small = (m->n[0] < 5 || m->n[1] < 5 || m->n[2] < 5) ? 1 : 0;
+  if ((m->d.precision == HYB_FP64 || m->ani) && m->nc == 0 &&
+      ((long long)m->n[0] * m->n[1] + (m->n[0] + (long long)m->n[1]) * kMaxMarch >= 1LL << 30 || m->n[2] >= 1 << 23))
     A.small = 1;
-    A.nedge = 0;
+  if (m->ani) {  // axis terms weighed by kap
+    A.ani = 1;
     for (int a = 0; a < 3; ++a) {
       A.kap[a] = (h * h) / (m->hv[a] * m->hv[a]);
       A.kapt[a] = (T)A.kap[a];
@@ -823,12 +948,16 @@ void base_args(const hyb_mesh* m, StepArgs<T>& A, double dt, int nslots) {
   if (m->d.fem_path == HYB_FEM_TET_ALL) {  // every level by the all-node kernels
     A.tet = 1;
     A.small = 1;
-    A.nedge = 0;
     A.acoef = (const double*)m->acopy.p;
     A.kuhn = (const double*)m->kuhn.p;
     A.kuhn_v = (const int*)m->kuhn_v.p;
   }
   A.nslots = nslots;
+  A.abc_mask = m->abc_mask;
+  A.dt = dt;
+  A.Np = m->Np;
+  A.nqx = quads_of_row(m);
+  step_geometry(m, &A.npb, &A.ntx, &A.nedge);
   if (m->nc > 0) {
     A.nref = m->nc;
     A.nrl = m->nrl;
@@ -850,8 +979,31 @@ void base_args(const hyb_mesh* m, StepArgs<T>& A, double dt, int nslots) {
   }
 }
 
-// The coefficient of slot s: its edge weights (and their plane in the
-// weight tensor map) and its refined voxels' a; per slot for a batch.
+// The plan's part of the launch arguments.
+template <typename T>
+hyb_status plan_args(hyb_mesh* m, StepArgs<T>& A, int nslots, int nsteps) {
+  HYB_TRY(build_plan(m, nslots));
+  HYB_TRY(ensure(m, m->table, (size_t)std::min(nsteps, launch_levels(m, nslots)) * nslots * sizeof(Slot<T>)));
+  A.table = (Slot<T>*)m->table.p;
+  const SweepPlan& P = m->plans[nslots];
+  A.nslab = P.nslab;
+  A.slabz = P.slabz;
+  A.ns = P.ns;
+  A.split = P.split;
+  A.ccen = P.ccen;
+  A.yo = P.yo;
+  A.ncur = P.ncur;
+  A.nstage = P.nstage;
+  A.sitems = (const int4*)P.items.p;
+  A.snitems = P.nitems;
+  A.need = (const int*)P.need.p;
+  A.rslab = (const int4*)P.rslab.p;
+  A.sync = (unsigned*)P.sync.p;
+  return HYB_OK;
+}
+
+// The coefficient of slot s: its edge weights and its refined voxels' a; per
+// slot for a batch.
 template <typename T>
 void slot_coef(const hyb_mesh* m, Slot<T>& S, int s) {
   const int q = m->batch ? s : 0;
@@ -902,6 +1054,87 @@ void forward_slots(const hyb_mesh* m, StepArgs<T>& A, const hyb_source* src, int
   }
 }
 
+template <typename T>
+hyb_status launch_piece(hyb_mesh* m, const StepArgs<T>& A, StepMode mode, cudaStream_t st) {
+  const SweepPlan& P = m->plans[A.nslots];
+  m->launches += launch_sweep<T>(A, mode, P.block, P.grid, P.smem, st) - 1;
+  HYB_LAUNCHED(m);
+  return HYB_OK;
+}
+
+// How the levels of a mesh run: the generic all-node kernel (lattices with
+// fewer than 5 nodes on an axis, the all-FEM path), the tile kernel (FP32
+// fields with equal steps), or the sweep kernel.  FP32 with equal steps stays
+// with the tiles, whose edge weights and history are staged: 257^3, eight
+// sources, refined, 0.49 / 0.54 ms a level against 0.66 / 0.92 ms by the sweep
+// kernel (without a FEM block 0.40 against 0.32).  FP64 and per-axis steps gain
+// 1.3 - 2.5 times from the sweep kernel at every size measured (its comment).
+enum class Path { kAllNodes, kTiles, kSweep };
+
+template <typename T>
+Path path_of(const StepArgs<T>& A) {
+  if (A.small) return Path::kAllNodes;
+  return sizeof(T) == 4 && !A.ani ? Path::kTiles : Path::kSweep;
+}
+
+// What the launches of a sweep with the fields `field` need besides its slots.
+template <typename T>
+hyb_status path_args(hyb_mesh* m, StepArgs<T>& A, int nslots, int nsteps, const DevBuf& field, int hist_levels,
+                     bool adjoint) {
+  switch (path_of(A)) {
+    case Path::kAllNodes: return HYB_OK;
+    case Path::kSweep: return plan_args<T>(m, A, nslots, nsteps);
+    case Path::kTiles:
+      HYB_TRY(step_maps<T>(m, A, field, nslots, hist_levels));
+      return step_items<T>(m, A, nslots, adjoint);
+  }
+  return HYB_OK;
+}
+
+// One level of every slot (not the sweep kernel).
+template <typename T>
+hyb_status launch_level(hyb_mesh* m, const StepArgs<T>& A, bool adjoint, cudaStream_t st) {
+  if (A.small) {
+    launch_all_nodes<T>(A, adjoint, st);
+  } else if constexpr (sizeof(T) == 4) {
+    launch_tile_step(A, adjoint, st);
+  }
+  HYB_LAUNCHED(m);
+  return HYB_OK;
+}
+
+// Forward steps k .. k + n - 1.  hl / chl: history slot of step k; the first
+// nh steps write one each.
+template <typename T>
+hyb_status forward_levels(hyb_mesh* m, StepArgs<T>& A, const hyb_source* src, int nsrc, int nsteps, double dt, int k,
+                          int n, T* trace, T* hl, T* chl, int nh, cudaStream_t st) {
+  const long long lvl = (long long)nsrc * m->hbox, clvl = (long long)nsrc * m->nc;
+  const bool sweep = path_of(A) == Path::kSweep;
+  const int most = sweep ? launch_levels(m, nsrc) : 1;
+  for (int l = 0; l < n; l += most) {
+    const int q = std::min(most, n - l);
+    const bool h = hl && l < nh;
+    forward_slots<T>(m, A, src, nsrc, nsteps, dt, k + l, trace, h ? hl + l * lvl : nullptr, h ? chl + l * clvl : nullptr);
+    if (!sweep) {
+      HYB_TRY(launch_level<T>(m, A, false, st));
+      continue;
+    }
+    A.nlev = q;
+    A.k0 = k + l;
+    A.dir = 1;
+    A.ring0 = (k + l) % 3;
+    A.fbase = (T*)m->U.p;
+    A.cbase = (T*)m->CU.p;
+    A.obs_step = m->obs_stride;
+    A.hist_step = lvl;
+    A.chist_step = clvl;
+    A.hist_l0 = 0;
+    A.hist_l1 = h ? nh - l : 0;
+    HYB_TRY(launch_piece<T>(m, A, kForward, st));
+  }
+  return HYB_OK;
+}
+
 // Levels 0 and -1 of one source (lattice field and centre values): the
 // initial state of Model Problem 1 if one was set, else zero.
 template <typename T>
@@ -932,7 +1165,7 @@ hyb_status forward_impl(hyb_mesh* m, const double* a, const hyb_source* src, int
   const int C = m->d.ckpt_every;
   const bool ckpt = C > 0;
   const size_t cb = (size_t)m->nc * sizeof(T);  // centre values of one level
-  HYB_TRY(ensure(m, m->U, 3 * (size_t)nsrc * fb));
+  HYB_TRY(ensure(m, m->U, 3 * (size_t)nsrc * fb + kFieldPad));
   HYB_TRY(ensure(m, m->CU, 3 * (size_t)nsrc * cb));
   if (m->d.fem_path == HYB_FEM_TET_ALL) HYB_TRY(ensure(m, m->acopy, (size_t)std::max(m->nu, 1LL) * sizeof(double)));
   if (keep && m->nown > 0) {
@@ -953,8 +1186,7 @@ hyb_status forward_impl(hyb_mesh* m, const double* a, const hyb_source* src, int
   m->batch = batch;
   StepArgs<T> A;
   base_args(m, A, dt, nsrc);
-  HYB_TRY(step_maps<T>(m, A, m->U, nsrc, 0));
-  HYB_TRY(step_items<T>(m, A, nsrc, false));
+  HYB_TRY(path_args<T>(m, A, nsrc, nsteps, m->U, 0, false));
   const bool tel = m->d.model == HYB_MODEL_TELEGRAPH;
   if (tel) {  // the edge weights of a = 1, the damping ratios from sigma
     if (!m->ones.p) HYB_TRY(upload(m, m->ones, std::vector<double>((size_t)std::max(m->nu, 1LL), 1.0)));
@@ -1001,10 +1233,17 @@ hyb_status forward_impl(hyb_mesh* m, const double* a, const hyb_source* src, int
         if (m->nc) HYB_CU(cudaMemsetAsync(chist, 0, (size_t)nsrc * cb, st));
       }
     }
-    const size_t lvl = (size_t)nsrc * m->hbox;
-    const size_t clvl = (size_t)nsrc * m->nc;
-    for (int k = 0; k < nsteps; ++k) {
-      if (keep && ckpt && m->nown > 0 && k > 0 && k % C == 0) {
+    // history slot of step k: u^{k+1} in slot k + 1 (the wave model; slot 0
+    // holds u^0), or, in the telegraph model, u^{k+1} - u^{k-1} in slot k;
+    // slots 0 .. nsteps - 1
+    const bool full = keep && !ckpt && m->nown > 0;
+    const int sh = tel ? 0 : 1;
+    if (!(keep && ckpt && m->nown > 0))
+      return forward_levels<T>(m, A, src, nsrc, nsteps, dt, 0, nsteps, trace,
+                               full ? hist + (size_t)sh * nsrc * m->hbox : nullptr,
+                               full ? chist + (size_t)sh * nsrc * m->nc : nullptr, full ? nsteps - sh : 0, st);
+    for (int k = 0; k < nsteps; k += C) {
+      if (k > 0) {
         const size_t seg = (size_t)(k / C);
         for (int s = 0; s < nsrc; ++s) {
           char* base = (char*)m->ckpt.p + ((seg * nsrc + s) * 2) * fb;
@@ -1019,14 +1258,7 @@ hyb_status forward_impl(hyb_mesh* m, const double* a, const hyb_source* src, int
           }
         }
       }
-      // history slot of step k: u^{k+1} in slot k + 1 (the wave model; slot 0
-      // holds u^0), or, in the telegraph model, u^{k+1} - u^{k-1} in slot k
-      const int slot = tel ? k : k + 1;
-      const bool hk = keep && !ckpt && m->nown > 0 && slot <= nsteps - 1;
-      T* hl = hk ? hist + (size_t)slot * lvl : nullptr;
-      T* chl = hk ? chist + (size_t)slot * clvl : nullptr;
-      forward_slots<T>(m, A, src, nsrc, nsteps, dt, k, trace, hl, chl);
-      HYB_TRY(step_launch(m, st, [&](cudaStream_t q) { return launch_forward_step<T>(A, q); }));
+      HYB_TRY(forward_levels<T>(m, A, src, nsrc, nsteps, dt, k, std::min(C, nsteps - k), trace, nullptr, nullptr, 0, st));
     }
     return HYB_OK;
   };
@@ -1065,6 +1297,7 @@ void adjoint_slots(const hyb_mesh* m, StepArgs<T>& A, const T* cot, int j, const
     S.zf_cur = (int)((S.cur - (const T*)m->L.p) / ((long long)m->px * m->n[1]));
     S.zf_prev = (int)((S.prev - (const T*)m->L.p) / ((long long)m->px * m->n[1]));
     S.zf_hist = S.hist_r ? (int)((S.hist_r - (const T*)m->hist.p) / ((long long)m->hpx * m->fn[1])) : 0;
+    set_entry(S, wave_of(m, m->src[s]));
     S.mask_f = mask_at(m, m->src[s], j, m->dt);
     S.mask_e = mask_at(m, m->src[s], j - 1, m->dt);
     S.mask_c = mask_at(m, m->src[s], j + 1, m->dt);
@@ -1145,23 +1378,21 @@ hyb_status adjoint_impl(hyb_mesh* m, const T* cot, int accumulate) {
   const bool ckpt = C > 0;
   const bool tel = m->d.model == HYB_MODEL_TELEGRAPH;
   const size_t cb = (size_t)m->nc * sizeof(T);
-  HYB_TRY(ensure(m, m->L, 3 * (size_t)nsrc * fb));
+  HYB_TRY(ensure(m, m->L, 3 * (size_t)nsrc * fb + kFieldPad));
   HYB_TRY(ensure(m, m->CL, 3 * (size_t)nsrc * cb));
   HYB_TRY(ensure(m, m->G, (size_t)nsrc * m->nu * sizeof(double)));
   StepArgs<T> A;   // adjoint steps
   base_args(m, A, dt, nsrc);
   StepArgs<T> F;   // recomputed forward steps
   base_args(m, F, dt, nsrc);
-  HYB_TRY(step_maps<T>(m, A, m->L, nsrc, ckpt ? C : nsteps));
-  HYB_TRY(step_maps<T>(m, F, m->U, nsrc, 0));
-  HYB_TRY(step_items<T>(m, A, nsrc, true));
-  HYB_TRY(step_items<T>(m, F, nsrc, false));
+  HYB_TRY(path_args<T>(m, A, nsrc, nsteps, m->L, ckpt ? C : nsteps, true));
+  HYB_TRY(path_args<T>(m, F, nsrc, nsteps, m->U, 0, false));
   const bool paper = m->d.adjoint_mode == HYB_ADJ_PAPER;
-  StepArgs<T> Pp;  // paper-mode steps: forward rows on lambda
+  StepArgs<T> Pp;  // paper-mode steps: forward rows on lambda, every face reflecting
   if (paper) {
     base_args(m, Pp, dt, nsrc);
-    HYB_TRY(step_maps<T>(m, Pp, m->L, nsrc, 0));
-    HYB_TRY(step_items<T>(m, Pp, nsrc, false));
+    HYB_TRY(path_args<T>(m, Pp, nsrc, nsteps, m->L, 0, false));
+    Pp.abc_mask = 0;
   }
   auto body = [&](cudaStream_t st) -> hyb_status {
     if (!accumulate) HYB_CU(cudaMemsetAsync(m->G.p, 0, (size_t)nsrc * m->nu * sizeof(double), st));
@@ -1179,33 +1410,51 @@ hyb_status adjoint_impl(hyb_mesh* m, const T* cot, int accumulate) {
     const size_t lvl = (size_t)nsrc * m->hbox;
     const size_t clvl = (size_t)nsrc * m->nc;
     const bool pairing = m->nu > 0 && m->nown > 0;
-    auto adj_step = [&](int j, const T* hl, const T* chl) -> hyb_status {
-      if (paper) {  // pair (u^j, lambda^j), then lambda^{j-1}
-        paper_slots<T>(m, Pp, cot, j, hl, chl);
-        if (hl) HYB_TRY(paper_pair<T>(m, Pp, st));
-        return step_launch(m, st, [&](cudaStream_t q) { return launch_forward_step<T>(Pp, q); });
+    // adjoint steps j, j - 1, .., j - n + 1; hl / chl: history level of step j;
+    // the steps from the l0-th on pair with theirs
+    auto adj_steps = [&](int j, int n, const T* hl, const T* chl, int l0) -> hyb_status {
+      StepArgs<T>& B = paper ? Pp : A;
+      const bool sweep = path_of(B) == Path::kSweep;
+      const int most = sweep ? launch_levels(m, nsrc) : 1;
+      for (int l = 0; l < n; l += most) {
+        const int q = std::min(most, n - l);
+        const bool h = hl && l + q > l0;
+        const T* hq = h ? hl - (long long)l * lvl : nullptr;
+        const T* cq = h ? chl - (long long)l * clvl : nullptr;
+        if (paper) paper_slots<T>(m, B, cot, j - l, hq, cq);
+        else adjoint_slots<T>(m, B, cot, j - l, hq, cq);
+        if (!sweep) {
+          if (paper && h) HYB_TRY(paper_pair<T>(m, B, st));
+          HYB_TRY(launch_level<T>(m, B, !paper, st));
+          continue;
+        }
+        B.nlev = q;
+        B.k0 = j - l;
+        B.dir = -1;
+        B.ring0 = (paper ? j - l : j - l + 1) % 3;
+        B.fbase = (T*)m->L.p;
+        B.cbase = (T*)m->CL.p;
+        B.obs_step = -(long long)m->obs_stride;
+        B.hist_step = -(long long)lvl;
+        B.chist_step = -(long long)clvl;
+        B.hist_l0 = std::max(0, l0 - l);
+        B.hist_l1 = h ? q : 0;
+        HYB_TRY(launch_piece<T>(m, B, paper ? kPaper : kAdjoint, st));
       }
-      adjoint_slots<T>(m, A, cot, j, hl, chl);
-      return step_launch(m, st, [&](cudaStream_t q) { return launch_adjoint_step<T>(A, q); });
+      return HYB_OK;
     };
     auto first_pair = [&]() -> hyb_status {
       if (!paper) return pair_first<T>(m, A, hist, chist, st);
       paper_slots<T>(m, Pp, nullptr, 0, hist, chist);  // (u^0, lambda^0)
       return paper_pair<T>(m, Pp, st);
     };
-    auto fwd_step = [&](int k, T* hl, T* chl) -> hyb_status {
-      forward_slots<T>(m, F, m->src, nsrc, nsteps, dt, k, nullptr, hl, chl);
-      return step_launch(m, st, [&](cudaStream_t q) { return launch_forward_step<T>(F, q); });
-    };
     if (!ckpt) {
-      for (int j = nsteps; j >= 1; --j) {
-        const bool pj = pairing && j <= nsteps - 1;
-        HYB_TRY(adj_step(j, pj ? hist + (size_t)j * lvl : nullptr, pj ? chist + (size_t)j * clvl : nullptr));
-      }
+      HYB_TRY(adj_steps(nsteps, nsteps, pairing ? hist + (size_t)nsteps * lvl : nullptr,
+                        pairing ? chist + (size_t)nsteps * clvl : nullptr, 1));
       if (pairing) HYB_TRY(first_pair());
       return HYB_OK;
     }
-    HYB_TRY(adj_step(nsteps, nullptr, nullptr));
+    HYB_TRY(adj_steps(nsteps, 1, nullptr, nullptr, 0));
     const int nseg = (nsteps + C - 1) / C;
     for (int seg = nseg - 1; seg >= 0; --seg) {
       const int kb = seg * C;
@@ -1235,12 +1484,13 @@ hyb_status adjoint_impl(hyb_mesh* m, const T* cot, int accumulate) {
         // recompute the segment's history (telegraph: one step further, for
         // u^{ke+1} - u^{ke-1} in the last slot)
         const int sh = tel ? 0 : 1;
-        for (int k = kb; k < ke + 1 - sh; ++k)
-          HYB_TRY(fwd_step(k, hist + (size_t)(k + sh - kb) * lvl, chist + (size_t)(k + sh - kb) * clvl));
+        HYB_TRY(forward_levels<T>(m, F, m->src, nsrc, nsteps, dt, kb, ke + 1 - sh - kb, (T*)nullptr,
+                                  hist + (size_t)sh * lvl, chist + (size_t)sh * clvl, ke + 1 - sh - kb, st));
       }
-      for (int j = ke; j >= std::max(kb, 1); --j)
-        HYB_TRY(adj_step(j, pairing ? hist + (size_t)(j - kb) * lvl : nullptr,
-                         pairing ? chist + (size_t)(j - kb) * clvl : nullptr));
+      const int j0 = std::max(kb, 1);
+      if (ke >= j0)
+        HYB_TRY(adj_steps(ke, ke - j0 + 1, pairing ? hist + (size_t)(ke - kb) * lvl : nullptr,
+                          pairing ? chist + (size_t)(ke - kb) * clvl : nullptr, 0));
     }
     if (pairing) HYB_TRY(first_pair());
     return HYB_OK;
@@ -1584,8 +1834,8 @@ hyb_status hyb_mesh_create(const hyb_mesh_desc* d, void* stream, hyb_mesh** out)
         cudaDeviceGetAttribute(&m->nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
       cudaGetLastError();
       st = fail(HYB_ERR_CUDA, "device query failed");
-    } else {
-      m->bps = std::min(step_blocks_per_sm(d->precision, 0), step_blocks_per_sm(d->precision, 1));
+    } else if (d->precision == HYB_FP32 && !ani) {
+      m->bps = std::min(tile_blocks_per_sm(false), tile_blocks_per_sm(true));
     }
   }
   if (st == HYB_OK && d->fem_path == HYB_FEM_TET_ALL) st = build_kuhn(m);
@@ -1625,9 +1875,12 @@ hyb_status hyb_mesh_destroy(hyb_mesh* m) {
                     &m->g, &m->atrial, &m->cot, &m->trace, &m->rmask, &m->rzr, &m->refvox, &m->refvox_id,
                     &m->k9, &m->rcid, &m->avox, &m->rpos, &m->rvxyz, &m->sdamp, &m->ones,
                     &m->CU, &m->CL, &m->chist, &m->cckpt, &m->I0, &m->IC0, &m->acopy, &m->kuhn, &m->kuhn_v};
+  release(m->table);
   for (DevBuf* b : bufs) release(*b);
   for (auto& dir : m->items)
     for (DevBuf& b : dir) release(b);
+  for (SweepPlan& P : m->plans)
+    for (DevBuf* b : {&P.items, &P.need, &P.rslab, &P.sync}) release(*b);
   if (m->hscal) cudaFreeHost(m->hscal);
   for (SweepGraph& g : m->graphs)
     if (g.exec) cudaGraphExecDestroy(g.exec);

@@ -22,11 +22,13 @@ __device__ __forceinline__ void mbar_init_fence() {
   asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
 }
 
-// orders this thread's earlier shared-memory accesses (and those ordered
-// before them by a block barrier) before later async-proxy accesses
-__device__ __forceinline__ void fence_proxy_async() {
+// orders this thread's earlier accesses (and those ordered before them) before
+// later async-proxy accesses: to the block's shared memory, or to global
+// memory (which costs about a microsecond, so once per item and not per plane)
+__device__ __forceinline__ void fence_proxy_async_shared() {
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
 }
+__device__ __forceinline__ void fence_proxy_async_global() { asm volatile("fence.proxy.async.global;" ::: "memory"); }
 
 __device__ __forceinline__ void mbar_arrive_expect_tx(uint64_t* bar, uint32_t bytes) {
   asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_addr(bar)), "r"(bytes)
@@ -73,6 +75,60 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, long l
     if (done) return true;
     if ((it & 7) == 0 && (clock64() - t0 > budget || *(const volatile int*)abort != 0)) return false;
   }
+}
+
+// ---- the sweep kernel's waits and copies ----
+// Limit of its waits that do not depend on other blocks: a block's own copies
+// and its own warps.
+constexpr long long kOwnCycles = 1LL << 31;
+
+// One try (the hardware may suspend the thread for a short while): has the
+// phase with the given parity of the barrier completed?
+__device__ __forceinline__ bool mbar_try(uint64_t* bar, uint32_t parity) {
+  uint32_t done;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(done)
+      : "r"(smem_addr(bar)), "r"(parity)
+      : "memory");
+  return done != 0;
+}
+
+// A wait for at most `budget` clock cycles, giving up early once *abort is
+// nonzero (a wait timed out; nullptr: not looked at), after a try that failed; a
+// negative budget gives up at once.  Out of line, so that the waits in the row
+// loops stay short.
+static __device__ __noinline__ bool mbar_wait_slow(uint64_t* bar, uint32_t parity, long long budget, const int* abort) {
+  if (budget < 0) return false;
+  const long long t0 = clock64();
+  for (unsigned it = 1;; ++it) {
+    if (mbar_try(bar, parity)) return true;
+    if ((it & 15) == 0 && (clock64() - t0 > budget || (abort && *(const volatile int*)abort != 0))) return false;
+  }
+}
+
+// The same for the service warps, which leave the issue slots to the row warps
+// between tries.
+static __device__ __noinline__ bool mbar_wait_idle(uint64_t* bar, uint32_t parity, long long budget, const int* abort) {
+  if (mbar_try(bar, parity)) return true;
+  if (budget < 0) return false;
+  const long long t0 = clock64();
+  for (unsigned it = 1;; ++it) {
+    __nanosleep(40);
+    if (mbar_try(bar, parity)) return true;
+    if ((it & 15) == 0 && (clock64() - t0 > budget || (abort && *(const volatile int*)abort != 0))) return false;
+  }
+}
+
+// Bulk copy of `bytes` (a multiple of 16) from global to shared memory, both
+// 16-byte aligned, completing on the barrier.
+__device__ __forceinline__ void bulk_load(void* dst, const void* src, uint32_t bytes, uint64_t* bar) {
+  asm volatile(
+      "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(smem_addr(dst)),
+      "l"(src), "r"(bytes), "r"(smem_addr(bar))
+      : "memory");
 }
 
 // Tiled 3-D bulk tensor copy of one box into shared memory, completing

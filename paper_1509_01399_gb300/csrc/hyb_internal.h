@@ -10,7 +10,8 @@
 
 namespace hyb {
 
-constexpr int kMaxSlots = 16;   // problems advanced by one step launch
+constexpr int kMaxSlots = 16;   // problems advanced by one sweep launch
+// ---- tile kernel (step_kernels.cu: FP32 fields, equal steps) ----
 constexpr int kStepBlock = 288;  // threads per block of the step kernel (9 warps)
 constexpr int kTileX = 32;       // interior thread tile (x): one warp per tile row
 constexpr int kTileY = 16;       // interior tile (y): two rows per consumer thread
@@ -39,15 +40,24 @@ struct Box {
 };
 // first node (x) of interior tile 0 for a mesh of the given precision
 inline int tile_x0(int precision) { return precision == HYB_FP32 ? Box<float>::x0 : Box<double>::x0; }
+
+// ---- sweep kernel (sweep_kernels.cu: FP64 fields, per-axis steps) ----
+constexpr int kMaxBlock = 224;   // row threads per block of the sweep kernel, at most (with the producer warp
+                                 // 256: two blocks of 128 registers a thread per SM)
+constexpr int kServiceThreads = 32;  // its producer warp
+constexpr int kSweepBlocksPerSm = 2;  // resident (registers, ring size)
+constexpr int kMaxRing = 208 * 1024;  // bytes of shared memory its rings may take per SM
+constexpr int kMaxStages = 16;   // plane stages of its shared-memory ring, at most
 constexpr int kReduceBlocks = 512;
 // The step kernels accumulate kGradPairScale times the voxel pairing of
 // Eq. (gradient1) (integer edge weights 2 and 1 instead of 1/3 and 1/6).
 constexpr double kGradPairScale = 6.0;
 constexpr int kReduceThreads = 256;
 
-// One problem (one source of one mesh) inside a step launch.
+// One problem (one source of one mesh) at one time level.  A sweep launch gets
+// the slots of its first level and advances them from level to level itself.
 template <typename T>
-struct Slot {
+struct alignas(16) Slot {
   const T* cur;      // forward: u^k        adjoint: lambda^{j+1}
   const T* prev;     // forward: u^{k-1}    adjoint: lambda^{j+2}
   T* next;           // forward: u^{k+1}    adjoint: lambda^j
@@ -68,6 +78,8 @@ struct Slot {
   double sh;         // lattice spacing h
   int si0[3];        // entry corner (node index)
   double somega, st1;
+  double tsw[6];     // last instant each entry face carries the flux
+  int entry;         // entry faces (bits)
   // paper-mode adjoint (forward rows on lambda): the cotangent row entering on
   // the observation face as inj_scale 2^b c_j, b the node's boundary axes
   const T* inj;
@@ -99,8 +111,8 @@ struct StepArgs {
   CUtensorMap tmw;   // edge weights: {wpx, wn1, 3 wn2}, box Box<T>::BX x kHBoxY x 1
   CUtensorMap tmh;   // history: {hpx, fn1, fn2 x boxes}, box Box<T>::BX x kHBoxY x 1
   CUtensorMap tmp;   // field buffer as tmf, box Box<T>::PX x kTileY x 1 (u^{k-1} off the faces)
-  int* err;          // [0]: set when a pipeline wait timed out
-  long long wait;    // cycles a pipeline wait may take (< 0: give up at once if not complete)
+  int* err;          // [0]: set when a bounded wait timed out
+  long long wait;    // cycles such a wait may take (< 0: give up at once if not complete)
   int nx, ny, nz;
   int px;            // row pitch of lattice fields
   int fl[3], fh[3];  // FEM-owned node range (inclusive); fl[0] > fh[0]: no FEM
@@ -114,8 +126,7 @@ struct StepArgs {
   int un[3];         // unknown voxel dims; voxel origins fl .. fl + un - 1
   T c2;              // tau^2 / h^2 (per-axis steps: tau^2 / dx_1^2)
   T r;               // (h - tau) / (h + tau), Eq. (eq:abs2)
-  // per-axis steps dx_1, dx_2, dx_3 that differ (ani = 1; every level then
-  // runs the per-axis kernels): kap[ax] = dx_1^2 / dx_ax^2 weighs the axis-ax
+  // per-axis steps dx_1, dx_2, dx_3 that differ (ani = 1): kap[ax] = dx_1^2 / dx_ax^2 weighs the axis-ax
   // terms of the lattice rows and the edge weights, ra[ax] = (dx_ax - tau) /
   // (dx_ax + tau) is the absorbing coefficient of the faces normal to axis ax
   int ani;
@@ -123,19 +134,46 @@ struct StepArgs {
   T kapt[3];         // kap in the field's precision
   T kdiag;           // -2 (kap[0] + kap[1] + kap[2]) in the field's precision: a lattice row's diagonal
   T ra[3];
+  int small;         // some axis has < 5 nodes, or the all-FEM path: one generic kernel per level
+  // ---- tile kernel ----
   int npb;           // interior: tiles per plane of the interior box
   int ntx;           // interior: tiles along x
   const int* items;  // interior work items, one per block: (slot, tile, z0, z1)
   int nitems;
-  int small;         // some axis has < 5 nodes: one generic kernel per level
   int nedge;         // edge tiles (128 nodes) per slot
-  int nhe, nhr;      // step kernel: leading blocks of edge tiles, trailing blocks of refined rows
+  int nhe, nhr;      // leading blocks of edge tiles, trailing blocks of refined rows
   int nslots;
+  // ---- a sweep launch (sweep_kernel): nlev consecutive levels of every slot ----
+  // The nodes are cut into slabs of slabz planes (slab s: planes 1 + s slabz ..,
+  // the first and last also the z face planes) and each slab's rows into work
+  // items, one block at a time each; `sitems` lists the items of one level of
+  // one slot in slab order (the same for every slot).
+  int nlev;
+  int k0, dir;       // time index of the first step (as in Slot::st), +1 / -1 per level
+  int ring0;         // ring slot (level mod 3) of `cur` at the first level
+  int abc_mask;      // absorbing faces of the mesh
+  double dt;
+  T* fbase;          // field ring [3][slot][Np], centre ring [3][slot][nref]
+  T* cbase;
+  long long Np;
+  long long obs_step, hist_step, chist_step;  // from level to level of obs_w / obs_r / inj and of the history
+  int hist_l0, hist_l1;  // levels (of this launch) that write or read history
+  int nslab, slabz;
+  Slot<T>* table;    // [nlev][nslots]: every slot at every level of the launch
+  int ns;            // stages of the shared-memory ring
+  int split;         // a stage's rows above, at and below the item's are copied apart (wide rows) or as one run
+  int ccen, yo, ncur, nstage;  // elements: first quad in a u^k stage, from row to row, of the u^k part, of a stage
+  int nqx;           // x quads (16 bytes) holding nodes 1 .. nx - 2
+  const int4* sitems;  // (kind | slab << 8, first, end, z end)
+  int snitems;
+  const int* need;   // per slab: items that signal it at each level
+  const int4* rslab; // per slab: first corner row, corner rows, first centre row, centre rows of the refined region
+  unsigned* sync;    // [0] items claimed, [1] blocks finished, [2 + slot * nslab + slab] items completed
   // refined region (nref == 0: nothing refined): unknown voxels bisected
-  // once (12 tetrahedra around a centre node).  Trailing blocks of the step
-  // launch evaluate the rows of their corners (the stencil row corrected by
-  // the refined voxels around the node) and of their centres; the interior
-  // blocks skip those nodes.
+  // once (12 tetrahedra around a centre node).  Blocks (items) of their own
+  // evaluate the rows of their corners (the stencil row corrected by the refined
+  // voxels around the node) and of their centres; the interior items skip
+  // those nodes.
   int nref;                   // refined voxels (= centre nodes)
   int nrl;                    // corners of refined voxels (lattice rows of the refined region)
   const uint2* rpos;          // each such corner (i | j << 16, k)
@@ -171,15 +209,26 @@ struct StepArgs {
   Slot<T> s[kMaxSlots];
 };
 
-// One time level of every slot: one launch of the step kernel (edge tiles,
-// refined rows and interior blocks), or on lattices with fewer than 5 nodes
-// on an axis one generic kernel over every node.
+// Step kinds: the forward rows, the transposed rows with the gradient
+// pairing, and the paper's adjoint (forward rows on lambda with the pairing).
+enum StepMode { kForward = 0, kAdjoint = 1, kPaper = 2 };
+
+// A.nlev consecutive levels of every slot: fills A.table, then one launch of
+// the sweep kernel (blocks of `block` row threads and a producer warp, `smem`
+// bytes of ring each).  Returns the kernels launched.
 template <typename T>
-int launch_forward_step(const StepArgs<T>& a, cudaStream_t st);
+int launch_sweep(const StepArgs<T>& a, StepMode mode, int block, int grid, int smem, cudaStream_t st);
+// One level of every slot by the tile kernel (edge tiles, interior tiles and
+// refined rows in one launch).
+void launch_tile_step(const StepArgs<float>& a, bool adjoint, cudaStream_t st);
+// Resident blocks per SM of the tile kernel, at least 1.
+int tile_blocks_per_sm(bool adjoint);
+// One level by the generic all-node kernel (A.small), from A.s as it stands.
 template <typename T>
-int launch_adjoint_step(const StepArgs<T>& a, cudaStream_t st);
-// Resident blocks per SM of the step kernel (for grid sizing), at least 1.
-int step_blocks_per_sm(int precision, int adjoint);
+void launch_all_nodes(const StepArgs<T>& a, bool adjoint, cudaStream_t st);
+// Resident blocks per SM of the sweep kernel by its registers and `smem` bytes of
+// ring (every variant of the precision gets that ring size), at least 1.
+int sweep_blocks_per_sm(int precision, int block, int smem);
 // G[c] += voxel pairing of (u^0 in hist box, lambda^1) for one slot.
 template <typename T>
 void launch_pair(const StepArgs<T>& a, const T* hist, const T* lam, cudaStream_t st);
@@ -195,9 +244,6 @@ void launch_set_coef(const StepArgs<T>& a, T* W, T* avox, const double* acoef, d
 // others); raises *flag when a sigma is negative or not finite.
 template <typename T>
 void launch_set_damp(const StepArgs<T>& a, T* sdamp, const double* sigma, double dt, int* flag, cudaStream_t st);
-// (The rows of the refined region, identical for the forward and the
-// mass-scaled adjoint, and the adjoint's gradient pairing of refined voxels
-// run in trailing blocks of the step kernel.)
 // Gradient pairing of refined voxels for level 0 (u^0 from the history
 // slots `hist`/`chist`, lambda^1 as the slots' cur/ccur).
 template <typename T>

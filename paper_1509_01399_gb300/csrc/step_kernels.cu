@@ -41,566 +41,14 @@
 // w_e = 2 or 1 (six times the edge weights 1/3 and 1/6); the host scales it
 // by -tau^2 / (6 h^2) (Eq. (gradient1)).
 //
-// Lattices whose steps differ per axis (the 7-point Laplacian of Sec. 7.3
-// with dx_1, dx_2, dx_3) do not use step_kernel: each level is a bulk launch
-// over the nodes off the faces (plain rows with per-axis weights) and a shell
-// launch over the face layers (the generic rows), see ani_fwd_bulk_kernel.
+// FP64 fields and lattices whose steps differ per axis take the sweep kernel
+// (sweep_kernels.cu) instead of step_kernel; lattices with fewer than 5 nodes
+// on an axis and the all-FEM path one generic kernel over every node.
 #include "async_copy.cuh"
-#include "hyb_internal.h"
+#include "rows.cuh"
 
 namespace hyb {
 namespace {
-
-__device__ __forceinline__ int face_bits(int i, int j, int k, int nx, int ny, int nz) {
-  return (i == 0 ? 1 : 0) | (i == nx - 1 ? 2 : 0) | (j == 0 ? 4 : 0) | (j == ny - 1 ? 8 : 0) |
-         (k == 0 ? 16 : 0) | (k == nz - 1 ? 32 : 0);
-}
-
-// Plane-wave flux term tau^2 (2 / h) g of node (i, j, k) on flux face f
-// (the mirror ghost u_g = u_in + 2 h g of d_n u = g, Eq. (f)):
-// g = amp (-(d . n_f)) p(t_k - d . (x - x0)), p(s) = sin(omega s) on [0, t1]
-// and 0 elsewhere.  The delay is formed in FP64; the pulse in the field's
-// precision.
-template <typename T>
-__device__ __forceinline__ T src_term(const Slot<T>& S, int f, int i, int j, int k) {
-  const double s =
-      S.st - S.sh * (S.sd[0] * (i - S.si0[0]) + S.sd[1] * (j - S.si0[1]) + S.sd[2] * (k - S.si0[2]));
-  if (!(s >= 0.0 && s <= S.st1)) return T(0);
-  if constexpr (sizeof(T) == 4) return (T)S.sf[f] * sinf((float)(S.somega * s));
-  else return (T)(S.sf[f] * sin(S.somega * s));
-}
-
-// Sum of the flux terms of the faces in `faces` (bits) that carry the flux.
-template <typename T>
-__device__ __forceinline__ T src_terms(const Slot<T>& S, int faces, int i, int j, int k) {
-  T v = T(0);
-  for (int b = faces & S.src_mask; b; b &= b - 1) v += src_term(S, __ffs(b) - 1, i, j, k);
-  return v;
-}
-
-__device__ __forceinline__ int face_index(int f, int i, int j, int k, int nx, int ny);
-
-// Paper-mode adjoint: the cotangent c of the observation-face node (i, j, k)
-// enters its row as -tau c / M, M = h^3 halved on every axis on which the
-// node lies on the outer boundary (the mirror ghost of d_n lambda = -(u - u~)).
-template <typename T>
-__device__ __forceinline__ T inj_term(const Slot<T>& S, int fall, int i, int j, int k, int nx, int ny) {
-  if (S.inj == nullptr || !((fall >> S.obs_face) & 1)) return T(0);
-  const int nb = ((fall & 3) ? 1 : 0) + ((fall & 12) ? 1 : 0) + ((fall & 48) ? 1 : 0);
-  return S.inj_scale * T(1 << nb) * S.inj[face_index(S.obs_face, i, j, k, nx, ny)];
-}
-
-// field index of node (i, j, k)
-template <typename T>
-__device__ __forceinline__ long long lin(const StepArgs<T>& A, int i, int j, int k) {
-  return (long long)i + (long long)A.px * ((long long)j + (long long)A.ny * k);
-}
-
-// index of node (i, j, k) in the FEM-owned (history) box
-template <typename T>
-__device__ __forceinline__ long long hidx(const StepArgs<T>& A, int i, int j, int k) {
-  return (long long)(i - A.hx0) + (long long)A.hpx * ((long long)(j - A.fl[1]) + (long long)A.fn[1] * (k - A.fl[2]));
-}
-
-template <typename T>
-__device__ __forceinline__ bool fem_owned(const StepArgs<T>& A, int i, int j, int k) {
-  return i >= A.fl[0] && i <= A.fh[0] && j >= A.fl[1] && j <= A.fh[1] && k >= A.fl[2] &&
-         k <= A.fh[2];
-}
-
-template <typename T>
-__device__ __forceinline__ long long widx(const StepArgs<T>& A, int i, int j, int k) {
-  return (long long)(i - A.wx0) +
-         (long long)A.wpx * ((long long)(j - A.wl[1]) + (long long)A.wn[1] * (k - A.wl[2]));
-}
-
-// sum over the six axis edges of W_e (u_nb - u_c) at a FEM-owned node
-template <typename T>
-__device__ __forceinline__ T fem_lap(const StepArgs<T>& A, const T* __restrict__ Wb, const T* __restrict__ u, long long id,
-                                     int i, int j, int k, T c, T zm, T zp) {
-  const long long w = widx(A, i, j, k);
-  const T* Wx = Wb;
-  const T* Wy = Wb + A.wsz;
-  const T* Wz = Wb + 2 * A.wsz;
-  const long long wy = A.wpx;
-  const long long wz = (long long)A.wpx * A.wn[1];
-  return Wx[w] * (u[id + 1] - c) + Wx[w - 1] * (u[id - 1] - c) + Wy[w] * (u[id + A.px] - c) +
-         Wy[w - wy] * (u[id - A.px] - c) + Wz[w] * (zp - c) + Wz[w - wz] * (zm - c);
-}
-
-// ---- the all-FEM path (HYB_FEM_TET_ALL): rows gathered over tetrahedra ----
-// Coefficient a of the voxel with origin (ox, oy, oz): its value on the
-// unknown voxels, 1 elsewhere (Eq. (2.3)).
-template <typename T>
-__device__ __forceinline__ double voxel_coef(const StepArgs<T>& A, int ox, int oy, int oz) {
-  const int x = ox - A.fl[0], y = oy - A.fl[1], z = oz - A.fl[2];
-  if (x >= 0 && y >= 0 && z >= 0 && x < A.un[0] && y < A.un[1] && z < A.un[2])
-    return A.acoef[x + (long long)A.un[0] * (y + (long long)A.un[1] * z)];
-  return 1.0;
-}
-
-template <typename T>
-__device__ __forceinline__ bool lattice_interior(const StepArgs<T>& A, int i, int j, int k) {
-  return i > 0 && j > 0 && k > 0 && i < A.nx - 1 && j < A.ny - 1 && k < A.nz - 1;
-}
-
-// The finite-element row of the interior node n = (i, j, k), gathered over
-// the Kuhn tetrahedra of the (up to eight) voxels that have n as a corner:
-// sum over those tetrahedra K of a_K K^K_{n q} (element stiffness, Sec. 7.2)
-// and the lumped mass M^L_n = sum |K| / 4.  With `u` set, returns the
-// Laplacian part -(M^L)^{-1} (K u)_n of Eq. (fem) (unit spacing); else the
-// coefficient of row n on node m = (mi, mj, mk) (the diagonal when m = n).
-template <typename T>
-__device__ __noinline__ T tet_row(const StepArgs<T>& A, const T* __restrict__ u, int i, int j, int k, int mi, int mj,
-                                  int mk) {
-  const T c = u ? u[lin(A, i, j, k)] : T(0);
-  T acc = T(0);
-  double mass = 0.0;
-  for (int cn = 0; cn < 8; ++cn) {
-    const int ox = i - (cn & 1), oy = j - ((cn >> 1) & 1), oz = k - (cn >> 2);
-    if (ox < 0 || oy < 0 || oz < 0 || ox > A.nx - 2 || oy > A.ny - 2 || oz > A.nz - 2) continue;
-    const T av = (T)voxel_coef(A, ox, oy, oz);
-    for (int t = 0; t < 6; ++t) {
-      const int* V = A.kuhn_v + 4 * t;
-      int ln = -1;
-      for (int q = 0; q < 4; ++q)
-        if (V[q] == cn) ln = q;
-      if (ln < 0) continue;
-      mass += A.kuhn[96 + t] * 0.25;
-      for (int q = 0; q < 4; ++q) {
-        const int cq = V[q];
-        const int qi = ox + (cq & 1), qj = oy + ((cq >> 1) & 1), qk = oz + (cq >> 2);
-        const T kv = av * (T)A.kuhn[16 * t + 4 * ln + q];
-        if (u) {
-          if (q != ln) acc += kv * (u[lin(A, qi, qj, qk)] - c);
-        } else if (qi == mi && qj == mj && qk == mk) {
-          acc += kv;
-        }
-      }
-    }
-  }
-  return -acc / (T)mass;
-}
-
-// Coefficient of the non-absorbing row of node n on node m (Laplacian part,
-// unit spacing) on the all-FEM path: the gathered FEM row on interior
-// nodes; on the outer boundary the FDM row (mirror ghost: 2 on the inward
-// neighbour, 1 on the in-face neighbours, -6 on the node itself).
-template <typename T>
-__device__ __forceinline__ T tet_coef(const StepArgs<T>& A, int ni, int nj, int nk, int mi, int mj, int mk) {
-  if (lattice_interior(A, ni, nj, nk)) return tet_row<T>(A, nullptr, ni, nj, nk, mi, mj, mk);
-  const int d0 = mi - ni, d1 = mj - nj, d2 = mk - nk;
-  if (d0 == 0 && d1 == 0 && d2 == 0) return A.ani ? A.kdiag : T(-6);
-  if (abs(d0) + abs(d1) + abs(d2) != 1) return T(0);
-  const int ax = d0 ? 0 : (d1 ? 1 : 2), s = d0 + d1 + d2;
-  const int c = ax == 0 ? ni : (ax == 1 ? nj : nk);
-  const int n = ax == 0 ? A.nx : (ax == 1 ? A.ny : A.nz);
-  const T w = ((s > 0 && c == 0) || (s < 0 && c == n - 1)) ? T(2) : T(1);
-  return A.ani ? w * A.kapt[ax] : w;
-}
-
-// Pairing of the voxel with origin (i, j, k) on the all-FEM path:
-// kGradPairScale sum over its tetrahedra of u^T K^K lambda (a = 1).
-template <typename T>
-__device__ __forceinline__ T tet_pair(const StepArgs<T>& A, const T* __restrict__ hb, const T* __restrict__ lam,
-                                      int i, int j, int k) {
-  T u[8], l[8];
-  for (int c = 0; c < 8; ++c) {
-    const int a = c & 1, b = (c >> 1) & 1, d = c >> 2;
-    u[c] = hb[hidx(A, i + a, j + b, k + d)];
-    l[c] = lam[lin(A, i + a, j + b, k + d)];
-  }
-  T acc = T(0);
-  for (int t = 0; t < 6; ++t)
-    for (int p = 0; p < 4; ++p)
-      for (int q = 0; q < 4; ++q)
-        acc += (T)A.kuhn[16 * t + 4 * p + q] * u[A.kuhn_v[4 * t + p]] * l[A.kuhn_v[4 * t + q]];
-  return T(6) * acc;
-}
-
-// Laplacian part (without 1/h^2) of a non-absorbing row at any node:
-// FEM stencil on FEM-owned nodes, 7-point with mirror ghosts elsewhere (on
-// the all-FEM path, the gathered FEM row on every interior node).
-template <typename T>
-__device__ __noinline__ T row_lap(const StepArgs<T>& A, const T* __restrict__ W, const T* __restrict__ u, int i, int j,
-                                  int k) {
-  if (A.tet && lattice_interior(A, i, j, k)) return tet_row<T>(A, u, i, j, k, 0, 0, 0);
-  const long long id = lin(A, i, j, k);
-  const long long sz = (long long)A.px * A.ny;
-  const T c = u[id];
-  if (fem_owned(A, i, j, k)) return fem_lap(A, W, u, id, i, j, k, c, u[id - sz], u[id + sz]);
-  T lx, ly, lz;
-  if (i == 0) lx = T(2) * (u[id + 1] - c);
-  else if (i == A.nx - 1) lx = T(2) * (u[id - 1] - c);
-  else lx = (u[id - 1] - c) + (u[id + 1] - c);
-  if (j == 0) ly = T(2) * (u[id + A.px] - c);
-  else if (j == A.ny - 1) ly = T(2) * (u[id - A.px] - c);
-  else ly = (u[id - A.px] - c) + (u[id + A.px] - c);
-  if (k == 0) lz = T(2) * (u[id + sz] - c);
-  else if (k == A.nz - 1) lz = T(2) * (u[id - sz] - c);
-  else lz = (u[id - sz] - c) + (u[id + sz] - c);
-  if (A.ani) return (A.kapt[0] * lx + A.kapt[1] * ly) + A.kapt[2] * lz;
-  return (lx + ly) + lz;
-}
-
-// Coefficient of u_b^k in the absorbing row of a node on the absorbing faces
-// fb (bits): r, or with per-axis steps the mean of its faces' coefficients.
-template <typename T>
-__device__ __forceinline__ T abc_self(const StepArgs<T>& A, int fb) {
-  if (!A.ani) return A.r;
-  T rs = T(0);
-  for (int b = fb; b; b &= b - 1) rs += A.ra[(__ffs(b) - 1) >> 1];
-  return rs / T(__popc(fb));
-}
-
-// u^{k+1} at any node, recursing into the inward neighbours of absorbing
-// rows (depth D bounds the recursion: a node lies on at most 3 faces).
-template <typename T, int D>
-__device__ __noinline__ T fwd_new(const StepArgs<T>& A, const Slot<T>& S, int i, int j, int k) {
-  const long long id = lin(A, i, j, k);
-  const int fall = face_bits(i, j, k, A.nx, A.ny, A.nz);
-  if constexpr (D > 0) {
-    const int fb = fall & S.mask_f;
-    if (fb) {
-      T acc = T(0);
-#pragma unroll
-      for (int f = 0; f < 6; ++f) {
-        if (fb & (1 << f)) {
-          const int ax = f >> 1;
-          const int step = (f & 1) ? -1 : 1;  // inward
-          const int i1 = i + (ax == 0 ? step : 0);
-          const int j1 = j + (ax == 1 ? step : 0);
-          const int k1 = k + (ax == 2 ? step : 0);
-          const T rf = A.ani ? A.ra[ax] : A.r;
-          acc += S.cur[lin(A, i1, j1, k1)] - rf * fwd_new<T, D - 1>(A, S, i1, j1, k1);
-        }
-      }
-      return abc_self(A, fb) * S.cur[id] + acc / T(__popc(fb));
-    }
-  }
-  const T c = S.cur[id];
-  T v = c + ((c - S.prev[id]) + A.c2 * row_lap(A, S.W, S.cur, i, j, k));
-  if (fall & S.src_mask) v += src_terms(S, fall, i, j, k);
-  if (S.inj) v += inj_term(S, fall, i, j, k, A.nx, A.ny);
-  return v;
-}
-
-// Coefficient of the non-absorbing row of node (i,j,k) on its neighbour
-// (i,j,k) + s e_ax (Laplacian part, without 1/h^2).
-template <typename T>
-__device__ __forceinline__ T row_coef(const StepArgs<T>& A, const T* __restrict__ W, int i, int j, int k, int ax,
-                                      int s) {
-  if (fem_owned(A, i, j, k)) {
-    const long long w = widx(A, i, j, k);
-    const long long ws = ax == 0 ? 1 : (ax == 1 ? (long long)A.wpx : (long long)A.wpx * A.wn[1]);
-    return W[ax * A.wsz + (s > 0 ? w : w - ws)];
-  }
-  const int c = ax == 0 ? i : (ax == 1 ? j : k);
-  const int n = ax == 0 ? A.nx : (ax == 1 ? A.ny : A.nz);
-  const T w = ((s > 0 && c == 0) || (s < 0 && c == n - 1)) ? T(2) : T(1);
-  return A.ani ? w * A.kapt[ax] : w;
-}
-
-template <typename T>
-__device__ __forceinline__ T row_diag(const StepArgs<T>& A, const T* __restrict__ W, int i, int j, int k) {
-  if (fem_owned(A, i, j, k)) {
-    const long long w = widx(A, i, j, k);
-    const long long wy = A.wpx;
-    const long long wz = (long long)A.wpx * A.wn[1];
-    return -(W[w] + W[w - 1] + W[A.wsz + w] + W[A.wsz + w - wy] + W[2 * A.wsz + w] +
-             W[2 * A.wsz + w - wz]);
-  }
-  return A.ani ? A.kdiag : T(-6);
-}
-
-__device__ __forceinline__ int face_index(int f, int i, int j, int k, int nx, int ny) {
-  const int ax = f >> 1;
-  if (ax == 2) return i + nx * j;
-  if (ax == 1) return i + nx * k;
-  return j + ny * k;
-}
-
-// Right-hand side of the transposed step at node m:
-// (B_j^T lambda^{j+1})_m - (C_{j+1}^T lambda^{j+2})_m + c^j_m.
-template <typename T>
-__device__ __noinline__ T adj_rhs(const StepArgs<T>& A, const Slot<T>& S, int i, int j, int k) {
-  const T* __restrict__ l1 = S.cur;
-  const long long id = lin(A, i, j, k);
-  const int fbm = face_bits(i, j, k, A.nx, A.ny, A.nz);
-  T rhs;
-  if (fbm & S.mask_f) rhs = abc_self(A, fbm & S.mask_f) * l1[id];
-  else rhs = (T(2) + A.c2 * row_diag(A, S.W, i, j, k)) * l1[id];
-#pragma unroll
-  for (int ax = 0; ax < 3; ++ax) {
-#pragma unroll
-    for (int t = 0; t < 2; ++t) {
-      const int s = t ? 1 : -1;
-      const int ni = i + (ax == 0 ? s : 0);
-      const int nj = j + (ax == 1 ? s : 0);
-      const int nk = k + (ax == 2 ? s : 0);
-      if (ni < 0 || ni >= A.nx || nj < 0 || nj >= A.ny || nk < 0 || nk >= A.nz) continue;
-      const long long nid = lin(A, ni, nj, nk);
-      const int fbn = face_bits(ni, nj, nk, A.nx, A.ny, A.nz) & S.mask_f;
-      if (fbn) {
-        // absorbing row of the neighbour couples to m only when m is its
-        // inward neighbour across the face on side s of axis ax
-        const int f = 2 * ax + (s > 0 ? 1 : 0);
-        if (fbn & (1 << f)) rhs += l1[nid] / T(__popc(fbn));
-      } else {
-        rhs += A.c2 * row_coef(A, S.W, ni, nj, nk, ax, -s) * l1[nid];
-      }
-    }
-  }
-  if (!(fbm & S.mask_c)) rhs -= S.prev[id];
-  if (S.obs_r && ((fbm >> S.obs_face) & 1)) rhs += S.obs_r[face_index(S.obs_face, i, j, k, A.nx, A.ny)];
-  return rhs;
-}
-
-// adj_rhs on the all-FEM path: the transposed row gathers the coefficients
-// of every neighbouring row (the 26 nodes around m) on m.
-template <typename T>
-__device__ __noinline__ T adj_rhs_tet(const StepArgs<T>& A, const Slot<T>& S, int i, int j, int k) {
-  const T* __restrict__ l1 = S.cur;
-  const long long id = lin(A, i, j, k);
-  const int fbm = face_bits(i, j, k, A.nx, A.ny, A.nz);
-  T rhs;
-  if (fbm & S.mask_f) rhs = abc_self(A, fbm & S.mask_f) * l1[id];
-  else rhs = (T(2) + A.c2 * tet_coef(A, i, j, k, i, j, k)) * l1[id];
-  for (int d = 0; d < 27; ++d) {
-    const int dx = d % 3 - 1, dy = (d / 3) % 3 - 1, dz = d / 9 - 1;
-    if (d == 13) continue;
-    const int ni = i + dx, nj = j + dy, nk = k + dz;
-    if (ni < 0 || ni >= A.nx || nj < 0 || nj >= A.ny || nk < 0 || nk >= A.nz) continue;
-    const long long nid = lin(A, ni, nj, nk);
-    const int fbn = face_bits(ni, nj, nk, A.nx, A.ny, A.nz) & S.mask_f;
-    if (fbn) {
-      // an absorbing row couples to m only when m is its inward neighbour
-      // across one of its absorbing faces
-      if (abs(dx) + abs(dy) + abs(dz) != 1) continue;
-      const int ax = dx ? 0 : (dy ? 1 : 2), s = -(dx + dy + dz);  // m = n + s e_ax
-      const int f = 2 * ax + (s > 0 ? 0 : 1);
-      if (fbn & (1 << f)) rhs += l1[nid] / T(__popc(fbn));
-    } else {
-      rhs += A.c2 * tet_coef(A, ni, nj, nk, i, j, k) * l1[nid];
-    }
-  }
-  if (!(fbm & S.mask_c)) rhs -= S.prev[id];
-  if (S.obs_r && ((fbm >> S.obs_face) & 1)) rhs += S.obs_r[face_index(S.obs_face, i, j, k, A.nx, A.ny)];
-  return rhs;
-}
-
-// Inlined copy of adj_rhs (below).
-// Right-hand side of the transposed step at node m:
-// (B_j^T lambda^{j+1})_m - (C_{j+1}^T lambda^{j+2})_m + c^j_m.
-// Inlined form of adj_rhs for the edge tiles.  Every load is issued first,
-// predicated, and the row summed afterwards: the nodes of an edge tile's warp
-// take different branches (faces, absorbing rows, FEM weights), and loads
-// inside those branches would each wait for memory in turn.
-template <typename T>
-__device__ __forceinline__ T adj_rhs_inl(const StepArgs<T>& A, const Slot<T>& S, int i, int j, int k) {
-  const T* __restrict__ l1 = S.cur;
-  const long long id = lin(A, i, j, k);
-  const int fbm = face_bits(i, j, k, A.nx, A.ny, A.nz);
-  const long long wy = A.wpx, wz = (long long)A.wpx * A.wn[1];
-  const bool fo = fem_owned(A, i, j, k);
-  const long long w = fo ? widx(A, i, j, k) : 0;
-  const T* W = S.W;
-  T wd[6];  // this node's edge weights (FEM-owned nodes)
-  wd[0] = fo ? W[w] : T(0);
-  wd[1] = fo ? W[w - 1] : T(0);
-  wd[2] = fo ? W[A.wsz + w] : T(0);
-  wd[3] = fo ? W[A.wsz + w - wy] : T(0);
-  wd[4] = fo ? W[2 * A.wsz + w] : T(0);
-  wd[5] = fo ? W[2 * A.wsz + w - wz] : T(0);
-  const T lc = l1[id];
-  const T pv = S.prev[id];
-  const bool obs = S.obs_r != nullptr && ((fbm >> S.obs_face) & 1);
-  const T ov = obs ? S.obs_r[face_index(S.obs_face, i, j, k, A.nx, A.ny)] : T(0);
-  T nb[6], cw[6];
-  int nfb[6];
-#pragma unroll
-  for (int ax = 0; ax < 3; ++ax) {
-#pragma unroll
-    for (int t = 0; t < 2; ++t) {
-      const int q = 2 * ax + t;
-      const int s = t ? 1 : -1;
-      const int ni = i + (ax == 0 ? s : 0);
-      const int nj = j + (ax == 1 ? s : 0);
-      const int nk = k + (ax == 2 ? s : 0);
-      const bool inb = ni >= 0 && ni < A.nx && nj >= 0 && nj < A.ny && nk >= 0 && nk < A.nz;
-      nb[q] = l1[inb ? lin(A, ni, nj, nk) : id];
-      nfb[q] = inb ? (face_bits(ni, nj, nk, A.nx, A.ny, A.nz) & S.mask_f) : -1;
-      // coefficient of the neighbour's non-absorbing row on this node (row_coef)
-      const bool nfo = inb && fem_owned(A, ni, nj, nk);
-      const long long ws = ax == 0 ? 1 : (ax == 1 ? wy : wz);
-      const long long nw = nfo ? ax * A.wsz + (s < 0 ? widx(A, ni, nj, nk) : widx(A, ni, nj, nk) - ws) : 0;
-      const T wv = nfo ? W[nw] : T(0);
-      const int c = ax == 0 ? ni : (ax == 1 ? nj : nk);
-      const int n = ax == 0 ? A.nx : (ax == 1 ? A.ny : A.nz);
-      cw[q] = nfo ? wv : (((s < 0 && c == 0) || (s > 0 && c == n - 1)) ? T(2) : T(1));
-    }
-  }
-  T rhs;
-  if (fbm & S.mask_f) rhs = A.r * lc;
-  else rhs = (T(2) + A.c2 * (fo ? -(wd[0] + wd[1] + wd[2] + wd[3] + wd[4] + wd[5]) : T(-6))) * lc;
-#pragma unroll
-  for (int q = 0; q < 6; ++q) {
-    if (nfb[q] < 0) continue;
-    if (nfb[q]) {
-      // absorbing row of the neighbour couples to m only when m is its
-      // inward neighbour across the face on side s of axis ax
-      const int f = 2 * (q >> 1) + (q & 1);
-      if (nfb[q] & (1 << f)) rhs += nb[q] / T(__popc(nfb[q]));
-    } else {
-      rhs += A.c2 * cw[q] * nb[q];
-    }
-  }
-  if (!(fbm & S.mask_c)) rhs -= pv;
-  return rhs + ov;
-}
-
-// lambda^j at node m: solve E_{j-1}^T lambda^j = rhs, where E couples an
-// absorbing node b to its inward neighbours with r / L_b.
-template <typename T, int D>
-__device__ __noinline__ T adj_new(const StepArgs<T>& A, const Slot<T>& S, int i, int j, int k) {
-  T v = A.tet ? adj_rhs_tet(A, S, i, j, k) : adj_rhs(A, S, i, j, k);
-  if constexpr (D > 0) {
-#pragma unroll
-    for (int ax = 0; ax < 3; ++ax) {
-#pragma unroll
-      for (int t = 0; t < 2; ++t) {
-        const int s = t ? 1 : -1;
-        const int bi = i + (ax == 0 ? s : 0);
-        const int bj = j + (ax == 1 ? s : 0);
-        const int bk = k + (ax == 2 ? s : 0);
-        if (bi < 0 || bi >= A.nx || bj < 0 || bj >= A.ny || bk < 0 || bk >= A.nz) continue;
-        const int f = 2 * ax + (s > 0 ? 1 : 0);
-        const int fbb = face_bits(bi, bj, bk, A.nx, A.ny, A.nz) & S.mask_e;
-        if (fbb & (1 << f)) v -= ((A.ani ? A.ra[ax] : A.r) / T(__popc(fbb))) * adj_new<T, D - 1>(A, S, bi, bj, bk);
-      }
-    }
-  }
-  return v;
-}
-
-// Six times the sum over the 12 axis edges of a voxel of
-// w_e (u_p - u_q)(l_p - l_q), corner c = a + 2b + 4d at offset (a, b, d);
-// w_e = 1/3 on the edges at the voxel's diagonal corners 0 and 7, 1/6 on the
-// others.  (The factor 6 keeps divisions out of the kernels; the host scale
-// of the gradient divides it out.)
-template <typename T>
-__device__ __forceinline__ T pair_sum(const T u[8], const T l[8]) {
-  const T d3 = (u[1] - u[0]) * (l[1] - l[0]) + (u[7] - u[6]) * (l[7] - l[6]) +
-               (u[2] - u[0]) * (l[2] - l[0]) + (u[7] - u[5]) * (l[7] - l[5]) +
-               (u[4] - u[0]) * (l[4] - l[0]) + (u[7] - u[3]) * (l[7] - l[3]);
-  const T d6 = (u[3] - u[2]) * (l[3] - l[2]) + (u[5] - u[4]) * (l[5] - l[4]) +
-               (u[3] - u[1]) * (l[3] - l[1]) + (u[6] - u[4]) * (l[6] - l[4]) +
-               (u[5] - u[1]) * (l[5] - l[1]) + (u[6] - u[2]) * (l[6] - l[2]);
-  return T(2) * d3 + d6;
-}
-
-// Telegraph reading: 12 times the pairing sum_i m_i lambda_i v_i of a voxel,
-// v = u^{k+1} - u^{k-1} at its corners (the stored history) and m_i its lumped
-// mass share of corner i in units of h^3: 1/4 on the diagonal corners 0 and
-// 7, 1/12 on the others.
-template <typename T>
-__device__ __forceinline__ T damp_sum(const T u[8], const T l[8]) {
-  const T d = u[0] * l[0] + u[7] * l[7];
-  const T o = ((u[1] * l[1] + u[2] * l[2]) + (u[3] * l[3] + u[4] * l[4])) + (u[5] * l[5] + u[6] * l[6]);
-  return T(3) * d + o;
-}
-
-// pair_sum with per-axis steps: the sums over the x, y and z edges weighed by
-// kap (the voxel is a brick; dx_1^2 / dx_ax^2 relative to the x edges).
-template <typename T>
-__device__ __forceinline__ T pair_sum_ani(const StepArgs<T>& A, const T u[8], const T l[8]) {
-  const T x = T(2) * ((u[1] - u[0]) * (l[1] - l[0]) + (u[7] - u[6]) * (l[7] - l[6])) +
-              ((u[3] - u[2]) * (l[3] - l[2]) + (u[5] - u[4]) * (l[5] - l[4]));
-  const T y = T(2) * ((u[2] - u[0]) * (l[2] - l[0]) + (u[7] - u[5]) * (l[7] - l[5])) +
-              ((u[3] - u[1]) * (l[3] - l[1]) + (u[6] - u[4]) * (l[6] - l[4]));
-  const T z = T(2) * ((u[4] - u[0]) * (l[4] - l[0]) + (u[7] - u[3]) * (l[7] - l[3])) +
-              ((u[5] - u[1]) * (l[5] - l[1]) + (u[6] - u[2]) * (l[6] - l[2]));
-  return (A.kapt[0] * x + A.kapt[1] * y) + A.kapt[2] * z;
-}
-
-// pair_sum of voxel (i,j,k): u from the FEM-owned box hb, lambda from the lattice
-template <typename T>
-__device__ __forceinline__ T voxel_pair(const StepArgs<T>& A, const T* __restrict__ hb,
-                                        const T* __restrict__ lam, int i, int j, int k) {
-  const long long hy = A.hpx;
-  const long long hz = (long long)A.hpx * A.fn[1];
-  const long long h0 = hidx(A, i, j, k);
-  const long long ly = A.px;
-  const long long lz = (long long)A.px * A.ny;
-  const long long l0 = lin(A, i, j, k);
-  T u[8], l[8];
-#pragma unroll
-  for (int c = 0; c < 8; ++c) {
-    const int a = c & 1, b = (c >> 1) & 1, d = c >> 2;
-    u[c] = hb[h0 + a + b * hy + d * hz];
-    l[c] = lam[l0 + a + b * ly + d * lz];
-  }
-  return A.sdamp ? damp_sum(u, l) : pair_sum(u, l);
-}
-
-// voxel_pair with per-axis steps (the per-axis and all-node kernels)
-template <typename T>
-__device__ __forceinline__ T voxel_pair_ani(const StepArgs<T>& A, const T* __restrict__ hb,
-                                            const T* __restrict__ lam, int i, int j, int k) {
-  T u[8], l[8];
-#pragma unroll
-  for (int c = 0; c < 8; ++c) {
-    const int a = c & 1, b = (c >> 1) & 1, d = c >> 2;
-    u[c] = hb[hidx(A, i + a, j + b, k + d)];
-    l[c] = lam[lin(A, i + a, j + b, k + d)];
-  }
-  return pair_sum_ani(A, u, l);
-}
-
-// Laplacian part (without 1/h^2) of a 7-point row with unit weights.
-template <typename T>
-__device__ __forceinline__ T lap7(T xm, T xp, T ym, T yp, T zm, T zp, T c) {
-  return (xm - c) + (xp - c) + (ym - c) + (yp - c) + (zm - c) + (zp - c);
-}
-
-// Laplacian part of a non-absorbing row (inlined form of row_lap).
-template <typename T>
-__device__ __forceinline__ T row_lap_inl(const StepArgs<T>& A, const T* __restrict__ W, const T* __restrict__ u, int i,
-                                         int j, int k) {
-  const long long id = lin(A, i, j, k);
-  const long long sz = (long long)A.px * A.ny;
-  const T c = u[id];
-  if (fem_owned(A, i, j, k)) return fem_lap(A, W, u, id, i, j, k, c, u[id - sz], u[id + sz]);
-  const T xm = i > 0 ? u[id - 1] : u[id + 1];
-  const T xp = i < A.nx - 1 ? u[id + 1] : u[id - 1];
-  const T ym = j > 0 ? u[id - A.px] : u[id + A.px];
-  const T yp = j < A.ny - 1 ? u[id + A.px] : u[id - A.px];
-  const T zm = k > 0 ? u[id - sz] : u[id + sz];
-  const T zp = k < A.nz - 1 ? u[id + sz] : u[id - sz];
-  return lap7(xm, xp, ym, yp, zm, zp, c);
-}
-
-// (TET: the all-node and per-axis kernels; the all-node ones also serve the all-FEM path)
-template <typename T, bool TET>
-__device__ __forceinline__ void pair_if_voxel(const StepArgs<T>& A, const Slot<T>& S, int si, int i, int j,
-                                              int k) {
-  if (S.hist_r == nullptr) return;
-  if (i < A.fl[0] || i >= A.fl[0] + A.un[0] || j < A.fl[1] || j >= A.fl[1] + A.un[1] || k < A.fl[2] ||
-      k >= A.fl[2] + A.un[2])
-    return;
-  const long long nv = (long long)A.un[0] * A.un[1] * A.un[2];
-  const long long vid = (long long)(i - A.fl[0]) +
-                        (long long)A.un[0] * ((j - A.fl[1]) + (long long)A.un[1] * (k - A.fl[2]));
-  if (A.refvox && A.refvox[vid]) return;
-  if (TET && A.tet) A.G[(long long)si * nv + vid] += (double)tet_pair(A, S.hist_r, S.cur, i, j, k);
-  else if (TET && A.ani) A.G[(long long)si * nv + vid] += (double)voxel_pair_ani(A, S.hist_r, S.cur, i, j, k);
-  else A.G[(long long)si * nv + vid] += (double)voxel_pair(A, S.hist_r, S.cur, i, j, k);
-}
-
-template <typename T>
-__device__ __forceinline__ long long axis_stride(const StepArgs<T>& A, int ax) {
-  return ax == 0 ? 1LL : (ax == 1 ? (long long)A.px : (long long)A.px * A.ny);
-}
 
 // The "edge set" (lattices with >= 5 nodes per axis): every node whose
 // coordinate is near a face (0, 1, n-2 or n-1) on at least two axes.  It is
@@ -1076,7 +524,7 @@ __device__ __forceinline__ void interior_levels(const StepArgs<T>& A, const Slot
         atomicExch(A.err, 1);
         break;
       }
-      fence_proxy_async();
+      fence_proxy_async_shared();
       pr.issue(g, false);
     }
     // let no copy be in flight when the block exits (the consumers may have
@@ -1338,7 +786,7 @@ __device__ __forceinline__ void fwd_edge_tile(const StepArgs<T>& A, int si, int 
   }
   T plain = T(0);  // the non-absorbing row, from level-k data only
   if (valid && !fb) {
-    plain = cself + ((cself - S.prev[id]) + A.c2 * row_lap_inl(A, S.W, S.cur, i, j, k));
+    plain = cself + ((cself - S.prev[id]) + A.c2 * row_lap_inl<T, false>(A, S.W, S.cur, i, j, k));
     if (fall & S.src_mask) plain += src_terms(S, fall, i, j, k);
     if (S.inj) plain += inj_term(S, fall, i, j, k, A.nx, A.ny);
   }
@@ -1377,7 +825,7 @@ __device__ __forceinline__ void adj_edge_tile(const StepArgs<T>& A, int si, int 
   const Slot<T>& S = A.s[si];
   int i = 0, j = 0, k = 0, nf = -1, q[3];
   const bool valid = blk < A.nedge && edge_tile_node(A, blk, t, i, j, k, q, nf);
-  lam[t] = valid ? adj_rhs_inl(A, S, i, j, k) : T(0);
+  lam[t] = valid ? adj_rhs_inl<T, false>(A, S, i, j, k) : T(0);
   __syncthreads();
   for (int level = 2; level >= 0; --level) {
     T v = T(0);
@@ -1477,163 +925,6 @@ __global__ void __launch_bounds__(128) adj_all_kernel(const __grid_constant__ St
   pair_if_voxel<T, true>(A, S, si, i, j, k);
 }
 
-// Per-axis steps: each level by two launches that partition the lattice.
-// The bulk launch covers the nodes at least w nodes from every face (w = 1
-// forward, 2 transposed): each thread marches kAniZ consecutive planes of one
-// node column (blockIdx.x: 128-node segment of the row, blockIdx.y = j - w,
-// blockIdx.z = slot * chunks + chunk), keeping u of the planes below and
-// above in registers, and takes their plain rows, which need no face logic;
-// the shell launch enumerates the other nodes (the w layers next to each
-// face) and takes them through the generic rows.
-constexpr int kAniZ = 8;
-
-template <typename T, int W>
-__device__ __forceinline__ bool ani_bulk_column(const StepArgs<T>& A, int& i, int& j, int& k0, int& k1, int& si) {
-  i = W + (int)(blockIdx.x * blockDim.x + threadIdx.x);
-  j = W + (int)blockIdx.y;
-  const int chunks = (A.nz - 2 * W + kAniZ - 1) / kAniZ;
-  si = (int)blockIdx.z / chunks;
-  k0 = W + ((int)blockIdx.z - si * chunks) * kAniZ;
-  k1 = min(k0 + kAniZ, A.nz - W);  // exclusive
-  return i <= A.nx - 1 - W;
-}
-
-// Nodes of the shell of width W of one slot: the W planes at each z face,
-// then the W rows at each y face of the remaining planes, then the W nodes
-// at each x face of the remaining rows.
-template <typename T, int W>
-__device__ __forceinline__ long long ani_shell_count(const StepArgs<T>& A) {
-  return 2LL * W * ((long long)A.nx * A.ny + (long long)A.nx * (A.nz - 2 * W) +
-                    (long long)(A.ny - 2 * W) * (A.nz - 2 * W));
-}
-
-template <typename T, int W>
-__device__ __forceinline__ bool ani_shell_node(const StepArgs<T>& A, int& i, int& j, int& k, int& si) {
-  const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  const long long cnt = ani_shell_count<T, W>(A);
-  if (t >= cnt * A.nslots) return false;
-  si = (int)(t / cnt);
-  long long r = t - (long long)si * cnt;
-  const long long pa = 2LL * W * A.nx * A.ny;
-  const long long pb = 2LL * W * A.nx * (A.nz - 2 * W);
-  auto layer = [](int q, int n) { return q < W ? q : n - 2 * W + q; };  // q in [0, 2W)
-  if (r < pa) {
-    i = (int)(r % A.nx);
-    r /= A.nx;
-    j = (int)(r % A.ny);
-    k = layer((int)(r / A.ny), A.nz);
-  } else if ((r -= pa) < pb) {
-    i = (int)(r % A.nx);
-    r /= A.nx;
-    j = layer((int)(r % (2 * W)), A.ny);
-    k = W + (int)(r / (2 * W));
-  } else {
-    r -= pb;
-    i = layer((int)(r % (2 * W)), A.nx);
-    r /= 2 * W;
-    j = W + (int)(r % (A.ny - 2 * W));
-    k = W + (int)(r / (A.ny - 2 * W));
-  }
-  return true;
-}
-
-// Forward: bulk = every node off the faces (lattice rows with kap, FEM rows
-// with the edge weights, which carry kap), shell = the face nodes.
-template <typename T>
-__global__ void __launch_bounds__(128) ani_fwd_bulk_kernel(const __grid_constant__ StepArgs<T> A) {
-  int i, j, k0, k1, si;
-  if (!ani_bulk_column<T, 1>(A, i, j, k0, k1, si)) return;
-  const Slot<T>& S = A.s[si];
-  const long long sz = (long long)A.px * A.ny;
-  const T* __restrict__ u = S.cur;
-  long long id = lin(A, i, j, k0);
-  T zm = u[id - sz], c = u[id];
-  const bool col_fem = i >= A.fl[0] && i <= A.fh[0] && j >= A.fl[1] && j <= A.fh[1];
-  for (int k = k0; k < k1; ++k, id += sz) {
-    const T zp = u[id + sz];
-    const bool fo = col_fem && k >= A.fl[2] && k <= A.fh[2];
-    T lap;
-    if (fo) {
-      lap = fem_lap(A, S.W, u, id, i, j, k, c, zm, zp);
-    } else {
-      const T lx = (u[id - 1] - c) + (u[id + 1] - c);
-      const T ly = (u[id - A.px] - c) + (u[id + A.px] - c);
-      const T lz = (zm - c) + (zp - c);
-      lap = (A.kapt[0] * lx + A.kapt[1] * ly) + A.kapt[2] * lz;
-    }
-    const T val = c + ((c - S.prev[id]) + A.c2 * lap);
-    S.next[id] = val;
-    if (fo && S.hist_w) S.hist_w[hidx(A, i, j, k)] = val;
-    zm = c;
-    c = zp;
-  }
-}
-
-template <typename T>
-__global__ void __launch_bounds__(128) ani_fwd_shell_kernel(const __grid_constant__ StepArgs<T> A) {
-  int i, j, k, si;
-  if (!ani_shell_node<T, 1>(A, i, j, k, si)) return;
-  const Slot<T>& S = A.s[si];
-  const long long id = lin(A, i, j, k);
-  const T val = fwd_new<T, 3>(A, S, i, j, k);
-  S.next[id] = val;
-  if (S.obs_w && ((face_bits(i, j, k, A.nx, A.ny, A.nz) >> S.obs_face) & 1))
-    S.obs_w[face_index(S.obs_face, i, j, k, A.nx, A.ny)] = val;
-}
-
-// Transposed step: bulk = every node two or more nodes from the faces (no
-// absorbing row among its neighbours, no observation), its transposed row
-// gathered from the neighbours' rows (edge weight of a FEM-owned neighbour,
-// kap of a lattice one) in the order of adj_rhs, plus the voxel pairing;
-// shell = the nodes within one node of a face.
-template <typename T>
-__global__ void __launch_bounds__(128, 8) ani_adj_bulk_kernel(const __grid_constant__ StepArgs<T> A) {
-  int i, j, k0, k1, si;
-  if (!ani_bulk_column<T, 2>(A, i, j, k0, k1, si)) return;
-  const Slot<T>& S = A.s[si];
-  const long long sz = (long long)A.px * A.ny;
-  const T* __restrict__ l1 = S.cur;
-  long long id = lin(A, i, j, k0);
-  T zm = l1[id - sz], c = l1[id];
-  // columns next to the FEM block: some rows around them carry edge weights
-  const bool col_near = i >= A.fl[0] - 1 && i <= A.fh[0] + 1 && j >= A.fl[1] - 1 && j <= A.fh[1] + 1;
-  const T cx = A.c2 * A.kapt[0], cy = A.c2 * A.kapt[1], cz = A.c2 * A.kapt[2];
-  for (int k = k0; k < k1; ++k, id += sz) {
-    const T zp = l1[id + sz];
-    T rhs;
-    if (col_near && k >= A.fl[2] - 1 && k <= A.fh[2] + 1) {
-      rhs = (T(2) + A.c2 * row_diag(A, S.W, i, j, k)) * c;
-      rhs += A.c2 * row_coef(A, S.W, i - 1, j, k, 0, 1) * l1[id - 1];
-      rhs += A.c2 * row_coef(A, S.W, i + 1, j, k, 0, -1) * l1[id + 1];
-      rhs += A.c2 * row_coef(A, S.W, i, j - 1, k, 1, 1) * l1[id - A.px];
-      rhs += A.c2 * row_coef(A, S.W, i, j + 1, k, 1, -1) * l1[id + A.px];
-      rhs += A.c2 * row_coef(A, S.W, i, j, k - 1, 2, 1) * zm;
-      rhs += A.c2 * row_coef(A, S.W, i, j, k + 1, 2, -1) * zp;
-    } else {  // the same sums with every coefficient a lattice one
-      rhs = (T(2) + A.c2 * A.kdiag) * c;
-      rhs += cx * l1[id - 1];
-      rhs += cx * l1[id + 1];
-      rhs += cy * l1[id - A.px];
-      rhs += cy * l1[id + A.px];
-      rhs += cz * zm;
-      rhs += cz * zp;
-    }
-    S.next[id] = rhs - S.prev[id];
-    pair_if_voxel<T, true>(A, S, si, i, j, k);
-    zm = c;
-    c = zp;
-  }
-}
-
-template <typename T>
-__global__ void __launch_bounds__(128) ani_adj_shell_kernel(const __grid_constant__ StepArgs<T> A) {
-  int i, j, k, si;
-  if (!ani_shell_node<T, 2>(A, i, j, k, si)) return;
-  const Slot<T>& S = A.s[si];
-  S.next[lin(A, i, j, k)] = adj_new<T, 3>(A, S, i, j, k);
-  pair_if_voxel<T, true>(A, S, si, i, j, k);
-}
-
 template <typename T>
 __global__ void pair_kernel(const __grid_constant__ StepArgs<T> A, const T* __restrict__ hist,
                             const T* __restrict__ lam, double* __restrict__ grad) {
@@ -1648,137 +939,6 @@ __global__ void pair_kernel(const __grid_constant__ StepArgs<T> A, const T* __re
   const int i = A.fl[0] + x, j = A.fl[1] + y, k = A.fl[2] + z;
   grad[t] += (double)(A.tet ? tet_pair(A, hist, lam, i, j, k)
                              : (A.ani ? voxel_pair_ani(A, hist, lam, i, j, k) : voxel_pair(A, hist, lam, i, j, k)));
-}
-
-// Refined region of one time level, in the trailing blocks of the step
-// launch (one thread per row), the same rows for the forward and the
-// mass-scaled adjoint.  A corner n of refined voxels: the Kuhn stencil row
-// lapW (the edge weights over the voxels around n) corrected on every refined
-// voxel v around n by a_v (K9 - K8) of n's corner in v, which couples the
-// voxel's diagonal corners 0 and 7 to its six others, the six others to 0
-// and 7, and every corner to the centre; divided by n's lumped mass in units
-// of h^3.  A centre c of voxel v: a_v K9 of the centre on the eight corners
-// over its mass.  Then u^{k+1} = u^k + ((u^k - u^{k-1}) + tau^2/h^2 lap).
-// Every load of a row is issued before the row is summed.
-template <typename T, bool ADJ>
-__device__ __forceinline__ void refined_corner(const StepArgs<T>& A, const Slot<T>& S, int r) {
-  const uint2 pos = A.rpos[r];
-  const int i = (int)(pos.x & 0xffffu), j = (int)(pos.x >> 16), k = (int)pos.y;
-  const long long sy = A.px, sz = (long long)A.px * A.ny;
-  const long long id = i + sy * j + sz * k;
-  const T* __restrict__ u = S.cur;
-  // the node's 3 x 3 x 3 neighbourhood (index (dx+1) + 3 (dy+1) + 9 (dz+1)):
-  // a refined voxel's K9 - K8 couples n only to the six face neighbours
-  // (which the stencil reads too) and to the six neighbours across the
-  // diagonals of the coordinate planes with equal signs; a corner of a
-  // refined voxel lies inside the FEM block, so all of them are lattice nodes
-  T nb[27];
-#pragma unroll
-  for (int q = 0; q < 27; ++q) nb[q] = T(0);
-  nb[13] = u[id];
-  nb[12] = u[id - 1];
-  nb[14] = u[id + 1];
-  nb[10] = u[id - sy];
-  nb[16] = u[id + sy];
-  nb[4] = u[id - sz];
-  nb[22] = u[id + sz];
-  nb[9] = u[id - 1 - sy];
-  nb[17] = u[id + 1 + sy];
-  nb[3] = u[id - 1 - sz];
-  nb[23] = u[id + 1 + sz];
-  nb[1] = u[id - sy - sz];
-  nb[25] = u[id + sy + sz];
-  const T c0 = nb[13], pv = S.prev[id];
-  const long long w = widx(A, i, j, k);
-  const T* Wx = S.W;
-  const T* Wy = S.W + A.wsz;
-  const T* Wz = S.W + 2 * A.wsz;
-  const long long wy = A.wpx, wz = (long long)A.wpx * A.wn[1];
-  const T lapW = Wx[w] * (nb[14] - c0) + Wx[w - 1] * (nb[12] - c0) + Wy[w] * (nb[16] - c0) +
-                 Wy[w - wy] * (nb[10] - c0) + Wz[w] * (nb[22] - c0) + Wz[w - wz] * (nb[4] - c0);
-  // the eight voxels around n (n is corner c of the voxel with origin n - c)
-  const int ox = i - A.fl[0], oy = j - A.fl[1], oz = k - A.fl[2];
-  const int v0 = ox + A.un[0] * (oy + A.un[1] * oz), vy = A.un[0], vz = A.un[0] * A.un[1];
-  int rc[8];
-#pragma unroll
-  for (int c = 0; c < 8; ++c) {
-    const int dx = c & 1, dy = (c >> 1) & 1, dz = c >> 2;
-    const bool in = ox - dx >= 0 && oy - dy >= 0 && oz - dz >= 0 && ox - dx < A.un[0] && oy - dy < A.un[1] &&
-                    oz - dz < A.un[2];
-    rc[c] = in ? A.rcid[v0 - dx - dy * vy - dz * vz] : -1;
-  }
-  T corr = T(0), mass = T(0);
-#pragma unroll
-  for (int c = 0; c < 8; ++c) {
-    const int dx = c & 1, dy = (c >> 1) & 1, dz = c >> 2;
-    const bool ref = rc[c] >= 0;
-    mass += ref ? A.rm9[c] : A.rm8[c];
-    const T av = ref ? S.avox[v0 - dx - dy * vy - dz * vz] : T(0);
-    const T uc = ref ? S.ccur[rc[c]] : c0;
-    T sv = A.rdK[9 * c + 8] * (uc - c0);
-#pragma unroll
-    for (int q = 0; q < 8; ++q) {
-      const bool diag_c = c == 0 || c == 7, diag_q = q == 0 || q == 7;
-      if (q == c || diag_c == diag_q) continue;
-      const int o = ((q & 1) - dx + 1) + 3 * (((q >> 1) & 1) - dy + 1) + 9 * ((q >> 2) - dz + 1);
-      sv += A.rdK[9 * c + q] * (nb[o] - c0);
-    }
-    corr += av * sv;
-  }
-  const T val = c0 + ((c0 - pv) + A.c2 * ((lapW - corr) / mass));
-  S.next[id] = val;
-  if (!ADJ && S.hist_w) S.hist_w[hidx(A, i, j, k)] = val;
-}
-
-// Pairing sum u^T K9 lambda over a refined voxel's 8 corners and centre
-// (index 8), K9 the stiffness of the refined unit voxel (a = 1).
-template <typename T, typename K>
-__device__ __forceinline__ T refined_pair_sum(const T (&u)[9], const T (&l)[9], const K* __restrict__ k9) {
-  T acc = T(0);
-#pragma unroll
-  for (int p = 0; p < 9; ++p) {
-    T row = T(0);
-#pragma unroll
-    for (int q = 0; q < 9; ++q) row += (T)k9[p * 9 + q] * l[q];
-    acc += u[p] * row;
-  }
-  return acc;
-}
-
-// Centre row of refined voxel v (centre order); in the transposed step with
-// pairing the same thread also adds the voxel's pairing of (u^j, lambda^{j+1})
-// to slot si's gradient, from the lambda values the row has loaded.
-template <typename T, bool ADJ>
-__device__ __forceinline__ void refined_centre(const StepArgs<T>& A, const Slot<T>& S, int v, int si) {
-  const int vid = A.refvox_id[v];
-  const uint2 xyz = A.rvxyz[v];
-  const int x = (int)(xyz.x & 0xffffu), y = (int)(xyz.x >> 16), z = (int)xyz.y;
-  const long long l0 = lin(A, A.fl[0] + x, A.fl[1] + y, A.fl[2] + z);
-  const long long sy = A.px, sz = (long long)A.px * A.ny;
-  T q[9];
-#pragma unroll
-  for (int c = 0; c < 8; ++c) q[c] = S.cur[l0 + (c & 1) + ((c >> 1) & 1) * sy + (c >> 2) * sz];
-  const T uc = S.ccur[v], up = S.cprev[v], av = S.avox[vid];
-  q[8] = uc;
-  T sv = T(0);
-#pragma unroll
-  for (int c = 0; c < 8; ++c) sv += A.rK9[72 + c] * (q[c] - uc);
-  const T vc = uc + ((uc - up) - A.c2 * av * sv / A.rm9[8]);
-  S.cnext[v] = vc;
-  if (!ADJ && S.chist_w) S.chist_w[v] = vc;
-  if constexpr (ADJ) {
-    if (!S.hist_r) return;
-    const long long h0 = hidx(A, A.fl[0] + x, A.fl[1] + y, A.fl[2] + z);
-    const long long hy = A.hpx, hz = (long long)A.hpx * A.fn[1];
-    T u[9];
-#pragma unroll
-    for (int c = 0; c < 8; ++c) u[c] = S.hist_r[h0 + (c & 1) + ((c >> 1) & 1) * hy + (c >> 2) * hz];
-    u[8] = S.chist_r[v];
-    const long long nv = (long long)A.un[0] * A.un[1] * A.un[2];
-    // the unit-voxel K9 from the launch parameters (kGradPairScale times the pairing, as the other kernels)
-    // the only update of this entry in the launch: a reduction without return needs no load
-    atomicAdd(A.G + (long long)si * nv + vid, (double)(T(kGradPairScale) * refined_pair_sum(u, q, A.rK9)));
-  }
 }
 
 // Threads of the refined trailing blocks, per slot: the corner rows, then
@@ -1931,34 +1091,17 @@ void launch_extract_face(const StepArgs<T>& a, const T* field, int f, T* row, cu
   extract_face_kernel<T><<<(n + 255) / 256, 256, 0, st>>>(a, field, f, row);
 }
 
+template <typename T>
+void launch_all_nodes(const StepArgs<T>& a, bool adjoint, cudaStream_t st) {
+  const long long n = (long long)a.nx * a.ny * a.nz * a.nslots;
+  if (adjoint)
+    adj_all_kernel<T><<<(unsigned)((n + 127) / 128), 128, 0, st>>>(a);
+  else
+    fwd_all_kernel<T><<<(unsigned)((n + 127) / 128), 128, 0, st>>>(a);
+}
+
 template <typename T, bool ADJ>
-int launch_step(const StepArgs<T>& a, cudaStream_t st) {
-  if (a.small) {
-    const int w = ADJ ? 2 : 1;  // shell width
-    if (a.ani && !a.tet && a.nx >= 5 && a.ny >= 5 && a.nz >= 5 && a.ny <= 65535 &&
-        (long long)(a.nz - 2 * w) * a.nslots <= 65535) {
-      const dim3 grid((unsigned)((a.nx - 2 * w + 127) / 128), (unsigned)(a.ny - 2 * w),
-                      (unsigned)(((a.nz - 2 * w + kAniZ - 1) / kAniZ) * a.nslots));
-      const long long shell = 2LL * w *
-                              ((long long)a.nx * a.ny + (long long)a.nx * (a.nz - 2 * w) +
-                               (long long)(a.ny - 2 * w) * (a.nz - 2 * w)) * a.nslots;
-      const unsigned sgrid = (unsigned)((shell + 127) / 128);
-      if (ADJ) {
-        ani_adj_bulk_kernel<T><<<grid, 128, 0, st>>>(a);
-        ani_adj_shell_kernel<T><<<sgrid, 128, 0, st>>>(a);
-      } else {
-        ani_fwd_bulk_kernel<T><<<grid, 128, 0, st>>>(a);
-        ani_fwd_shell_kernel<T><<<sgrid, 128, 0, st>>>(a);
-      }
-      return 2;
-    }
-    const long long n = (long long)a.nx * a.ny * a.nz * a.nslots;
-    if (ADJ)
-      adj_all_kernel<T><<<(unsigned)((n + 127) / 128), 128, 0, st>>>(a);
-    else
-      fwd_all_kernel<T><<<(unsigned)((n + 127) / 128), 128, 0, st>>>(a);
-    return 1;
-  }
+void launch_step(const StepArgs<T>& a, cudaStream_t st) {
   StepArgs<T> b = a;
   b.nhe = ((a.nedge + 1) / 2) * a.nslots;
   const long long nref_threads = (long long)(a.nrl + a.nref) * a.nslots;
@@ -1980,17 +1123,11 @@ int launch_step(const StepArgs<T>& a, cudaStream_t st) {
     cudaLaunchKernelEx(&cfg, step_kernel<T, ADJ, true>, b);
   else
     cudaLaunchKernelEx(&cfg, step_kernel<T, ADJ, false>, b);
-  return 1;
 }
 
-template <typename T>
-int launch_forward_step(const StepArgs<T>& a, cudaStream_t st) {
-  return launch_step<T, false>(a, st);
-}
-
-template <typename T>
-int launch_adjoint_step(const StepArgs<T>& a, cudaStream_t st) {
-  return launch_step<T, true>(a, st);
+void launch_tile_step(const StepArgs<float>& a, bool adjoint, cudaStream_t st) {
+  if (adjoint) launch_step<float, true>(a, st);
+  else launch_step<float, false>(a, st);
 }
 
 template <typename T, bool ADJ>
@@ -2008,9 +1145,8 @@ int step_occupancy() {
   return n > 0 ? n : 1;
 }
 
-int step_blocks_per_sm(int precision, int adjoint) {
-  if (precision == HYB_FP32) return adjoint ? step_occupancy<float, true>() : step_occupancy<float, false>();
-  return adjoint ? step_occupancy<double, true>() : step_occupancy<double, false>();
+int tile_blocks_per_sm(bool adjoint) {
+  return adjoint ? step_occupancy<float, true>() : step_occupancy<float, false>();
 }
 
 template <typename T>
@@ -2053,8 +1189,7 @@ void launch_extract_owned(const StepArgs<T>& a, const T* field, T* box, cudaStre
 }
 
 #define HYB_INSTANTIATE(T)                                                                       \
-  template int launch_forward_step<T>(const StepArgs<T>&, cudaStream_t);                         \
-  template int launch_adjoint_step<T>(const StepArgs<T>&, cudaStream_t);                         \
+  template void launch_all_nodes<T>(const StepArgs<T>&, bool, cudaStream_t);                     \
   template void launch_pair<T>(const StepArgs<T>&, const T*, const T*, cudaStream_t);            \
   template void launch_set_coef<T>(const StepArgs<T>&, T*, T*, const double*, double, int*,     \
                                    cudaStream_t);                                                \
