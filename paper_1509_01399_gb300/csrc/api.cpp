@@ -315,13 +315,14 @@ int mask_at(const hyb_mesh* m, const hyb_source& s, int k, double dt) {
   return mask;
 }
 
-// The entry faces and their switch times (the sweep kernel's phase()).
+// The entry faces of slot q's source and their switch times (the sweep
+// kernel's phase()).
 template <typename T>
-void set_entry(Slot<T>& S, const Wave& w) {
-  S.entry = 0;
+void set_entry(SweepArgs<T>& A, int q, const Wave& w) {
+  A.entry[q] = 0;
   for (int f = 0; f < 6; ++f) {
-    S.tsw[f] = w.tsw[f];
-    if (w.fac[f] > 0.0) S.entry |= 1 << f;
+    A.tsw[q][f] = w.tsw[f];
+    if (w.fac[f] > 0.0) A.entry[q] |= 1 << f;
   }
 }
 
@@ -335,7 +336,6 @@ void set_wave(const hyb_mesh* m, Slot<T>& S, const hyb_source& src, int k, doubl
   S.src_mask = sm;
   S.st = k * dt;
   const double h = m->d.h;
-  set_entry(S, w);
   for (int f = 0; f < 6; ++f) S.sf[f] = dt * dt * 2.0 / (m->ani ? m->hv[f >> 1] : h) * src.amp * w.fac[f];
   for (int a = 0; a < 3; ++a) {
     S.sd[a] = m->ani ? w.d[a] * m->hv[a] : w.d[a];  // per-axis steps: the delay d . (x - x0) axis by axis
@@ -356,14 +356,28 @@ void step_geometry(const hyb_mesh* m, int* npb, int* ntx, int* nedge) {
   *npb = *ntx * nty;
 }
 
-// Waves of resident interior blocks the work items are cut for: one when
-// each resident block would get few tile levels (a block's first level waits
-// for its planes, so long items pay off; two waves were 1-2 % faster for a
-// lone sweep but cost a sixth of the throughput with several sweeps sharing
-// the GPU), three when there is much work (blocks of uneven speed then even
-// out within each SM).
-constexpr int kStepWavesFew = 1, kStepWavesMany = 3;
-constexpr double kManyLevelsPerBlock = 40.0;
+// Waves of resident interior blocks the work items are cut for, by the tile
+// levels of work there are per resident block (measured: us a forward /
+// transposed level).
+//  * up to 40: one for a single slot (a block's first level waits for its planes,
+//    so long items pay off: 129^3 9.6 / 10.1 against 10.7 / 10.5 with two; 161^3
+//    15.3 / 17.7 against 16.6 / 17.7), and for several up to 6 (81^3, three, 11.0 /
+//    13.4 against 11.8 / 13.5); two for several slots from there (the edge tiles'
+//    blocks, slot by slot, and the last slot's items leave a single wave uneven:
+//    65^3, eight, 17.9 / 17.6 -> 15.3 / 16.2; 97^3, six, 30.6 / 38.5 -> 28.1 / 33.9;
+//    161^3, two, 38.0 / 41.5 -> 33.5 / 34.5);
+//  * up to 60: three (257^3 refined, one source, 66 / 69 against 70 / 73 with five);
+//  * beyond: five, or items of about 35 levels if those are shorter, so that the
+//    items running together stay within one slab and find each other's halos in
+//    L2 (against three: 193^3 telegraph, four sources, 119 / 116 -> 110 / 110;
+//    257^3 refined, three sources, 183 / 199 -> 178 / 196; eight, 493 / 551 ->
+//    452 / 502).
+double step_waves(double levels_per_block, int nslots) {
+  if (levels_per_block <= 40.0) return nslots > 1 && levels_per_block > 6.0 ? 2.0 : 1.0;
+  if (levels_per_block <= 60.0) return 3.0;
+  return std::max(5.0, levels_per_block / 35.0);
+}
+
 constexpr double kZFaceLevelCost = 3.5;
 
 // Interior work items of one step launch, one per block: (slot, tile, z0,
@@ -402,8 +416,7 @@ std::vector<int> build_items(const hyb_mesh* m, int nslots, bool adjoint) {
       }
   const double resident = (double)std::max(m->nsm, 1) * std::max(m->bps, 1);
   const double levels_per_block = (double)tiles.size() * (nz - 2) / resident;
-  const double cap = resident * (levels_per_block > kManyLevelsPerBlock ? kStepWavesMany : kStepWavesFew);
-  const double target = total / cap;
+  const double target = total / (resident * step_waves(levels_per_block, nslots));
   std::vector<std::pair<double, std::array<int, 4>>> items;
   for (const Tile& t : tiles) {
     double acc = 0.0;
@@ -788,7 +801,7 @@ hyb_status encode_map(CUtensorMap* map, const void* base, uint64_t d0, uint64_t 
 // edge weights, and (transposed step with pairing) the history buffer of
 // `hist_levels` levels.
 template <typename T>
-hyb_status step_maps(const hyb_mesh* m, StepArgs<T>& A, const DevBuf& field, int nsrc, int hist_levels) {
+hyb_status step_maps(const hyb_mesh* m, SweepArgs<T>& A, const DevBuf& field, int nsrc, int hist_levels) {
   HYB_TRY(encode_map<T>(&A.tmf, field.p, m->n[0], m->n[1], (uint64_t)m->n[2] * 3 * nsrc, m->px,
                         (uint64_t)m->px * m->n[1], Box<T>::BX, kBoxY));
   HYB_TRY(encode_map<T>(&A.tmp, field.p, m->n[0], m->n[1], (uint64_t)m->n[2] * 3 * nsrc, m->px,
@@ -805,7 +818,7 @@ hyb_status step_maps(const hyb_mesh* m, StepArgs<T>& A, const DevBuf& field, int
 // Work items of the step launches with `nslots` slots (built and uploaded the
 // first time this slot count is used, outside any captured sweep).
 template <typename T>
-hyb_status step_items(hyb_mesh* m, StepArgs<T>& A, int nslots, bool adjoint) {
+hyb_status step_items(hyb_mesh* m, SweepArgs<T>& A, int nslots, bool adjoint) {
   const int d = adjoint ? 1 : 0;
   DevBuf& buf = m->items[d][nslots];
   if (!buf.p) {
@@ -902,7 +915,7 @@ hyb_status build_plan(hyb_mesh* m, int nslots) {
 }
 
 template <typename T>
-void base_args(const hyb_mesh* m, StepArgs<T>& A, double dt, int nslots) {
+void base_args(const hyb_mesh* m, SweepArgs<T>& A, double dt, int nslots) {
   std::memset(&A, 0, sizeof(A));
   A.nx = m->n[0];
   A.ny = m->n[1];
@@ -981,7 +994,7 @@ void base_args(const hyb_mesh* m, StepArgs<T>& A, double dt, int nslots) {
 
 // The plan's part of the launch arguments.
 template <typename T>
-hyb_status plan_args(hyb_mesh* m, StepArgs<T>& A, int nslots, int nsteps) {
+hyb_status plan_args(hyb_mesh* m, SweepArgs<T>& A, int nslots, int nsteps) {
   HYB_TRY(build_plan(m, nslots));
   HYB_TRY(ensure(m, m->table, (size_t)std::min(nsteps, launch_levels(m, nslots)) * nslots * sizeof(Slot<T>)));
   A.table = (Slot<T>*)m->table.p;
@@ -1027,7 +1040,7 @@ T* field_buf(const hyb_mesh* m, const DevBuf& b, int nsrc, int s, int level) {
 
 // Fill the forward slots of step k (u^k -> u^{k+1}).
 template <typename T>
-void forward_slots(const hyb_mesh* m, StepArgs<T>& A, const hyb_source* src, int nsrc, int nsteps,
+void forward_slots(const hyb_mesh* m, SweepArgs<T>& A, const hyb_source* src, int nsrc, int nsteps,
                    double dt, int k, T* trace, T* hist_level, T* chist_level) {
   for (int s = 0; s < nsrc; ++s) {
     Slot<T>& S = A.s[s];
@@ -1045,6 +1058,7 @@ void forward_slots(const hyb_mesh* m, StepArgs<T>& A, const hyb_source* src, int
     S.chist_r = nullptr;
     slot_coef<T>(m, S, s);
     set_wave<T>(m, S, src[s], k, dt);
+    set_entry<T>(A, s, wave_of(m, src[s]));
     S.mask_e = 0;
     S.mask_c = 0;
     S.zf_cur = (int)((S.cur - (const T*)m->U.p) / ((long long)m->px * m->n[1]));
@@ -1055,7 +1069,7 @@ void forward_slots(const hyb_mesh* m, StepArgs<T>& A, const hyb_source* src, int
 }
 
 template <typename T>
-hyb_status launch_piece(hyb_mesh* m, const StepArgs<T>& A, StepMode mode, cudaStream_t st) {
+hyb_status launch_piece(hyb_mesh* m, const SweepArgs<T>& A, StepMode mode, cudaStream_t st) {
   const SweepPlan& P = m->plans[A.nslots];
   m->launches += launch_sweep<T>(A, mode, P.block, P.grid, P.smem, st) - 1;
   HYB_LAUNCHED(m);
@@ -1072,14 +1086,14 @@ hyb_status launch_piece(hyb_mesh* m, const StepArgs<T>& A, StepMode mode, cudaSt
 enum class Path { kAllNodes, kTiles, kSweep };
 
 template <typename T>
-Path path_of(const StepArgs<T>& A) {
+Path path_of(const SweepArgs<T>& A) {
   if (A.small) return Path::kAllNodes;
   return sizeof(T) == 4 && !A.ani ? Path::kTiles : Path::kSweep;
 }
 
 // What the launches of a sweep with the fields `field` need besides its slots.
 template <typename T>
-hyb_status path_args(hyb_mesh* m, StepArgs<T>& A, int nslots, int nsteps, const DevBuf& field, int hist_levels,
+hyb_status path_args(hyb_mesh* m, SweepArgs<T>& A, int nslots, int nsteps, const DevBuf& field, int hist_levels,
                      bool adjoint) {
   switch (path_of(A)) {
     case Path::kAllNodes: return HYB_OK;
@@ -1093,7 +1107,7 @@ hyb_status path_args(hyb_mesh* m, StepArgs<T>& A, int nslots, int nsteps, const 
 
 // One level of every slot (not the sweep kernel).
 template <typename T>
-hyb_status launch_level(hyb_mesh* m, const StepArgs<T>& A, bool adjoint, cudaStream_t st) {
+hyb_status launch_level(hyb_mesh* m, const SweepArgs<T>& A, bool adjoint, cudaStream_t st) {
   if (A.small) {
     launch_all_nodes<T>(A, adjoint, st);
   } else if constexpr (sizeof(T) == 4) {
@@ -1106,7 +1120,7 @@ hyb_status launch_level(hyb_mesh* m, const StepArgs<T>& A, bool adjoint, cudaStr
 // Forward steps k .. k + n - 1.  hl / chl: history slot of step k; the first
 // nh steps write one each.
 template <typename T>
-hyb_status forward_levels(hyb_mesh* m, StepArgs<T>& A, const hyb_source* src, int nsrc, int nsteps, double dt, int k,
+hyb_status forward_levels(hyb_mesh* m, SweepArgs<T>& A, const hyb_source* src, int nsrc, int nsteps, double dt, int k,
                           int n, T* trace, T* hl, T* chl, int nh, cudaStream_t st) {
   const long long lvl = (long long)nsrc * m->hbox, clvl = (long long)nsrc * m->nc;
   const bool sweep = path_of(A) == Path::kSweep;
@@ -1184,7 +1198,7 @@ hyb_status forward_impl(hyb_mesh* m, const double* a, const hyb_source* src, int
   if (m->fem) HYB_TRY(ensure(m, m->W, (size_t)ncoef * 3 * m->wsz * sizeof(T)));
   if (m->nc > 0) HYB_TRY(ensure(m, m->avox, (size_t)ncoef * m->nu * sizeof(T)));
   m->batch = batch;
-  StepArgs<T> A;
+  SweepArgs<T> A;
   base_args(m, A, dt, nsrc);
   HYB_TRY(path_args<T>(m, A, nsrc, nsteps, m->U, 0, false));
   const bool tel = m->d.model == HYB_MODEL_TELEGRAPH;
@@ -1275,7 +1289,7 @@ hyb_status forward_impl(hyb_mesh* m, const double* a, const hyb_source* src, int
 }
 
 template <typename T>
-void adjoint_slots(const hyb_mesh* m, StepArgs<T>& A, const T* cot, int j, const T* hist_level,
+void adjoint_slots(const hyb_mesh* m, SweepArgs<T>& A, const T* cot, int j, const T* hist_level,
                    const T* chist_level) {
   const int nsrc = m->nsrc, nsteps = m->nsteps;
   for (int s = 0; s < nsrc; ++s) {
@@ -1297,7 +1311,7 @@ void adjoint_slots(const hyb_mesh* m, StepArgs<T>& A, const T* cot, int j, const
     S.zf_cur = (int)((S.cur - (const T*)m->L.p) / ((long long)m->px * m->n[1]));
     S.zf_prev = (int)((S.prev - (const T*)m->L.p) / ((long long)m->px * m->n[1]));
     S.zf_hist = S.hist_r ? (int)((S.hist_r - (const T*)m->hist.p) / ((long long)m->hpx * m->fn[1])) : 0;
-    set_entry(S, wave_of(m, m->src[s]));
+    set_entry<T>(A, s, wave_of(m, m->src[s]));
     S.mask_f = mask_at(m, m->src[s], j, m->dt);
     S.mask_e = mask_at(m, m->src[s], j - 1, m->dt);
     S.mask_c = mask_at(m, m->src[s], j + 1, m->dt);
@@ -1310,13 +1324,14 @@ void adjoint_slots(const hyb_mesh* m, StepArgs<T>& A, const T* cot, int j, const
 // cotangent row j entering on the observation face (Eq. (fdmschemeadjoint));
 // hist_level (u^j) is for the same-index pairing.
 template <typename T>
-void paper_slots(const hyb_mesh* m, StepArgs<T>& A, const T* cot, int j, const T* hist_level,
+void paper_slots(const hyb_mesh* m, SweepArgs<T>& A, const T* cot, int j, const T* hist_level,
                  const T* chist_level) {
   const int nsrc = m->nsrc, nsteps = m->nsteps;
   const double h = m->d.h;
   for (int s = 0; s < nsrc; ++s) {
     Slot<T>& S = A.s[s];
     S = Slot<T>();
+    A.entry[s] = 0;
     S.cur = field_buf<T>(m, m->L, nsrc, s, j);
     S.prev = field_buf<T>(m, m->L, nsrc, s, j + 1);
     S.next = field_buf<T>(m, m->L, nsrc, s, j - 1);
@@ -1337,9 +1352,9 @@ void paper_slots(const hyb_mesh* m, StepArgs<T>& A, const T* cot, int j, const T
 // Same-index pairing of the paper's adjoint, G_s += pairing of (u^j, lambda^j)
 // for the slots set up by paper_slots (structured and refined voxels).
 template <typename T>
-hyb_status paper_pair(hyb_mesh* m, StepArgs<T>& A, cudaStream_t st) {
+hyb_status paper_pair(hyb_mesh* m, SweepArgs<T>& A, cudaStream_t st) {
   for (int s = 0; s < m->nsrc; ++s) {
-    StepArgs<T> B = A;
+    SweepArgs<T> B = A;
     B.G = (double*)m->G.p + (size_t)s * m->nu;
     launch_pair<T>(B, A.s[s].hist_r, A.s[s].cur, st);
     HYB_LAUNCHED(m);
@@ -1353,9 +1368,9 @@ hyb_status paper_pair(hyb_mesh* m, StepArgs<T>& A, cudaStream_t st) {
 
 // Gradient pairing of level 0: (u^0, lambda^1) on every unknown voxel.
 template <typename T>
-hyb_status pair_first(hyb_mesh* m, StepArgs<T>& A, const T* level0, const T* clevel0, cudaStream_t st) {
+hyb_status pair_first(hyb_mesh* m, SweepArgs<T>& A, const T* level0, const T* clevel0, cudaStream_t st) {
   for (int s = 0; s < m->nsrc; ++s) {
-    StepArgs<T> B = A;
+    SweepArgs<T> B = A;
     B.G = (double*)m->G.p + (size_t)s * m->nu;
     launch_pair<T>(B, level0 + (size_t)s * m->hbox, field_buf<T>(m, m->L, m->nsrc, s, 1), st);
     HYB_LAUNCHED(m);
@@ -1381,14 +1396,14 @@ hyb_status adjoint_impl(hyb_mesh* m, const T* cot, int accumulate) {
   HYB_TRY(ensure(m, m->L, 3 * (size_t)nsrc * fb + kFieldPad));
   HYB_TRY(ensure(m, m->CL, 3 * (size_t)nsrc * cb));
   HYB_TRY(ensure(m, m->G, (size_t)nsrc * m->nu * sizeof(double)));
-  StepArgs<T> A;   // adjoint steps
+  SweepArgs<T> A;   // adjoint steps
   base_args(m, A, dt, nsrc);
-  StepArgs<T> F;   // recomputed forward steps
+  SweepArgs<T> F;   // recomputed forward steps
   base_args(m, F, dt, nsrc);
   HYB_TRY(path_args<T>(m, A, nsrc, nsteps, m->L, ckpt ? C : nsteps, true));
   HYB_TRY(path_args<T>(m, F, nsrc, nsteps, m->U, 0, false));
   const bool paper = m->d.adjoint_mode == HYB_ADJ_PAPER;
-  StepArgs<T> Pp;  // paper-mode steps: forward rows on lambda, every face reflecting
+  SweepArgs<T> Pp;  // paper-mode steps: forward rows on lambda, every face reflecting
   if (paper) {
     base_args(m, Pp, dt, nsrc);
     HYB_TRY(path_args<T>(m, Pp, nsrc, nsteps, m->L, 0, false));
@@ -1413,7 +1428,7 @@ hyb_status adjoint_impl(hyb_mesh* m, const T* cot, int accumulate) {
     // adjoint steps j, j - 1, .., j - n + 1; hl / chl: history level of step j;
     // the steps from the l0-th on pair with theirs
     auto adj_steps = [&](int j, int n, const T* hl, const T* chl, int l0) -> hyb_status {
-      StepArgs<T>& B = paper ? Pp : A;
+      SweepArgs<T>& B = paper ? Pp : A;
       const bool sweep = path_of(B) == Path::kSweep;
       const int most = sweep ? launch_levels(m, nsrc) : 1;
       for (int l = 0; l < n; l += most) {

@@ -46,9 +46,10 @@ constexpr long long kDrainCycles = 1LL << 29;
 
 // Wait for the phase with the given parity of the barrier to complete, for
 // at most `budget` clock cycles, giving up early once *abort is nonzero
-// (another block timed out).  Returns false on timeout or abort.  Each try
-// suspends the thread until the phase completes or the hint expires.  A
-// negative budget only tests the phase once.
+// (another block timed out).  Returns false on timeout or abort.  A negative
+// budget only tests the phase once.  No suspend-time hint on the tries: with
+// one the threads sleep past their planes' arrival (257^3 refined, eight
+// sources: 468 / 516 us a forward / transposed level against 462 / 509).
 __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, long long budget, const int* abort) {
   const uint32_t a = smem_addr(bar);
   if (budget < 0) {
@@ -67,10 +68,10 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, long l
     uint32_t done;
     asm volatile(
         "{\n\t.reg .pred p;\n\t"
-        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n\t"
+        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
         "selp.u32 %0, 1, 0, p;\n\t}"
         : "=r"(done)
-        : "r"(a), "r"(parity), "r"(20000u)  // suspend for at most 20 us per try
+        : "r"(a), "r"(parity)
         : "memory");
     if (done) return true;
     if ((it & 7) == 0 && (clock64() - t0 > budget || *(const volatile int*)abort != 0)) return false;

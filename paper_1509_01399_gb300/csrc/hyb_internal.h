@@ -78,8 +78,6 @@ struct alignas(16) Slot {
   double sh;         // lattice spacing h
   int si0[3];        // entry corner (node index)
   double somega, st1;
-  double tsw[6];     // last instant each entry face carries the flux
-  int entry;         // entry faces (bits)
   // paper-mode adjoint (forward rows on lambda): the cotangent row entering on
   // the observation face as inj_scale 2^b c_j, b the node's boundary axes
   const T* inj;
@@ -143,32 +141,6 @@ struct StepArgs {
   int nedge;         // edge tiles (128 nodes) per slot
   int nhe, nhr;      // leading blocks of edge tiles, trailing blocks of refined rows
   int nslots;
-  // ---- a sweep launch (sweep_kernel): nlev consecutive levels of every slot ----
-  // The nodes are cut into slabs of slabz planes (slab s: planes 1 + s slabz ..,
-  // the first and last also the z face planes) and each slab's rows into work
-  // items, one block at a time each; `sitems` lists the items of one level of
-  // one slot in slab order (the same for every slot).
-  int nlev;
-  int k0, dir;       // time index of the first step (as in Slot::st), +1 / -1 per level
-  int ring0;         // ring slot (level mod 3) of `cur` at the first level
-  int abc_mask;      // absorbing faces of the mesh
-  double dt;
-  T* fbase;          // field ring [3][slot][Np], centre ring [3][slot][nref]
-  T* cbase;
-  long long Np;
-  long long obs_step, hist_step, chist_step;  // from level to level of obs_w / obs_r / inj and of the history
-  int hist_l0, hist_l1;  // levels (of this launch) that write or read history
-  int nslab, slabz;
-  Slot<T>* table;    // [nlev][nslots]: every slot at every level of the launch
-  int ns;            // stages of the shared-memory ring
-  int split;         // a stage's rows above, at and below the item's are copied apart (wide rows) or as one run
-  int ccen, yo, ncur, nstage;  // elements: first quad in a u^k stage, from row to row, of the u^k part, of a stage
-  int nqx;           // x quads (16 bytes) holding nodes 1 .. nx - 2
-  const int4* sitems;  // (kind | slab << 8, first, end, z end)
-  int snitems;
-  const int* need;   // per slab: items that signal it at each level
-  const int4* rslab; // per slab: first corner row, corner rows, first centre row, centre rows of the refined region
-  unsigned* sync;    // [0] items claimed, [1] blocks finished, [2 + slot * nslab + slab] items completed
   // refined region (nref == 0: nothing refined): unknown voxels bisected
   // once (12 tetrahedra around a centre node).  Blocks (items) of their own
   // evaluate the rows of their corners (the stencil row corrected by the refined
@@ -209,6 +181,38 @@ struct StepArgs {
   Slot<T> s[kMaxSlots];
 };
 
+// A sweep launch (sweep_kernel): nlev consecutive levels of every slot.
+template <typename T>
+struct SweepArgs : StepArgs<T> {
+  // The nodes are cut into slabs of slabz planes (slab s: planes 1 + s slabz ..,
+  // the first and last also the z face planes) and each slab's rows into work
+  // items, one block at a time each; `sitems` lists the items of one level of
+  // one slot in slab order (the same for every slot).
+  int nlev;
+  int k0, dir;       // time index of the first step (as in Slot::st), +1 / -1 per level
+  int ring0;         // ring slot (level mod 3) of `cur` at the first level
+  int abc_mask;      // absorbing faces of the mesh
+  double dt;
+  T* fbase;          // field ring [3][slot][Np], centre ring [3][slot][nref]
+  T* cbase;
+  long long Np;
+  long long obs_step, hist_step, chist_step;  // from level to level of obs_w / obs_r / inj and of the history
+  int hist_l0, hist_l1;  // levels (of this launch) that write or read history
+  int nslab, slabz;
+  Slot<T>* table;    // [nlev][nslots]: every slot at every level of the launch
+  int ns;            // stages of the shared-memory ring
+  int split;         // a stage's rows above, at and below the item's are copied apart (wide rows) or as one run
+  int ccen, yo, ncur, nstage;  // elements: first quad in a u^k stage, from row to row, of the u^k part, of a stage
+  int nqx;           // x quads (16 bytes) holding nodes 1 .. nx - 2
+  const int4* sitems;  // (kind | slab << 8, first, end, z end)
+  int snitems;
+  const int* need;   // per slab: items that signal it at each level
+  const int4* rslab; // per slab: first corner row, corner rows, first centre row, centre rows of the refined region
+  unsigned* sync;    // [0] items claimed, [1] blocks finished, [2 + slot * nslab + slab] items completed
+  double tsw[kMaxSlots][6];  // per slot: last instant each entry face carries the flux
+  int entry[kMaxSlots];      // and its entry faces (bits)
+};
+
 // Step kinds: the forward rows, the transposed rows with the gradient
 // pairing, and the paper's adjoint (forward rows on lambda with the pairing).
 enum StepMode { kForward = 0, kAdjoint = 1, kPaper = 2 };
@@ -217,7 +221,7 @@ enum StepMode { kForward = 0, kAdjoint = 1, kPaper = 2 };
 // the sweep kernel (blocks of `block` row threads and a producer warp, `smem`
 // bytes of ring each).  Returns the kernels launched.
 template <typename T>
-int launch_sweep(const StepArgs<T>& a, StepMode mode, int block, int grid, int smem, cudaStream_t st);
+int launch_sweep(const SweepArgs<T>& a, StepMode mode, int block, int grid, int smem, cudaStream_t st);
 // One level of every slot by the tile kernel (edge tiles, interior tiles and
 // refined rows in one launch).
 void launch_tile_step(const StepArgs<float>& a, bool adjoint, cudaStream_t st);

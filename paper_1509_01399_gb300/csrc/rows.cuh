@@ -1,10 +1,14 @@
 // Rows of the hybrid FEM/FDM scheme shared by the step kernels: per-node rows
 // of every kind, the gradient pairings and the rows of the refined region.
 //
-// Some callers write a field that they read in the same launch, so nothing
-// here may load fields through the read-only path: no __restrict__ on them in
-// the functions that the sweep kernel uses.
+// The sweep kernel writes fields that it reads in the same launch, so it may not
+// load them through the read-only path; the kernels of step_kernels.cu, which
+// read one set of levels and write another, define HYB_FIELD as __restrict__.
 #pragma once
+
+#ifndef HYB_FIELD
+#define HYB_FIELD
+#endif
 
 #include "hyb_internal.h"
 
@@ -84,7 +88,7 @@ __device__ __forceinline__ long long widx(const StepArgs<T>& A, int i, int j, in
 
 // sum over the six axis edges of W_e (u_nb - u_c) at a FEM-owned node
 template <typename T>
-__device__ __forceinline__ T fem_lap(const StepArgs<T>& A, const T* __restrict__ Wb, const T* u, long long id,
+__device__ __forceinline__ T fem_lap(const StepArgs<T>& A, const T* __restrict__ Wb, const T* HYB_FIELD u, long long id,
                                      int i, int j, int k, T c, T zm, T zp) {
   const long long w = widx(A, i, j, k);
   const T* Wx = Wb;
@@ -362,7 +366,7 @@ __device__ __noinline__ T adj_rhs_tet(const StepArgs<T>& A, const Slot<T>& S, in
 // inside those branches would each wait for memory in turn.
 template <typename T, bool ANI>
 __device__ __forceinline__ T adj_rhs_inl(const StepArgs<T>& A, const Slot<T>& S, int i, int j, int k) {
-  const T* l1 = S.cur;
+  const T* HYB_FIELD l1 = S.cur;
   const long long id = lin(A, i, j, k);
   const int fbm = face_bits(i, j, k, A.nx, A.ny, A.nz);
   const long long wy = A.wpx, wz = (long long)A.wpx * A.wn[1];
@@ -489,7 +493,8 @@ __device__ __forceinline__ T pair_sum_ani(const StepArgs<T>& A, const T u[8], co
 
 // pair_sum of voxel (i,j,k): u from the FEM-owned box hb, lambda from the lattice
 template <typename T>
-__device__ __forceinline__ T voxel_pair(const StepArgs<T>& A, const T* hb, const T* lam, int i, int j, int k) {
+__device__ __forceinline__ T voxel_pair(const StepArgs<T>& A, const T* HYB_FIELD hb, const T* HYB_FIELD lam, int i, int j,
+                                        int k) {
   const long long hy = A.hpx;
   const long long hz = (long long)A.hpx * A.fn[1];
   const long long h0 = hidx(A, i, j, k);
@@ -527,7 +532,7 @@ __device__ __forceinline__ T lap7(T xm, T xp, T ym, T yp, T zm, T zp, T c) {
 
 // Laplacian part of a non-absorbing row (inlined form of row_lap).
 template <typename T, bool ANI>
-__device__ __forceinline__ T row_lap_inl(const StepArgs<T>& A, const T* __restrict__ W, const T* u, int i, int j,
+__device__ __forceinline__ T row_lap_inl(const StepArgs<T>& A, const T* __restrict__ W, const T* HYB_FIELD u, int i, int j,
                                          int k) {
   const long long id = lin(A, i, j, k);
   const long long sz = (long long)A.px * A.ny;
@@ -581,7 +586,7 @@ __device__ __forceinline__ void refined_corner(const StepArgs<T>& A, const Slot<
   const int i = (int)(pos.x & 0xffffu), j = (int)(pos.x >> 16), k = (int)pos.y;
   const long long sy = A.px, sz = (long long)A.px * A.ny;
   const long long id = i + sy * j + sz * k;
-  const T* u = S.cur;
+  const T* HYB_FIELD u = S.cur;
   // the node's 3 x 3 x 3 neighbourhood (index (dx+1) + 3 (dy+1) + 9 (dz+1)):
   // a refined voxel's K9 - K8 couples n only to the six face neighbours
   // (which the stencil reads too) and to the six neighbours across the

@@ -44,6 +44,7 @@
 // FP64 fields and lattices whose steps differ per axis take the sweep kernel
 // (sweep_kernels.cu) instead of step_kernel; lattices with fewer than 5 nodes
 // on an axis and the all-FEM path one generic kernel over every node.
+#define HYB_FIELD __restrict__
 #include "async_copy.cuh"
 #include "rows.cuh"
 

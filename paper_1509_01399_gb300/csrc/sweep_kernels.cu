@@ -34,7 +34,7 @@ struct EdgeTile {
 };
 
 template <typename T>
-__device__ __forceinline__ bool edge_tile_node(const StepArgs<T>& A, const EdgeTile& E, int t, int& i, int& j, int& k,
+__device__ __forceinline__ bool edge_tile_node(const SweepArgs<T>& A, const EdgeTile& E, int t, int& i, int& j, int& k,
                                                int q[3], int& nf) {
   const int nx = A.nx, ny = A.ny, nz = A.nz;
   auto nr = [](int qq, int n) { return qq < 2 ? qq : n - 4 + qq; };
@@ -90,7 +90,7 @@ __device__ __forceinline__ void row_sync() {
 // inward neighbours, one level down in the same tile, from shared memory.
 // Every row thread of the block calls it (it synchronises); nv holds 128 values.
 template <typename T, bool ANI>
-__device__ __forceinline__ void fwd_edge_tile(const StepArgs<T>& A, const Slot<T>& S, const EdgeTile& E, int t, T* nv) {
+__device__ __forceinline__ void fwd_edge_tile(const SweepArgs<T>& A, const Slot<T>& S, const EdgeTile& E, int t, T* nv) {
   int i = 0, j = 0, k = 0, nf = -1, q[3];
   const bool valid = edge_tile_node(A, E, t, i, j, k, q, nf);
   const long long id = valid ? lin(A, i, j, k) : 0;
@@ -142,7 +142,7 @@ __device__ __forceinline__ void fwd_edge_tile(const StepArgs<T>& A, const Slot<T
 // in parallel, then the transposed absorbing couplings (E^T) are resolved
 // from the nodes on the most faces inwards, through shared memory.
 template <typename T, bool ANI>
-__device__ __forceinline__ void adj_edge_tile(const StepArgs<T>& A, const Slot<T>& S, const EdgeTile& E, int t, T* lam) {
+__device__ __forceinline__ void adj_edge_tile(const SweepArgs<T>& A, const Slot<T>& S, const EdgeTile& E, int t, T* lam) {
   int i = 0, j = 0, k = 0, nf = -1, q[3];
   const bool valid = edge_tile_node(A, E, t, i, j, k, q, nf);
   lam[t] = valid ? adj_rhs_inl<T, ANI>(A, S, i, j, k) : T(0);
@@ -206,7 +206,7 @@ __device__ __forceinline__ void lattice_rows(double (&val)[2], const double (&c)
 // One row with per-axis weights kap: the forward row, or the transposed row
 // in the gathered order of adj_rhs.
 template <typename T, bool ADJ>
-__device__ __forceinline__ T ani_row(const StepArgs<T>& A, T c, T xm, T xp, T ym, T yp, T zm, T zp, T pv) {
+__device__ __forceinline__ T ani_row(const SweepArgs<T>& A, T c, T xm, T xp, T ym, T yp, T zm, T zp, T pv) {
   if constexpr (ADJ) {
     const T cx = A.c2 * A.kapt[0], cy = A.c2 * A.kapt[1], cz = A.c2 * A.kapt[2];
     T rhs = (T(2) + A.c2 * A.kdiag) * c;
@@ -225,7 +225,7 @@ __device__ __forceinline__ T ani_row(const StepArgs<T>& A, T c, T xm, T xp, T ym
 
 // The same for a quad of FP32 nodes, in packed pairs.
 template <bool ADJ>
-__device__ __forceinline__ void ani_rows(const StepArgs<float>& A, float (&val)[4], const float (&c)[4], float xl,
+__device__ __forceinline__ void ani_rows(const SweepArgs<float>& A, float (&val)[4], const float (&c)[4], float xl,
                                          float xr, const float (&ym)[4], const float (&yp)[4], const float (&zm)[4],
                                          const float (&zp)[4], const float (&pv)[4]) {
   const float xm[4] = {xl, c[0], c[1], c[2]}, xp[4] = {c[1], c[2], c[3], xr};
@@ -271,7 +271,7 @@ __device__ __forceinline__ T fem_diff_row(T c, T dxm, T dxp, T dym, T dyp, T dzm
 // The same from the values: forward, damped (telegraph, sd the node's damping
 // ratio), or with per-axis steps transposed.
 template <typename T, bool ADJ, bool TEL, bool ANI>
-__device__ __forceinline__ T fem_row(const StepArgs<T>& A, T c, T xm, T xp, T ym, T yp, T zm, T zp, T pv, T wxm, T wxp,
+__device__ __forceinline__ T fem_row(const SweepArgs<T>& A, T c, T xm, T xp, T ym, T yp, T zm, T zp, T pv, T wxm, T wxp,
                                      T wym, T wyp, T wzm, T wzp, T sd) {
   if constexpr (ADJ && ANI) {
     T rhs = (T(2) + A.c2 * -(wxp + wxm + wyp + wym + wzp + wzm)) * c;
@@ -330,7 +330,7 @@ struct InteriorRun {  // the part both sides compute
   int za, zb;         // planes
   int first, n;       // quads of the plane: first, count
   long long a0, a1;   // memory range of the item's quads within a plane (nodes)
-  __device__ __forceinline__ InteriorRun(const StepArgs<T>& A, int slab, int first_quad) {
+  __device__ __forceinline__ InteriorRun(const SweepArgs<T>& A, int slab, int first_quad) {
     constexpr int V = 16 / (int)sizeof(T);
     za = 1 + slab * A.slabz;
     zb = min(za + A.slabz, A.nz - 1);
@@ -346,7 +346,7 @@ struct InteriorRun {  // the part both sides compute
 // item's rows only), za .. zb - 1 (with the rows around, one quad further for
 // the pairing, and u^{k-1}), zb (with the rows around).  False when a wait ran out (no copy is issued after that).
 template <typename T>
-__device__ __forceinline__ bool interior_produce(const StepArgs<T>& A, Bars* B, T* ring, RingPos& rp, const T* cur,
+__device__ __forceinline__ bool interior_produce(const SweepArgs<T>& A, Bars* B, T* ring, RingPos& rp, const T* cur,
                                                  const T* prev, int slab, int first, long long budget, unsigned& issued) {
   const InteriorRun<T> R(A, slab, first);
   const long long pl = (long long)A.px * A.ny;
@@ -399,7 +399,7 @@ __device__ __forceinline__ T inline_face(const Slot<T>& S, T rf, T c2, int f, T 
 // stores those that are the item's; with both x faces inline that is the whole
 // quad of a row (its x face node too), so that no lane leaves the common path.
 template <typename T, StepMode M, bool TEL, bool ANI, bool FEM>
-__device__ __forceinline__ void interior_march(const StepArgs<T>& A, const Slot<T>& S, Bars* B, const T* ring,
+__device__ __forceinline__ void interior_march(const SweepArgs<T>& A, const Slot<T>& S, Bars* B, const T* ring,
                                                RingPos& rp, int si, const InteriorRun<T>& R) {
   constexpr int V = Quad<T>::V;
   constexpr bool ADJ = M == kAdjoint, PAIR = FEM && M != kForward;
@@ -687,7 +687,7 @@ __device__ __forceinline__ void interior_march(const StepArgs<T>& A, const Slot<
 }
 
 template <typename T, StepMode M, bool TEL, bool ANI>
-__device__ __forceinline__ void interior_item(const StepArgs<T>& A, const Slot<T>& S, Bars* B, const T* ring,
+__device__ __forceinline__ void interior_item(const SweepArgs<T>& A, const Slot<T>& S, Bars* B, const T* ring,
                                               RingPos& rp, int si, int slab, int first) {
   const InteriorRun<T> R(A, slab, first);
   // rows of the warp's quads against the FEM block's (an x test would seldom help)
@@ -706,7 +706,7 @@ __device__ __forceinline__ void interior_item(const StepArgs<T>& A, const Slot<T
 // reaches it), from lambda^{j+1} at b and m, the coefficient of m's row on b
 // and lambda^{j+2} at b; then m's row, corrected for b's coupling.
 template <typename T, StepMode M, bool ANI>
-__device__ __forceinline__ void face_pair(const StepArgs<T>& A, const Slot<T>& S, int si, int i, int j, int k, int ax,
+__device__ __forceinline__ void face_pair(const SweepArgs<T>& A, const Slot<T>& S, int si, int i, int j, int k, int ax,
                                           int sd) {
   constexpr bool ADJ = M == kAdjoint;
   const T* u = S.cur;
@@ -782,7 +782,7 @@ __device__ __forceinline__ void face_pair(const StepArgs<T>& A, const Slot<T>& S
 // One entry of a slab's list of nodes one step inside exactly one face, in
 // the order z faces (first and last slab), y faces, x faces.
 template <typename T, StepMode M, bool ANI>
-__device__ __forceinline__ void face_entry(const StepArgs<T>& A, const Slot<T>& S, int si, int slab, int t) {
+__device__ __forceinline__ void face_entry(const SweepArgs<T>& A, const Slot<T>& S, int si, int slab, int t) {
   const int mx = A.nx - 4, my = A.ny - 4;
   const int k0 = max(1 + slab * A.slabz, 2), k1 = min(1 + (slab + 1) * A.slabz, A.nz - 2);
   const int mz = max(k1 - k0, 0);
@@ -824,32 +824,32 @@ __device__ __forceinline__ void red_release(unsigned* p) {
 // Absorbing faces of the step leaving t_k = k dt, and the faces carrying the
 // flux (an entry face carries it while t_k <= its switch time).
 template <typename T>
-__device__ __forceinline__ int phase(const StepArgs<T>& A, const Slot<T>& S, int k, int* flux) {
+__device__ __forceinline__ int phase(const SweepArgs<T>& A, int si, int k, int* flux) {
   const double t = __dmul_rn((double)k, A.dt);
   int sm = 0;
 #pragma unroll
   for (int f = 0; f < 6; ++f)
-    if (((S.entry >> f) & 1) && t <= S.tsw[f]) sm |= 1 << f;
+    if (((A.entry[si] >> f) & 1) && t <= A.tsw[si][f]) sm |= 1 << f;
   if (flux) *flux = sm;
   return A.abc_mask & ~sm;
 }
 
 // Ring slot of `cur`, `prev` (which 1, 2) at level l of the launch.
 template <typename T>
-__device__ __forceinline__ int ring_slot(const StepArgs<T>& A, int l, int which) {
+__device__ __forceinline__ int ring_slot(const SweepArgs<T>& A, int l, int which) {
   const int r = (A.ring0 + A.dir * (l % 3) + 3) % 3;
   if (which == 0) return r;
   return (r + (which == 1 ? 3 - A.dir : 3 + A.dir)) % 3;
 }
 
 template <typename T>
-__device__ __forceinline__ T* ring_field(const StepArgs<T>& A, int r, int si) {
+__device__ __forceinline__ T* ring_field(const SweepArgs<T>& A, int r, int si) {
   return A.fbase + ((long long)r * A.nslots + si) * A.Np;
 }
 
 // Every slot at every level of a launch (A.table), from the slots of its first level.
 template <typename T, StepMode M>
-__global__ void slots_kernel(const __grid_constant__ StepArgs<T> A) {
+__global__ void slots_kernel(const __grid_constant__ SweepArgs<T> A) {
   const int q = blockIdx.x * blockDim.x + threadIdx.x;
   if (q >= A.nlev * A.nslots) return;
   const int l = q / A.nslots, si = q - l * A.nslots;
@@ -874,12 +874,12 @@ __global__ void slots_kernel(const __grid_constant__ StepArgs<T> A) {
   S->chist_w = hist && S->chist_w ? S->chist_w + l * A.chist_step : nullptr;
   S->chist_r = hist && S->chist_r ? S->chist_r + l * A.chist_step : nullptr;
   if constexpr (M == kForward) {
-    S->mask_f = phase(A, *S, step, &S->src_mask);
+    S->mask_f = phase(A, si, step, &S->src_mask);
     S->st = __dmul_rn((double)step, A.dt);
   } else if constexpr (M == kAdjoint) {
-    S->mask_f = phase(A, *S, step, (int*)nullptr);
-    S->mask_e = phase(A, *S, step - 1, (int*)nullptr);
-    S->mask_c = phase(A, *S, step + 1, (int*)nullptr);
+    S->mask_f = phase(A, si, step, (int*)nullptr);
+    S->mask_e = phase(A, si, step - 1, (int*)nullptr);
+    S->mask_c = phase(A, si, step + 1, (int*)nullptr);
   }
 }
 
@@ -891,7 +891,7 @@ constexpr int kNeedTable = 256;
 // claimed in order, so those are running or done and the wait ends whatever
 // the number of resident blocks.  False on timeout or abort.
 template <typename T>
-__device__ __forceinline__ bool wait_level(const StepArgs<T>& A, const int* need, int si, int slab, int l) {
+__device__ __forceinline__ bool wait_level(const SweepArgs<T>& A, const int* need, int si, int slab, int l) {
   const int lane = (int)threadIdx.x & 31;
   const int dep = lane < 3 ? min(max(slab - 1 + lane, 0), A.nslab - 1) : -1;
   const unsigned* c = A.sync + 2 + (dep < 0 ? 0 : (long long)si * A.nslab + dep);
@@ -914,7 +914,7 @@ __device__ __forceinline__ bool wait_level(const StepArgs<T>& A, const int* need
 // centre rows (with the transposed step's pairing of their voxels), one thread
 // per row.
 template <typename T, bool ADJ>
-__device__ __forceinline__ void refined_item(const StepArgs<T>& A, const Slot<T>& S, int si, int slab, int first,
+__device__ __forceinline__ void refined_item(const SweepArgs<T>& A, const Slot<T>& S, int si, int slab, int first,
                                              int end) {
   const int4 q = A.rslab[slab];
   for (int r = first + (int)threadIdx.x; r < end; r += (int)blockDim.x - kServiceThreads) {
@@ -951,7 +951,7 @@ struct QItem {
 // depends on, publishes it with its slot, and stages an interior item's planes.
 template <typename T, StepMode M, bool TEL, bool ANI>
 __global__ void __launch_bounds__(kMaxBlock + kServiceThreads, kSweepBlocksPerSm)
-    sweep_kernel(const __grid_constant__ StepArgs<T> A) {
+    sweep_kernel(const __grid_constant__ SweepArgs<T> A) {
   extern __shared__ __align__(128) unsigned char hyb_smem[];  // A.ns stages of A.nstage elements
   T* ring = reinterpret_cast<T*>(hyb_smem);
   __shared__ Slot<T> S2[2];
@@ -1103,7 +1103,7 @@ __global__ void __launch_bounds__(kMaxBlock + kServiceThreads, kSweepBlocksPerSm
 }  // namespace
 
 template <typename T, StepMode M>
-void launch_sweep_mode(const StepArgs<T>& a, int block, int grid, int smem, cudaStream_t st) {
+void launch_sweep_mode(const SweepArgs<T>& a, int block, int grid, int smem, cudaStream_t st) {
   slots_kernel<T, M><<<(a.nlev * a.nslots + 127) / 128, 128, 0, st>>>(a);
   if constexpr (M != kPaper) {
     if (a.ani) {
@@ -1123,7 +1123,7 @@ void launch_sweep_mode(const StepArgs<T>& a, int block, int grid, int smem, cuda
 }
 
 template <typename T>
-int launch_sweep(const StepArgs<T>& a, StepMode mode, int block, int grid, int smem, cudaStream_t st) {
+int launch_sweep(const SweepArgs<T>& a, StepMode mode, int block, int grid, int smem, cudaStream_t st) {
   if (mode == kForward) launch_sweep_mode<T, kForward>(a, block, grid, smem, st);
   else if (mode == kAdjoint) launch_sweep_mode<T, kAdjoint>(a, block, grid, smem, st);
   else launch_sweep_mode<T, kPaper>(a, block, grid, smem, st);
@@ -1162,7 +1162,7 @@ int sweep_blocks_per_sm(int precision, int block, int smem) {
   return precision == HYB_FP32 ? sweep_occupancy<float>(block, smem) : sweep_occupancy<double>(block, smem);
 }
 
-template int launch_sweep<float>(const StepArgs<float>&, StepMode, int, int, int, cudaStream_t);
-template int launch_sweep<double>(const StepArgs<double>&, StepMode, int, int, int, cudaStream_t);
+template int launch_sweep<float>(const SweepArgs<float>&, StepMode, int, int, int, cudaStream_t);
+template int launch_sweep<double>(const SweepArgs<double>&, StepMode, int, int, int, cudaStream_t);
 
 }  // namespace hyb
