@@ -1632,7 +1632,7 @@ hyb_status cg_impl(hyb_mesh* m, double* a, const T* obs, const hyb_source* src, 
   HYB_TRY(ensure(m, m->atrial, (size_t)nu * sizeof(double)));
   HYB_TRY(ensure(m, m->part, (size_t)std::max(kMisfitParts, kCgParts * kReduceBlocks) * sizeof(double)));
   HYB_TRY(ensure(m, m->scal, 16 * sizeof(double)));
-  double* part = (double*)m->part.p;
+  auto part = [m]() { return (double*)m->part.p; };  // (a misfit over large faces may move the buffer)
   double* scal = (double*)m->scal.p;
   double* g = (double*)m->g.p;
   T* tr = (T*)m->trace.p;
@@ -1643,10 +1643,10 @@ hyb_status cg_impl(hyb_mesh* m, double* a, const T* obs, const hyb_source* src, 
   HYB_TRY(adjoint_impl<T>(m, (const T*)m->cot.p, 0));
   launch_grad_finalize((const double*)m->G.p, nsrc, a, grad_scale(m), P->gamma, vol, P->a0, g, nu, m->st);
   HYB_LAUNCHED(m);
-  launch_cg_norms(g, a, P->a0, P->a_min, P->a_max, nu, part, m->st);
+  launch_cg_norms(g, a, P->a0, P->a_min, P->a_max, nu, part(), m->st);
   HYB_LAUNCHED(m);
   for (int q = 0; q < kCgParts; ++q) {
-    launch_sum(part + q * kReduceBlocks, kReduceBlocks, scal + 5 + q, m->st);
+    launch_sum(part() + q * kReduceBlocks, kReduceBlocks, scal + 5 + q, m->st);
     HYB_LAUNCHED(m);
   }
   HYB_CU(cudaMemcpyAsync(m->hscal + 5, scal + 5, kCgParts * sizeof(double), cudaMemcpyDeviceToHost, m->st));
@@ -1659,11 +1659,11 @@ hyb_status cg_impl(hyb_mesh* m, double* a, const T* obs, const hyb_source* src, 
   launch_cg_direction(g, a, P->a_min, P->a_max, vol, beta, S->d, nu, m->st);
   HYB_LAUNCHED(m);
   auto dir_stats = [&](double* dJ0, double* dmax) -> hyb_status {
-    launch_cg_dir_stats(g, S->d, nu, part, m->st);
+    launch_cg_dir_stats(g, S->d, nu, part(), m->st);
     HYB_LAUNCHED(m);
-    launch_sum(part, kReduceBlocks, scal + 2, m->st);
+    launch_sum(part(), kReduceBlocks, scal + 2, m->st);
     HYB_LAUNCHED(m);
-    launch_max(part + kReduceBlocks, kReduceBlocks, scal + 3, m->st);
+    launch_max(part() + kReduceBlocks, kReduceBlocks, scal + 3, m->st);
     HYB_LAUNCHED(m);
     HYB_CU(cudaMemcpyAsync(m->hscal + 2, scal + 2, 2 * sizeof(double), cudaMemcpyDeviceToHost, m->st));
     HYB_CU(cudaStreamSynchronize(m->st));
@@ -1684,9 +1684,9 @@ hyb_status cg_impl(hyb_mesh* m, double* a, const T* obs, const hyb_source* src, 
   const bool reseed = S->iter == 0 || !(S->alpha > 0.0) || !(J0 < S->J);
   const double at = reseed ? 0.5 / std::max(dmax, 1e-300) : S->alpha;
   double* atr = (double*)m->atrial.p;
-  launch_cg_axpy_clip(a, S->d, at, P->a_min, P->a_max, P->a0, atr, nu, part, m->st);
+  launch_cg_axpy_clip(a, S->d, at, P->a_min, P->a_max, P->a0, atr, nu, part(), m->st);
   HYB_LAUNCHED(m);
-  launch_sum(part, kReduceBlocks, scal + 4, m->st);
+  launch_sum(part(), kReduceBlocks, scal + 4, m->st);
   HYB_LAUNCHED(m);
   HYB_TRY(forward_impl<T>(m, atr, src, nsrc, nsteps, dt, tr, false));
   double Jtd = 0.0;
@@ -1695,7 +1695,7 @@ hyb_status cg_impl(hyb_mesh* m, double* a, const T* obs, const hyb_source* src, 
   HYB_CU(cudaStreamSynchronize(m->st));
   const double Jt = Jtd + 0.5 * P->gamma * vol * m->hscal[4];
   const double alpha = quadratic_step(J0, dJ0, at, Jt);
-  launch_cg_axpy_clip(a, S->d, alpha, P->a_min, P->a_max, P->a0, a, nu, part, m->st);
+  launch_cg_axpy_clip(a, S->d, alpha, P->a_min, P->a_max, P->a0, a, nu, part(), m->st);
   HYB_LAUNCHED(m);
   S->gnorm2 = gpn2;
   S->alpha = alpha;

@@ -51,3 +51,30 @@ def test_misfit_and_cotangent(H, n, nsteps, weights, precision):
     tol = 1e-15 if precision == "fp64" else 6e-8
     np.testing.assert_allclose(cot.double().cpu().numpy(), want_cot, rtol=tol, atol=0)
     m.close()
+
+
+def test_cg_step_with_more_partials_than_the_reductions(H):
+    """Two faces of 1025^2 entries: the misfit wants a larger buffer of partial
+    sums than the other reductions of a CG step, in the middle of the step.
+    The report against the same step's gradient in separate calls."""
+    import torch
+    n, h, nsteps, dt, gamma = (1025, 1025, 9), 0.1, 24, 0.05, 0.01
+    m = H.HybMesh(n, h, (2, 2, 2), (6, 6, 6), (1,) * 6, "fp64", 0, 4.0)
+    srcs = [synth.Source(f, 12.0) for f in (4, 5)]
+    gen = torch.Generator(device="cuda").manual_seed(4)
+    a = 1.0 + torch.rand(m.n_unknown, generator=gen, device="cuda", dtype=torch.float64)
+    obs = torch.randn((2, nsteps + 1, m.obs_stride), generator=gen, device="cuda", dtype=torch.float64)
+    # the step first: its misfit has to grow the buffer itself
+    step = a.clone()
+    rep = m.cg_step(step, obs, srcs, nsteps, dt, m.new_cg_state(), gamma=gamma, a0=1.0, a_min=1.0, a_max=4.0)
+    tr = m.forward(a, srcs, nsteps, dt)
+    J, cot = m.misfit(tr, obs, 1, want_cot=True)
+    m.adjoint(cot)
+    g = m.gradient(a, gamma=gamma, a0=1.0)
+    vol = h ** 3
+    want_J = J + 0.5 * gamma * vol * float(((a - 1.0) ** 2).sum())
+    want_g = float((g @ g) / vol) ** 0.5
+    # the same arithmetic, sums in another order
+    assert abs(rep.J - want_J) <= 1e-12 * want_J
+    assert abs(rep.gnorm - want_g) <= 1e-12 * want_g
+    m.close()
