@@ -58,7 +58,7 @@ def test_cg_step_with_more_partials_than_the_reductions(H):
     sums than the other reductions of a CG step, in the middle of the step.
     The report against the same step's gradient in separate calls."""
     import torch
-    n, h, nsteps, dt, gamma = (1025, 1025, 9), 0.1, 24, 0.05, 0.01
+    n, h, nsteps, dt, gamma = (1025, 1025, 9), 0.1, 48, 0.025, 0.01
     m = H.HybMesh(n, h, (2, 2, 2), (6, 6, 6), (1,) * 6, "fp64", 0, 4.0)
     srcs = [synth.Source(f, 12.0) for f in (4, 5)]
     gen = torch.Generator(device="cuda").manual_seed(4)
