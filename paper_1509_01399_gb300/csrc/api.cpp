@@ -1541,10 +1541,8 @@ double grad_scale(const hyb_mesh* m) {
   return -dt * dt / (h * h) / kGradPairScale;
 }
 
-template <typename T>
-hyb_status misfit_impl(hyb_mesh* m, const T* trace, const T* obs, int weights, double* J, T* cot) {
-  if (!m->have_run) return fail(HYB_ERR_STATE, "hyb_misfit needs a preceding hyb_forward");
-  MisfitGeom g;
+// Geometry and weights of the misfit of the last forward's traces.
+void misfit_geom(const hyb_mesh* m, int weights, MisfitGeom& g) {
   std::memset(&g, 0, sizeof g);
   g.n_src = m->nsrc;
   g.nsteps = m->nsteps;
@@ -1561,11 +1559,19 @@ hyb_status misfit_impl(hyb_mesh* m, const T* trace, const T* obs, int weights, d
   g.wt = quad ? m->dt : 1.0;
   for (int s = 0; s < m->nsrc; ++s) g.hh[s] = quad ? face_cell_area(m, m->src[s].face) : 1.0;
   g.halve = quad ? 1 : 0;
-  HYB_TRY(ensure(m, m->part, (size_t)misfit_parts(g) * sizeof(double)));
+}
+
+template <typename T>
+hyb_status misfit_impl(hyb_mesh* m, const T* trace, const T* obs, int weights, double* J, T* cot) {
+  if (!m->have_run) return fail(HYB_ERR_STATE, "hyb_misfit needs a preceding hyb_forward");
+  MisfitGeom g;
+  misfit_geom(m, weights, g);
+  const long long parts = misfit_parts(g, g.n_src) * g.n_src;
+  HYB_TRY(ensure(m, m->part, (size_t)parts * sizeof(double)));
   HYB_TRY(ensure(m, m->scal, 16 * sizeof(double)));
-  const int parts = launch_misfit<T>(g, trace, obs, cot, (double*)m->part.p, m->st);
+  launch_misfit<T>(g, g.n_src, trace, obs, cot, (double*)m->part.p, m->st);
   HYB_LAUNCHED(m);
-  launch_sum((double*)m->part.p, parts, (double*)m->scal.p + 8, m->st);
+  launch_sum((double*)m->part.p, (int)parts, (double*)m->scal.p + 8, m->st);
   HYB_LAUNCHED(m);
   if (J) {
     HYB_CU(cudaMemcpyAsync(m->hscal + 8, (double*)m->scal.p + 8, sizeof(double), cudaMemcpyDeviceToHost, m->st));
@@ -1575,37 +1581,24 @@ hyb_status misfit_impl(hyb_mesh* m, const T* trace, const T* obs, int weights, d
   return HYB_OK;
 }
 
-// Per-slot misfit of a batch: slot s's trace rows reduced on their own (the
-// same launches and summation order as a one-slot mesh), J of slot s to
-// J_host[s] (host, synchronises), cotangent rows as hyb_misfit.
+// Per-slot misfit of a batch: every slot's rows by the blocks a one-slot mesh
+// would use, all in one launch, and summed on their own (the same summation
+// order); J of slot s to J_host[s] (host, synchronises), cotangent rows as
+// hyb_misfit.
 template <typename T>
 hyb_status misfit_batch_impl(hyb_mesh* m, const T* trace, const T* obs, int weights, double* J_host, T* cot) {
   if (!m->have_run) return fail(HYB_ERR_STATE, "hyb_misfit_batch needs a preceding forward");
   const int nsrc = m->nsrc;
-  const size_t rows = (size_t)(m->nsteps + 1) * m->obs_stride;
   HYB_TRY(ensure(m, m->scal, (16 + kMaxSlots) * sizeof(double)));
   double* out = (double*)m->scal.p + 16;
-  const bool quad = weights == HYB_WEIGHTS_QUADRATURE;
-  for (int s = 0; s < nsrc; ++s) {
-    MisfitGeom g;
-    std::memset(&g, 0, sizeof g);
-    g.n_src = 1;
-    g.nsteps = m->nsteps;
-    g.stride = m->obs_stride;
-    const int ax = m->src[s].face >> 1;
-    g.face[0] = m->src[s].face;
-    g.np[0] = m->n[ax == 0 ? 1 : 0];
-    g.nq[0] = m->n[ax == 2 ? 1 : 2];
-    g.wt = quad ? m->dt : 1.0;
-    g.hh[0] = quad ? face_cell_area(m, m->src[s].face) : 1.0;
-    g.halve = quad ? 1 : 0;
-    HYB_TRY(ensure(m, m->part, (size_t)misfit_parts(g) * sizeof(double)));
-    const int parts =
-        launch_misfit<T>(g, trace + s * rows, obs + s * rows, cot ? cot + s * rows : nullptr, (double*)m->part.p, m->st);
-    HYB_LAUNCHED(m);
-    launch_sum((double*)m->part.p, parts, out + s, m->st);
-    HYB_LAUNCHED(m);
-  }
+  MisfitGeom g;
+  misfit_geom(m, weights, g);
+  const long long parts = misfit_parts(g, 1);
+  HYB_TRY(ensure(m, m->part, (size_t)parts * nsrc * sizeof(double)));
+  launch_misfit<T>(g, 1, trace, obs, cot, (double*)m->part.p, m->st);
+  HYB_LAUNCHED(m);
+  launch_sum((double*)m->part.p, (int)parts, out, m->st, nsrc);
+  HYB_LAUNCHED(m);
   if (J_host) {
     HYB_CU(cudaMemcpyAsync(m->hscal, out, nsrc * sizeof(double), cudaMemcpyDeviceToHost, m->st));
     HYB_CU(cudaStreamSynchronize(m->st));

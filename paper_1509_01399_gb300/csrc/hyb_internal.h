@@ -270,13 +270,16 @@ struct MisfitGeom {
   double hh[kMaxSlots];              // face weight scale per source (1, or the in-face cell area)
   int halve;                         // halve the face weight on the face border
 };
-// Returns the number of partials written, at most misfit_parts(g).
+// The blocks are shaped for `share` sources sharing the GPU (so that a source's
+// partials do not depend on how many run in the launch); every source writes
+// misfit_parts(g, share) partials.
 constexpr int kMisfitParts = 4096;
-long long misfit_parts(const MisfitGeom& g);
+long long misfit_parts(const MisfitGeom& g, int share);
 template <typename T>
-int launch_misfit(const MisfitGeom& g, const T* trace, const T* obs, T* cot, double* partials, cudaStream_t st);
-// out[0] = sum of `n` partials (one block, fixed order).
-void launch_sum(const double* partials, int n, double* out, cudaStream_t st);
+void launch_misfit(const MisfitGeom& g, int share, const T* trace, const T* obs, T* cot, double* partials,
+                   cudaStream_t st);
+// out[q] = sum of the q-th `n` partials, q < count (one block each, fixed order).
+void launch_sum(const double* partials, int n, double* out, cudaStream_t st, int count = 1);
 // g = scale * sum_s G_s + gamma * vol * (a - a0), G holding n_src arrays of n
 void launch_grad_finalize(const double* G, int n_src, const double* a, double scale, double gamma,
                           double vol, double a0, double* g, long long n, cudaStream_t st);

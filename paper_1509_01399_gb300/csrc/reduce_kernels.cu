@@ -139,11 +139,13 @@ __global__ void __launch_bounds__(kReduceThreads) misfit_kernel(const MisfitGeom
   if (threadIdx.x == 0) partials[((size_t)s * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x] = acc;
 }
 
+// out[b] = sum of the b-th n entries of p (block b).
 __global__ void sum_kernel(const double* __restrict__ p, int n, double* out) {
+  p += (size_t)blockIdx.x * n;
   double acc = 0.0;
   for (int i = threadIdx.x; i < n; i += blockDim.x) acc += p[i];
   acc = block_sum(acc);
-  if (threadIdx.x == 0) *out = acc;
+  if (threadIdx.x == 0) out[blockIdx.x] = acc;
 }
 
 __global__ void max_kernel(const double* __restrict__ p, int n, double* out) {
@@ -238,33 +240,37 @@ __global__ void __launch_bounds__(kReduceThreads) cg_axpy_clip_kernel(
 
 }  // namespace
 
-// Column blocks of one trace row.
-static long long misfit_cols(const MisfitGeom& g) {
+// Blocks of one source's misfit: columns, and rows per block, so that `share`
+// sources together make about kMisfitParts / 2 blocks, each of at least eight rows.
+static void misfit_shape(const MisfitGeom& g, int share, long long* cols, long long* rows) {
   const int per = kReduceThreads * kMisfitCols;
-  return ((long long)g.stride + per - 1) / per;
+  const long long all = g.nsteps + 1;
+  *cols = ((long long)g.stride + per - 1) / per;
+  *rows = (all * *cols * share + kMisfitParts / 2 - 1) / (kMisfitParts / 2);
+  if (*rows < 8) *rows = 8;
+  if (*rows > all) *rows = all;
 }
 
-long long misfit_parts(const MisfitGeom& g) {
-  const long long least = misfit_cols(g) * g.n_src;
-  return least > kMisfitParts ? least : kMisfitParts;
+long long misfit_parts(const MisfitGeom& g, int share) {
+  long long cols, rows;
+  misfit_shape(g, share, &cols, &rows);
+  return cols * ((g.nsteps + 1 + rows - 1) / rows);
 }
 
 template <typename T>
-int launch_misfit(const MisfitGeom& g, const T* trace, const T* obs, T* cot, double* partials, cudaStream_t st) {
-  const long long cols = misfit_cols(g);
-  // rows per block: about kMisfitParts / 2 blocks, at most kMisfitParts
-  const long long all = g.nsteps + 1;
-  long long rows = (all * cols * g.n_src + kMisfitParts / 2 - 1) / (kMisfitParts / 2);
-  while (cols * g.n_src * ((all + rows - 1) / rows) > kMisfitParts && rows < all) ++rows;
-  const dim3 grid((unsigned)cols, (unsigned)((all + rows - 1) / rows), (unsigned)g.n_src);
+void launch_misfit(const MisfitGeom& g, int share, const T* trace, const T* obs, T* cot, double* partials,
+                   cudaStream_t st) {
+  long long cols, rows;
+  misfit_shape(g, share, &cols, &rows);
+  const dim3 grid((unsigned)cols, (unsigned)((g.nsteps + 1 + rows - 1) / rows), (unsigned)g.n_src);
   misfit_kernel<T><<<grid, kReduceThreads, 0, st>>>(g, (int)rows, trace, obs, cot, partials);
-  return (int)(grid.x * grid.y * grid.z);
 }
-template int launch_misfit<float>(const MisfitGeom&, const float*, const float*, float*, double*, cudaStream_t);
-template int launch_misfit<double>(const MisfitGeom&, const double*, const double*, double*, double*, cudaStream_t);
+template void launch_misfit<float>(const MisfitGeom&, int, const float*, const float*, float*, double*, cudaStream_t);
+template void launch_misfit<double>(const MisfitGeom&, int, const double*, const double*, double*, double*,
+                                    cudaStream_t);
 
-void launch_sum(const double* partials, int n, double* out, cudaStream_t st) {
-  sum_kernel<<<1, 256, 0, st>>>(partials, n, out);
+void launch_sum(const double* partials, int n, double* out, cudaStream_t st, int count) {
+  sum_kernel<<<count, n > 1024 ? 1024 : 256, 0, st>>>(partials, n, out);
 }
 
 void launch_max(const double* partials, int n, double* out, cudaStream_t st) {
