@@ -350,11 +350,11 @@ def run_anisotropic(H, dev, peak, peak_kind, nsteps=600, reps=2, sweep_levels=10
     roof = {}
     for k, b, ms in (("forward", fb, fwd_ms), ("adjoint", ab, adj_ms)):
         gbs = b / (ms * 1e-3) / 1e9
-        roof[k] = {"kernel": "sweep_kernel<float,%s> (per axis), one level of a launch of many" % k,
+        roof[k] = {"kernel": "step_kernel<float,%s> (per-axis steps)" % k,
                    "bound": "hbm", "achieved": gbs, "peak": peak, "unit": "GB/s", "frac": gbs / peak,
                    "peak_kind": peak_kind, "algorithmic_bytes_per_launch": b, "launch_ms": ms}
     return {"workload": "257 x 193 x 321 lattice on [-1,1]^3, steps 2/256, 2/192, 2/320, FEM block = central half, "
-                        "8 sources, no refinement, %d steps, checkpoints every 50, FP32 (sweep kernel)" % nsteps,
+                        "8 sources, no refinement, %d steps, checkpoints every 50, FP32" % nsteps,
             "gradient_ms": el, "value": per / (el * 1e-3) / 1e9, "unit": UNIT,
             "counted": "n_src x lattice nodes x N_t x 2 (forward + adjoint) per gradient evaluation",
             "roofline": roof, "J": J, "gnorm": gn}

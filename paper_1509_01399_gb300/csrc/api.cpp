@@ -118,7 +118,7 @@ struct hyb_mesh {
   DevBuf I0, IC0;               // initial state of Model Problem 1: u^0, u^{-1} (padded fields), centres
   DevBuf acopy, kuhn, kuhn_v;   // all-FEM path: coefficient of the last forward, Kuhn element tables
   bool have_init = false;
-  bool ani = false;          // the lattice steps differ per axis (every level by the bulk and shell kernels)
+  bool ani = false;          // the lattice steps differ per axis
   double hv[3] = {0, 0, 0};  // lattice step per axis
   cudaStream_t cap = nullptr;  // private stream used only to capture sweep graphs
   // work items of a level per slot count; built once and kept (captured sweep
@@ -445,9 +445,9 @@ std::vector<int> build_items(const hyb_mesh* m, int nslots, bool adjoint) {
   return out;
 }
 
-// x groups of 16 bytes that hold the nodes 1 .. nx - 2.
+// x groups of 16 bytes (two FP64 values) that hold the nodes 1 .. nx - 2.
 int quads_of_row(const hyb_mesh* m) {
-  return (m->n[0] - 2) / (m->d.precision == HYB_FP32 ? 4 : 2) + 1;
+  return (m->n[0] - 2) / 2 + 1;
 }
 
 // Bytes behind a field ring that the last item's plane copy may reach into.
@@ -846,7 +846,7 @@ hyb_status build_plan(hyb_mesh* m, int nslots) {
   SweepPlan& P = m->plans[nslots];
   if (P.nitems) return HYB_OK;
   const int nx = m->n[0], ny = m->n[1], nz = m->n[2], px = m->px;
-  const int V = m->d.precision == HYB_FP32 ? 4 : 2;
+  constexpr int V = 2;
   const int nqx = quads_of_row(m);
   const long long nq = (long long)(ny - 2) * nqx;
   const double work = (double)nslots * nq * (nz - 2);  // quads of a level
@@ -868,7 +868,7 @@ hyb_status build_plan(hyb_mesh* m, int nslots) {
   while (bps > 1 && kMaxRing / bps / stage < 4) --bps;
   P.ns = std::min(kMaxStages, kMaxRing / bps / stage);
   P.smem = P.ns * stage;
-  const int resident = m->nsm * sweep_blocks_per_sm(m->d.precision, block, P.smem);
+  const int resident = m->nsm * sweep_blocks_per_sm(block, P.smem);
   const int B = (int)std::min((double)kMaxMarch, std::max(1.0, std::floor(work / block / (kItemsPerBlock * resident))));
   const int nslab = (nz - 2 + B - 1) / B;
   std::vector<int> items, need(nslab, 0), rslab(4 * (size_t)nslab, 0);
@@ -944,11 +944,13 @@ void base_args(const hyb_mesh* m, SweepArgs<T>& A, double dt, int nslots) {
   A.c2 = (T)(dt * dt / (h * h));
   A.r = (T)((h - dt) / (h + dt));
   // the generic kernel: lattices without an interior, and beyond the sweep
-  // kernel's 32-bit item indices
+  // kernel's 32-bit item indices or, with per-axis steps, the tile kernel's
+  // 32-bit node offsets
   A.small = (m->n[0] < 5 || m->n[1] < 5 || m->n[2] < 5) ? 1 : 0;
-  if ((m->d.precision == HYB_FP64 || m->ani) && m->nc == 0 &&
+  if (m->d.precision == HYB_FP64 && m->nc == 0 &&
       ((long long)m->n[0] * m->n[1] + (m->n[0] + (long long)m->n[1]) * kMaxMarch >= 1LL << 30 || m->n[2] >= 1 << 23))
     A.small = 1;
+  if (m->d.precision == HYB_FP32 && m->ani && (long long)m->px * m->n[1] * m->n[2] >= 1LL << 31) A.small = 1;
   if (m->ani) {  // axis terms weighed by kap
     A.ani = 1;
     for (int a = 0; a < 3; ++a) {
@@ -1070,25 +1072,29 @@ void forward_slots(const hyb_mesh* m, SweepArgs<T>& A, const hyb_source* src, in
 
 template <typename T>
 hyb_status launch_piece(hyb_mesh* m, const SweepArgs<T>& A, StepMode mode, cudaStream_t st) {
-  const SweepPlan& P = m->plans[A.nslots];
-  m->launches += launch_sweep<T>(A, mode, P.block, P.grid, P.smem, st) - 1;
-  HYB_LAUNCHED(m);
+  if constexpr (sizeof(T) == 8) {
+    const SweepPlan& P = m->plans[A.nslots];
+    m->launches += launch_sweep(A, mode, P.block, P.grid, P.smem, st) - 1;
+    HYB_LAUNCHED(m);
+  }
   return HYB_OK;
 }
 
 // How the levels of a mesh run: the generic all-node kernel (lattices with
 // fewer than 5 nodes on an axis, the all-FEM path), the tile kernel (FP32
-// fields with equal steps), or the sweep kernel.  FP32 with equal steps stays
-// with the tiles, whose edge weights and history are staged: 257^3, eight
-// sources, refined, 0.49 / 0.54 ms a level against 0.66 / 0.92 ms by the sweep
-// kernel (without a FEM block 0.40 against 0.32).  FP64 and per-axis steps gain
-// 1.3 - 2.5 times from the sweep kernel at every size measured (its comment).
+// fields), or the sweep kernel (FP64 fields).  The tiles stage the edge weights
+// and history that FP32 rows would wait for: 257^3, eight sources, refined,
+// 0.47 / 0.51 ms a level against 0.66 / 0.92 ms by the sweep kernel (without a FEM
+// block 0.40 against 0.32); per-axis steps, 257 x 193 x 321 with eight sources,
+// 0.38 / 0.41 ms against 0.52 / 0.71, and faster at every size down to 21 x 18 x
+// 26 (10.3 against 11.1 us a step pair).  FP64 rows wait for the FP64 pipe, and
+// gain 1.5 - 1.7 times from the sweep kernel at every size measured (its comment).
 enum class Path { kAllNodes, kTiles, kSweep };
 
 template <typename T>
 Path path_of(const SweepArgs<T>& A) {
   if (A.small) return Path::kAllNodes;
-  return sizeof(T) == 4 && !A.ani ? Path::kTiles : Path::kSweep;
+  return sizeof(T) == 4 ? Path::kTiles : Path::kSweep;
 }
 
 // What the launches of a sweep with the fields `field` need besides its slots.
@@ -1842,7 +1848,7 @@ hyb_status hyb_mesh_create(const hyb_mesh_desc* d, void* stream, hyb_mesh** out)
         cudaDeviceGetAttribute(&m->nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
       cudaGetLastError();
       st = fail(HYB_ERR_CUDA, "device query failed");
-    } else if (d->precision == HYB_FP32 && !ani) {
+    } else if (d->precision == HYB_FP32) {
       m->bps = std::min(tile_blocks_per_sm(false), tile_blocks_per_sm(true));
     }
   }

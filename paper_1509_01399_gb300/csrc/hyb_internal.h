@@ -11,7 +11,7 @@
 namespace hyb {
 
 constexpr int kMaxSlots = 16;   // problems advanced by one sweep launch
-// ---- tile kernel (step_kernels.cu: FP32 fields, equal steps) ----
+// ---- tile kernel (step_kernels.cu: FP32 fields) ----
 constexpr int kStepBlock = 288;  // threads per block of the step kernel (9 warps)
 constexpr int kTileX = 32;       // interior thread tile (x): one warp per tile row
 constexpr int kTileY = 16;       // interior tile (y): two rows per consumer thread
@@ -41,7 +41,7 @@ struct Box {
 // first node (x) of interior tile 0 for a mesh of the given precision
 inline int tile_x0(int precision) { return precision == HYB_FP32 ? Box<float>::x0 : Box<double>::x0; }
 
-// ---- sweep kernel (sweep_kernels.cu: FP64 fields, per-axis steps) ----
+// ---- sweep kernel (sweep_kernels.cu: FP64 fields) ----
 constexpr int kMaxBlock = 224;   // row threads per block of the sweep kernel, at most (with the producer warp
                                  // 256: two blocks of 128 registers a thread per SM)
 constexpr int kServiceThreads = 32;  // its producer warp
@@ -220,8 +220,7 @@ enum StepMode { kForward = 0, kAdjoint = 1, kPaper = 2 };
 // A.nlev consecutive levels of every slot: fills A.table, then one launch of
 // the sweep kernel (blocks of `block` row threads and a producer warp, `smem`
 // bytes of ring each).  Returns the kernels launched.
-template <typename T>
-int launch_sweep(const SweepArgs<T>& a, StepMode mode, int block, int grid, int smem, cudaStream_t st);
+int launch_sweep(const SweepArgs<double>& a, StepMode mode, int block, int grid, int smem, cudaStream_t st);
 // One level of every slot by the tile kernel (edge tiles, interior tiles and
 // refined rows in one launch).
 void launch_tile_step(const StepArgs<float>& a, bool adjoint, cudaStream_t st);
@@ -232,7 +231,7 @@ template <typename T>
 void launch_all_nodes(const StepArgs<T>& a, bool adjoint, cudaStream_t st);
 // Resident blocks per SM of the sweep kernel by its registers and `smem` bytes of
 // ring (every variant of the precision gets that ring size), at least 1.
-int sweep_blocks_per_sm(int precision, int block, int smem);
+int sweep_blocks_per_sm(int block, int smem);
 // G[c] += voxel pairing of (u^0 in hist box, lambda^1) for one slot.
 template <typename T>
 void launch_pair(const StepArgs<T>& a, const T* hist, const T* lam, cudaStream_t st);

@@ -511,7 +511,7 @@ __device__ __forceinline__ T voxel_pair(const StepArgs<T>& A, const T* HYB_FIELD
   return A.sdamp ? damp_sum(u, l) : pair_sum(u, l);
 }
 
-// voxel_pair with per-axis steps (the per-axis and all-node kernels)
+// voxel_pair with per-axis steps
 template <typename T>
 __device__ __forceinline__ T voxel_pair_ani(const StepArgs<T>& A, const T* hb, const T* lam, int i, int j, int k) {
   T u[8], l[8];
@@ -549,7 +549,7 @@ __device__ __forceinline__ T row_lap_inl(const StepArgs<T>& A, const T* __restri
   return lap7(xm, xp, ym, yp, zm, zp, c);
 }
 
-// (TET: the all-node and per-axis kernels; the all-node ones also serve the all-FEM path)
+// (TET: per-axis steps or the all-FEM path may be on)
 template <typename T, bool TET>
 __device__ __forceinline__ void pair_if_voxel(const StepArgs<T>& A, const Slot<T>& S, int si, int i, int j,
                                               int k) {

@@ -41,9 +41,16 @@
 // w_e = 2 or 1 (six times the edge weights 1/3 and 1/6); the host scales it
 // by -tau^2 / (6 h^2) (Eq. (gradient1)).
 //
-// FP64 fields and lattices whose steps differ per axis take the sweep kernel
-// (sweep_kernels.cu) instead of step_kernel; lattices with fewer than 5 nodes
-// on an axis and the all-FEM path one generic kernel over every node.
+// Lattices whose steps differ per axis (ANI) weigh the axis terms by kap and take
+// the faces' own absorbing coefficients, by variants of the same kernel without
+// refinement (those weights are operands from the argument block and cost no
+// registers): 257 x 193 x 321, eight sources, 0.38 / 0.41 ms a level (forward /
+// transposed), 0.95 / 2.11 ms by two kernels over the nodes and 0.52 / 0.71 ms by
+// the sweep kernel before.
+//
+// FP64 fields take the sweep kernel (sweep_kernels.cu) instead of step_kernel;
+// lattices with fewer than 5 nodes on an axis and the all-FEM path one generic
+// kernel over every node.
 #define HYB_FIELD __restrict__
 #include "async_copy.cuh"
 #include "rows.cuh"
@@ -274,7 +281,7 @@ struct Producer {
 // one step inside a z face (dzs = -1 / +1: the low / high one) and the node
 // also produces the face node next to it.  Tiles without FACE hold no node
 // one step inside an x or y face.
-template <typename T, bool ADJ, bool FEMT, bool FACE, bool ZF, bool REF, bool TEL>
+template <typename T, bool ADJ, bool FEMT, bool FACE, bool ZF, bool REF, bool TEL, bool ANI>
 __device__ __forceinline__ void interior_node(const StepArgs<T>& A, const Slot<T>& S, T* __restrict__ gnext,
                                               const Col& C, int k, int off, int dzs, const T* Ck, const T* Cm,
                                               const T* Cp, const T* Pk, const T* Wk, const T* Wm, const T* Hk,
@@ -286,9 +293,10 @@ __device__ __forceinline__ void interior_node(const StepArgs<T>& A, const Slot<T
   const T c0 = Ck[0], cm = Cm[0], cp = Cp[0], pv = Pk[0];
   const T xm = Ck[-1], xp = Ck[1], ym = Ck[-kBoxX], yp = Ck[kBoxX];
   bool lf = false;
-  T wxm = T(1), wxp = T(1), wym = T(1), wyp = T(1);
+  const T k0 = ANI ? A.kapt[0] : T(1), k1 = ANI ? A.kapt[1] : T(1), k2 = ANI ? A.kapt[2] : T(1);
+  T wxm = k0, wxp = k0, wym = k1, wyp = k1;
   if constexpr (FEMT) lf = C.xy_fem && k >= A.fl[2] && k <= A.fh[2];
-  T wzm = T(1), wzp = T(1);
+  T wzm = k2, wzp = k2;
   T val;
   if (FEMT && lf) {
     wxm = Wk[-1];
@@ -303,6 +311,9 @@ __device__ __forceinline__ void interior_node(const StepArgs<T>& A, const Slot<T
       val = c0 + ((c0 - pv) * (T(1) - sd) + c2 * lap) / (T(1) + sd);
     else
       val = c0 + ((c0 - pv) + c2 * lap);
+  } else if constexpr (ANI) {
+    val = c0 + ((c0 - pv) + c2 * ((k0 * ((xm - c0) + (xp - c0)) + k1 * ((ym - c0) + (yp - c0))) +
+                                  k2 * ((cm - c0) + (cp - c0))));
   } else if constexpr (sizeof(T) == 4) {  // unit weights: the neighbour sum minus 6 u^k
     val = c0 + ((c0 - pv) + c2 * ((((xm + xp) + (ym + yp)) + (cm + cp)) - T(6) * c0));
   } else {  // FP64 sums the six differences
@@ -314,14 +325,15 @@ __device__ __forceinline__ void interior_node(const StepArgs<T>& A, const Slot<T
     const T ub = Cb[0];
     const bool abc = (S.mask_f >> f) & 1;
     const int offb = off + dzs * A.px * A.ny;
+    const T rf = ANI ? A.ra[2] : A.r;
     if constexpr (!ADJ) {
       T vb;
       if (abc) {
-        vb = A.r * ub + (c0 - A.r * val);
+        vb = rf * ub + (c0 - rf * val);
       } else {
-        T lb = T(2) * (c0 - ub);
-        lb += (Cb[-1] - ub) + (Cb[1] - ub);
-        lb += (Cb[-kBoxX] - ub) + (Cb[kBoxX] - ub);
+        T lb = T(2) * k2 * (c0 - ub);
+        lb += k0 * ((Cb[-1] - ub) + (Cb[1] - ub));
+        lb += k1 * ((Cb[-kBoxX] - ub) + (Cb[kBoxX] - ub));
         vb = ub + ((ub - S.prev[offb]) + c2 * lb);  // (u^{k-1} of the face plane is not staged)
         if ((S.src_mask >> f) & 1) vb += src_term(S, f, C.i, C.j, k + dzs);
         if (S.inj && S.obs_face == f) vb += S.inj_scale * T(2) * S.inj[face_index(f, C.i, C.j, k + dzs, A.nx, A.ny)];
@@ -330,16 +342,16 @@ __device__ __forceinline__ void interior_node(const StepArgs<T>& A, const Slot<T
       if (S.obs_w && S.obs_face == f) S.obs_w[face_index(f, C.i, C.j, k + dzs, A.nx, A.ny)] = vb;
     } else {
       const T coef_mb = dzs > 0 ? wzp : wzm;
-      T lb = abc ? A.r * ub : (T(2) - T(6) * c2) * ub;
+      T lb = abc ? rf * ub : (ANI ? T(2) + c2 * A.kdiag : T(2) - T(6) * c2) * ub;
       lb += c2 * coef_mb * c0;
       if (!abc) {
-        lb += c2 * (Cb[-1] + Cb[1]);
-        lb += c2 * (Cb[-kBoxX] + Cb[kBoxX]);
+        lb += c2 * k0 * (Cb[-1] + Cb[1]);
+        lb += c2 * k1 * (Cb[-kBoxX] + Cb[kBoxX]);
       }
       if (!((S.mask_c >> f) & 1)) lb -= S.prev[offb];
       if (S.obs_r && S.obs_face == f) lb += S.obs_r[face_index(f, C.i, C.j, k + dzs, A.nx, A.ny)];
-      val += (abc ? ub : T(2) * c2 * ub) - c2 * coef_mb * ub;
-      if ((S.mask_e >> f) & 1) val -= A.r * lb;
+      val += (abc ? ub : T(2) * c2 * k2 * ub) - c2 * coef_mb * ub;
+      if ((S.mask_e >> f) & 1) val -= rf * lb;
       gnext[offb] = lb;
     }
   }
@@ -354,6 +366,7 @@ __device__ __forceinline__ void interior_node(const StepArgs<T>& A, const Slot<T
       const bool abc = (S.mask_f >> f) & 1;
       const int offb = off + (ax == 0 ? sd : sd * A.px);
       const int bi = C.i + (ax == 0 ? sd : 0), bj = C.j + (ax == 1 ? sd : 0);
+      const T rf = ANI ? A.ra[ax] : A.r, kn = ax == 0 ? k0 : k1, kt = ax == 0 ? k1 : k0;  // across, along the face
       // Forward: the absorbing row of Eq. (eq:abs2) from u^k at b and m and
       // the new value at m, or the mirror-ghost row with the source flux.
       // Transposed: b's row in closed form (no transposed absorbing coupling
@@ -363,11 +376,11 @@ __device__ __forceinline__ void interior_node(const StepArgs<T>& A, const Slot<T
       if constexpr (!ADJ) {
         T vb;
         if (abc) {
-          vb = A.r * ub + (c0 - A.r * val);
+          vb = rf * ub + (c0 - rf * val);
         } else {
-          T lb = T(2) * (c0 - ub);
-          lb += (Ck[ob - o1] - ub) + (Ck[ob + o1] - ub);
-          lb += (Cm[ob] - ub) + (Cp[ob] - ub);
+          T lb = T(2) * kn * (c0 - ub);
+          lb += kt * ((Ck[ob - o1] - ub) + (Ck[ob + o1] - ub));
+          lb += k2 * ((Cm[ob] - ub) + (Cp[ob] - ub));
           vb = ub + ((ub - Pk[ob]) + c2 * lb);
           if ((S.src_mask >> f) & 1) vb += src_term(S, f, bi, bj, k);
           if (S.inj && S.obs_face == f) vb += S.inj_scale * T(2) * S.inj[face_index(f, bi, bj, k, A.nx, A.ny)];
@@ -376,16 +389,16 @@ __device__ __forceinline__ void interior_node(const StepArgs<T>& A, const Slot<T
         if (S.obs_w && S.obs_face == f) S.obs_w[face_index(f, bi, bj, k, A.nx, A.ny)] = vb;
       } else {
         const T coef_mb = ax == 0 ? (sd > 0 ? wxp : wxm) : (sd > 0 ? wyp : wym);
-        T lb = abc ? A.r * ub : (T(2) - T(6) * c2) * ub;
+        T lb = abc ? rf * ub : (ANI ? T(2) + c2 * A.kdiag : T(2) - T(6) * c2) * ub;
         lb += c2 * coef_mb * c0;
         if (!abc) {
-          lb += c2 * (Ck[ob - o1] + Ck[ob + o1]);
-          lb += c2 * (Cm[ob] + Cp[ob]);
+          lb += c2 * kt * (Ck[ob - o1] + Ck[ob + o1]);
+          lb += c2 * k2 * (Cm[ob] + Cp[ob]);
         }
         if (!((S.mask_c >> f) & 1)) lb -= Pk[ob];
         if (S.obs_r && S.obs_face == f) lb += S.obs_r[face_index(f, bi, bj, k, A.nx, A.ny)];
-        val += (abc ? ub : T(2) * c2 * ub) - c2 * coef_mb * ub;
-        if ((S.mask_e >> f) & 1) val -= A.r * lb;
+        val += (abc ? ub : T(2) * c2 * kn * ub) - c2 * coef_mb * ub;
+        if ((S.mask_e >> f) & 1) val -= rf * lb;
         gnext[offb] = lb;
       }
     }
@@ -406,7 +419,7 @@ __device__ __forceinline__ void interior_node(const StepArgs<T>& A, const Slot<T
     if (C.xy_vox && k < A.fl[2] + A.un[2] && !(REF && (rf & 2))) {
       const T u[8] = {Hk[0], Hk[1], Hk[kBoxX], Hk[kBoxX + 1], Hp[0], Hp[1], Hp[kBoxX], Hp[kBoxX + 1]};
       const T l[8] = {c0, xp, yp, Ck[kBoxX + 1], cp, Cp[1], Cp[kBoxX], Cp[kBoxX + 1]};
-      atomicAdd(A.G + (long long)C.si * ((long long)vz * A.un[2]) + vid, (double)(TEL ? damp_sum(u, l) : pair_sum(u, l)));
+      atomicAdd(A.G + (long long)C.si * ((long long)vz * A.un[2]) + vid, (double)(TEL ? damp_sum(u, l) : (ANI ? pair_sum_ani(A, u, l) : pair_sum(u, l))));
     }
   }
 }
@@ -424,7 +437,7 @@ struct XFace {
 };
 constexpr unsigned kFaceLanes = 0x1fffeu;  // lanes 1 .. 16 of the producer warp
 
-template <typename T, bool ADJ, bool DEEP>
+template <typename T, bool ADJ, bool DEEP, bool ANI>
 __device__ __forceinline__ void xface_levels(const StepArgs<T>& A, const Slot<T>& S, const Producer<T, DEEP>& pr,
                                              const XFace& X, int z0, int z1, long long budget) {
   using P = kPipe<T>;
@@ -436,7 +449,8 @@ __device__ __forceinline__ void xface_levels(const StepArgs<T>& A, const Slot<T>
   const int sd = X.sd;
   constexpr int kBoxX = Box<T>::BX;
   const int o = (r + 1) * kBoxX + (X.mi - X.i0 + Box<T>::hx);  // m in a u box
-  const T c2 = A.c2;
+  const T c2 = A.c2, rf = ANI ? A.ra[0] : A.r;
+  const T k0 = ANI ? A.kapt[0] : T(1), k1 = ANI ? A.kapt[1] : T(1), k2 = ANI ? A.kapt[2] : T(1);
   const bool abc = (S.mask_f >> f) & 1;
   T* __restrict__ gnext = S.next;
   const int pl = A.px * A.ny;
@@ -456,7 +470,10 @@ __device__ __forceinline__ void xface_levels(const StepArgs<T>& A, const Slot<T>
       const T c0 = Ck[0], xm = Ck[-1], xp = Ck[1], ym = Ck[-kBoxX], yp = Ck[kBoxX];
       const T cm = Cm[0], cp = Cp[0], pv = Pk[0];
       T val;
-      if constexpr (sizeof(T) == 4)
+      if constexpr (ANI)
+        val = c0 + ((c0 - pv) + c2 * ((k0 * ((xm - c0) + (xp - c0)) + k1 * ((ym - c0) + (yp - c0))) +
+                                      k2 * ((cm - c0) + (cp - c0))));
+      else if constexpr (sizeof(T) == 4)
         val = c0 + ((c0 - pv) + c2 * ((((xm + xp) + (ym + yp)) + (cm + cp)) - T(6) * c0));
       else
         val = c0 + ((c0 - pv) + c2 * lap7(xm, xp, ym, yp, cm, cp, c0));
@@ -465,11 +482,11 @@ __device__ __forceinline__ void xface_levels(const StepArgs<T>& A, const Slot<T>
       if constexpr (!ADJ) {
         T vb;
         if (abc) {
-          vb = A.r * ub + (c0 - A.r * val);
+          vb = rf * ub + (c0 - rf * val);
         } else {
-          T lb = T(2) * (c0 - ub);
-          lb += (Ck[sd - kBoxX] - ub) + (Ck[sd + kBoxX] - ub);
-          lb += (Cm[sd] - ub) + (Cp[sd] - ub);
+          T lb = T(2) * k0 * (c0 - ub);
+          lb += k1 * ((Ck[sd - kBoxX] - ub) + (Ck[sd + kBoxX] - ub));
+          lb += k2 * ((Cm[sd] - ub) + (Cp[sd] - ub));
           vb = ub + ((ub - Pk[sd]) + c2 * lb);
           if ((S.src_mask >> f) & 1) vb += src_term(S, f, X.mi + sd, j, k);
           if (S.inj && S.obs_face == f) vb += S.inj_scale * T(2) * S.inj[face_index(f, X.mi + sd, j, k, A.nx, A.ny)];
@@ -477,16 +494,16 @@ __device__ __forceinline__ void xface_levels(const StepArgs<T>& A, const Slot<T>
         gnext[offb] = vb;
         if (S.obs_w && S.obs_face == f) S.obs_w[face_index(f, X.mi + sd, j, k, A.nx, A.ny)] = vb;
       } else {
-        T lb = abc ? A.r * ub : (T(2) - T(6) * c2) * ub;
-        lb += c2 * c0;
+        T lb = abc ? rf * ub : (ANI ? T(2) + c2 * A.kdiag : T(2) - T(6) * c2) * ub;
+        lb += c2 * k0 * c0;
         if (!abc) {
-          lb += c2 * (Ck[sd - kBoxX] + Ck[sd + kBoxX]);
-          lb += c2 * (Cm[sd] + Cp[sd]);
+          lb += c2 * k1 * (Ck[sd - kBoxX] + Ck[sd + kBoxX]);
+          lb += c2 * k2 * (Cm[sd] + Cp[sd]);
         }
         if (!((S.mask_c >> f) & 1)) lb -= Pk[sd];
         if (S.obs_r && S.obs_face == f) lb += S.obs_r[face_index(f, X.mi + sd, j, k, A.nx, A.ny)];
-        val += (abc ? ub : T(2) * c2 * ub) - c2 * ub;
-        if ((S.mask_e >> f) & 1) val -= A.r * lb;
+        val += (abc ? ub : T(2) * c2 * k0 * ub) - c2 * k0 * ub;
+        if ((S.mask_e >> f) & 1) val -= rf * lb;
         gnext[offb] = lb;
       }
       gnext[off] = val;
@@ -499,7 +516,7 @@ __device__ __forceinline__ void xface_levels(const StepArgs<T>& A, const Slot<T>
 // Consumer loop of an interior block, specialised by whether the tile meets
 // the FEM block (FEMT) and whether it holds nodes one step inside an x or y
 // face (FACE).  Each consumer thread owns two tile rows (ty and ty + 8).
-template <typename T, bool ADJ, bool FEMT, bool FACE, bool REF, bool TEL = false>
+template <typename T, bool ADJ, bool FEMT, bool FACE, bool REF, bool TEL, bool ANI>
 __device__ __forceinline__ void interior_levels(const StepArgs<T>& A, const Slot<T>& S, const Col (&C)[2],
                                                 const Producer<T, !FEMT>& pr, const bool (&active)[2],
                                                 const XFace& X, int z0, int z1) {
@@ -514,7 +531,7 @@ __device__ __forceinline__ void interior_levels(const StepArgs<T>& A, const Slot
     // at level g - D - 1 (the edge-weight and stored-u rings are the
     // shortest), so they are issued once every consumer warp is done with it.
     if (t != kProd) {
-      if (FACE && X.on && t <= kProd + 16) xface_levels<T, ADJ, !FEMT>(A, S, pr, X, z0, z1, budget);
+      if (FACE && X.on && t <= kProd + 16) xface_levels<T, ADJ, !FEMT, ANI>(A, S, pr, X, z0, z1, budget);
       return;
     }
     for (int g = 0; g < D && z0 + g < z1; ++g) pr.issue(z0 + g, g == 0);
@@ -624,17 +641,17 @@ __device__ __forceinline__ void interior_levels(const StepArgs<T>& A, const Slot
     const int dzs = k == 1 ? -1 : (k == nz - 2 ? 1 : 0);
     if (dzs != 0) {
       if (act0)
-        interior_node<T, ADJ, FEMT, FACE, true, REF, TEL>(A, S, gnext, C[0], k, off0, dzs, Ck + o0, Cm + o0, Cp + o0,
+        interior_node<T, ADJ, FEMT, FACE, true, REF, TEL, ANI>(A, S, gnext, C[0], k, off0, dzs, Ck + o0, Cm + o0, Cp + o0,
                                                 Pk + p0, Wk + o0, Wm + o0, Hk + h0, Hp + h0, rf0, sd0);
       if (act1)
-        interior_node<T, ADJ, FEMT, FACE, true, REF, TEL>(A, S, gnext, C[1], k, off1, dzs, Ck + o1, Cm + o1, Cp + o1,
+        interior_node<T, ADJ, FEMT, FACE, true, REF, TEL, ANI>(A, S, gnext, C[1], k, off1, dzs, Ck + o1, Cm + o1, Cp + o1,
                                                 Pk + p1, Wk + o1, Wm + o1, Hk + h1, Hp + h1, rf1, sd1);
     } else {
       if (act0)
-        interior_node<T, ADJ, FEMT, FACE, false, REF, TEL>(A, S, gnext, C[0], k, off0, 0, Ck + o0, Cm + o0, Cp + o0,
+        interior_node<T, ADJ, FEMT, FACE, false, REF, TEL, ANI>(A, S, gnext, C[0], k, off0, 0, Ck + o0, Cm + o0, Cp + o0,
                                                  Pk + p0, Wk + o0, Wm + o0, Hk + h0, Hp + h0, rf0, sd0);
       if (act1)
-        interior_node<T, ADJ, FEMT, FACE, false, REF, TEL>(A, S, gnext, C[1], k, off1, 0, Ck + o1, Cm + o1, Cp + o1,
+        interior_node<T, ADJ, FEMT, FACE, false, REF, TEL, ANI>(A, S, gnext, C[1], k, off1, 0, Ck + o1, Cm + o1, Cp + o1,
                                                  Pk + p1, Wk + o1, Wm + o1, Hk + h1, Hp + h1, rf1, sd1);
     }
     __syncwarp();  // the warp's reads of level k's stages are done
@@ -656,7 +673,7 @@ __device__ __forceinline__ void interior_levels(const StepArgs<T>& A, const Slot
 // (slot, tile, z range; the host balances the items by cost): eight
 // consumer warps (two tile rows per thread) and a producer warp.  Nodes one
 // step inside a face also produce the face node next to them.
-template <typename T, bool ADJ, bool TEL>
+template <typename T, bool ADJ, bool TEL, bool ANI>
 __device__ __forceinline__ void interior_block(const StepArgs<T>& A, int b, T* sm) {
   static_assert(kTileX == 32, "one warp per tile row");
   static_assert(kTileX * kTileY / 2 + 32 == kStepBlock, "eight consumer warps (two rows each) and a producer warp");
@@ -739,27 +756,27 @@ __device__ __forceinline__ void interior_block(const StepArgs<T>& A, int b, T* s
     pr.setup(A, S, sm, full, z0, z1, i0, j0, pairing, face_tile);
     if constexpr (TEL) {  // telegraph reading (no refinement)
       if (face_tile)
-        interior_levels<T, ADJ, true, true, false, true>(A, S, C, pr, active, X, z0, z1);
+        interior_levels<T, ADJ, true, true, false, true, false>(A, S, C, pr, active, X, z0, z1);
       else
-        interior_levels<T, ADJ, true, false, false, true>(A, S, C, pr, active, X, z0, z1);
-    } else if (ref_tile) {
+        interior_levels<T, ADJ, true, false, false, true, false>(A, S, C, pr, active, X, z0, z1);
+    } else if (!ANI && ref_tile) {  // (no refinement with per-axis steps)
       if (face_tile)
-        interior_levels<T, ADJ, true, true, true>(A, S, C, pr, active, X, z0, z1);
+        interior_levels<T, ADJ, true, true, !ANI, false, ANI>(A, S, C, pr, active, X, z0, z1);
       else
-        interior_levels<T, ADJ, true, false, true>(A, S, C, pr, active, X, z0, z1);
+        interior_levels<T, ADJ, true, false, !ANI, false, ANI>(A, S, C, pr, active, X, z0, z1);
     } else {
       if (face_tile)
-        interior_levels<T, ADJ, true, true, false>(A, S, C, pr, active, X, z0, z1);
+        interior_levels<T, ADJ, true, true, false, false, ANI>(A, S, C, pr, active, X, z0, z1);
       else
-        interior_levels<T, ADJ, true, false, false>(A, S, C, pr, active, X, z0, z1);
+        interior_levels<T, ADJ, true, false, false, false, ANI>(A, S, C, pr, active, X, z0, z1);
     }
   } else {
     Producer<T, true> pr;
     pr.setup(A, S, sm, full, z0, z1, i0, j0, false, face_tile);
     if (face_tile)
-      interior_levels<T, ADJ, false, true, false>(A, S, C, pr, active, X, z0, z1);
+      interior_levels<T, ADJ, false, true, false, false, ANI>(A, S, C, pr, active, X, z0, z1);
     else
-      interior_levels<T, ADJ, false, false, false>(A, S, C, pr, active, X, z0, z1);
+      interior_levels<T, ADJ, false, false, false, false, ANI>(A, S, C, pr, active, X, z0, z1);
   }
 }
 
@@ -768,7 +785,7 @@ __device__ __forceinline__ void interior_block(const StepArgs<T>& A, int b, T* s
 // nodes; an absorbing row (Eq. (eq:abs2)) reads the new values of its
 // inward neighbours, one level down in the same tile, from shared memory.
 // Every thread of the block calls it (it synchronises); nv holds 128 values.
-template <typename T>
+template <typename T, bool ANI>
 __device__ __forceinline__ void fwd_edge_tile(const StepArgs<T>& A, int si, int blk, int t, T* nv) {
   const Slot<T>& S = A.s[si];
   int i = 0, j = 0, k = 0, nf = -1, q[3];
@@ -787,7 +804,7 @@ __device__ __forceinline__ void fwd_edge_tile(const StepArgs<T>& A, int si, int 
   }
   T plain = T(0);  // the non-absorbing row, from level-k data only
   if (valid && !fb) {
-    plain = cself + ((cself - S.prev[id]) + A.c2 * row_lap_inl<T, false>(A, S.W, S.cur, i, j, k));
+    plain = cself + ((cself - S.prev[id]) + A.c2 * row_lap_inl<T, ANI>(A, S.W, S.cur, i, j, k));
     if (fall & S.src_mask) plain += src_terms(S, fall, i, j, k);
     if (S.inj) plain += inj_term(S, fall, i, j, k, A.nx, A.ny);
   }
@@ -803,9 +820,9 @@ __device__ __forceinline__ void fwd_edge_tile(const StepArgs<T>& A, int si, int 
         const int fa = (fb >> (2 * ax)) & 3;
         if (!fa) continue;
         const int t1 = edge_tile_peer(t, blk, q, ax, (fa & 1) ? 1 : 2);
-        acc += cin[ax] - A.r * nv[t1];
+        acc += cin[ax] - (ANI ? A.ra[ax] : A.r) * nv[t1];
       }
-      v = A.r * cself + acc / T(__popc(fb));
+      v = (ANI ? abc_self(A, fb) : A.r) * cself + acc / T(__popc(fb));
     }
     __syncthreads();
     if (mine) nv[t] = v;
@@ -821,12 +838,12 @@ __device__ __forceinline__ void fwd_edge_tile(const StepArgs<T>& A, int si, int 
 // Edge tile of the transposed step: every thread gathers its transposed row
 // in parallel, then the transposed absorbing couplings (E^T) are resolved
 // from the nodes on the most faces inwards, through shared memory.
-template <typename T>
+template <typename T, bool ANI>
 __device__ __forceinline__ void adj_edge_tile(const StepArgs<T>& A, int si, int blk, int t, T* lam) {
   const Slot<T>& S = A.s[si];
   int i = 0, j = 0, k = 0, nf = -1, q[3];
   const bool valid = blk < A.nedge && edge_tile_node(A, blk, t, i, j, k, q, nf);
-  lam[t] = valid ? adj_rhs_inl<T, false>(A, S, i, j, k) : T(0);
+  lam[t] = valid ? adj_rhs_inl<T, ANI>(A, S, i, j, k) : T(0);
   __syncthreads();
   for (int level = 2; level >= 0; --level) {
     T v = T(0);
@@ -841,7 +858,7 @@ __device__ __forceinline__ void adj_edge_tile(const StepArgs<T>& A, int si, int 
         const int f = 2 * ax + (s > 0 ? 1 : 0);
         const int fbb = face_bits(bi, bj, bk, A.nx, A.ny, A.nz) & S.mask_e;
         if (!(fbb & (1 << f))) continue;
-        v -= (A.r / T(__popc(fbb))) * lam[edge_tile_peer(t, blk, q, ax, q[ax] == 1 ? 0 : 3)];
+        v -= ((ANI ? A.ra[ax] : A.r) / T(__popc(fbb))) * lam[edge_tile_peer(t, blk, q, ax, q[ax] == 1 ? 0 : 3)];
       }
     }
     __syncthreads();
@@ -850,7 +867,7 @@ __device__ __forceinline__ void adj_edge_tile(const StepArgs<T>& A, int si, int 
   }
   if (!valid) return;
   S.next[lin(A, i, j, k)] = lam[t];
-  pair_if_voxel<T, false>(A, S, si, i, j, k);
+  pair_if_voxel<T, ANI>(A, S, si, i, j, k);
 }
 
 template <typename T, bool ADJ>
@@ -862,7 +879,7 @@ __device__ __forceinline__ void refined_rows(const StepArgs<T>& A, long long t);
 // the refined region (gathers of short latency-bound rows, which fill the
 // slots the interior blocks free towards the end of the level).  All blocks
 // read levels k, k-1 and write disjoint nodes of level k+1.
-template <typename T, bool ADJ, bool TEL>
+template <typename T, bool ADJ, bool TEL, bool ANI>
 __global__ void __launch_bounds__(kStepBlock, sizeof(T) == 4 ? 4 : 2) step_kernel(const __grid_constant__ StepArgs<T> A) {
   extern __shared__ __align__(128) unsigned char hyb_smem[];  // kPipe<T>::bytes
   T* sh = reinterpret_cast<T*>(hyb_smem);
@@ -876,18 +893,18 @@ __global__ void __launch_bounds__(kStepBlock, sizeof(T) == 4 ? 4 : 2) step_kerne
     const int blk = half < 2 ? 2 * (b - si * ne2) + half : A.nedge;
     const int t = (int)(threadIdx.x & 127);
     if constexpr (ADJ)
-      adj_edge_tile<T>(A, si, blk, t, sh + 128 * half);
+      adj_edge_tile<T, ANI>(A, si, blk, t, sh + 128 * half);
     else
-      fwd_edge_tile<T>(A, si, blk, t, sh + 128 * half);
+      fwd_edge_tile<T, ANI>(A, si, blk, t, sh + 128 * half);
     return;
   }
   b -= A.nhe;
   if (b >= A.nitems) {
     pdl_wait();
-    refined_rows<T, ADJ>(A, (long long)(b - A.nitems) * kStepBlock + threadIdx.x);
+    if constexpr (!ANI) refined_rows<T, ADJ>(A, (long long)(b - A.nitems) * kStepBlock + threadIdx.x);
     return;
   }
-  interior_block<T, ADJ, TEL>(A, b, sh);
+  interior_block<T, ADJ, TEL, ANI>(A, b, sh);
 }
 
 // Lattices with fewer than 5 nodes on some axis: every node by the generic
@@ -1120,10 +1137,12 @@ void launch_step(const StepArgs<T>& a, cudaStream_t st) {
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  if (a.sdamp)
-    cudaLaunchKernelEx(&cfg, step_kernel<T, ADJ, true>, b);
+  if (a.ani)
+    cudaLaunchKernelEx(&cfg, step_kernel<T, ADJ, false, true>, b);
+  else if (a.sdamp)
+    cudaLaunchKernelEx(&cfg, step_kernel<T, ADJ, true, false>, b);
   else
-    cudaLaunchKernelEx(&cfg, step_kernel<T, ADJ, false>, b);
+    cudaLaunchKernelEx(&cfg, step_kernel<T, ADJ, false, false>, b);
 }
 
 void launch_tile_step(const StepArgs<float>& a, bool adjoint, cudaStream_t st) {
@@ -1134,15 +1153,13 @@ void launch_tile_step(const StepArgs<float>& a, bool adjoint, cudaStream_t st) {
 template <typename T, bool ADJ>
 int step_occupancy() {
   int n = 0;
-  if (cudaFuncSetAttribute(step_kernel<T, ADJ, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)kPipe<T>::bytes) != cudaSuccess ||
-      cudaFuncSetAttribute(step_kernel<T, ADJ, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)kPipe<T>::bytes) != cudaSuccess ||
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, step_kernel<T, ADJ, false>, kStepBlock, kPipe<T>::bytes) !=
-          cudaSuccess) {
-    cudaGetLastError();
-    return 1;
-  }
+  for (auto kernel : {step_kernel<T, ADJ, true, false>, step_kernel<T, ADJ, false, true>, step_kernel<T, ADJ, false, false>})
+    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPipe<T>::bytes) !=
+            cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kernel, kStepBlock, kPipe<T>::bytes) != cudaSuccess) {
+      cudaGetLastError();
+      return 1;
+    }
   return n > 0 ? n : 1;
 }
 

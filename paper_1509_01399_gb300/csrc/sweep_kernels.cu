@@ -1,6 +1,6 @@
 // The sweep kernel: a run of consecutive time levels of every slot in one
-// launch, for FP64 fields and for per-axis steps (FP32 fields with equal steps
-// take the staged tiles of step_kernels.cu).
+// launch, for FP64 fields (FP32 fields take the staged tiles of
+// step_kernels.cu).
 //
 // Blocks claim work items (level, slot, item) in order and an item waits only
 // for the previous level's items around it.  Items are runs of interior rows
@@ -170,22 +170,15 @@ __device__ __forceinline__ void adj_edge_tile(const SweepArgs<T>& A, const Slot<
   if (valid) S.next[lin(A, i, j, k)] = lam[t];
 }
 
-// 16-byte groups of consecutive nodes along x ("quads": four FP32 or two
-// FP64 values; rows start on 32-byte boundaries, so quads are aligned).
+// 16-byte groups of consecutive nodes along x ("quads"; rows start on 32-byte
+// boundaries, so quads are aligned).
 template <typename T>
 struct Quad {
   static constexpr int V = 16 / (int)sizeof(T);
 };
-__device__ __forceinline__ void ldq(float (&v)[4], const float* p) {
-  const float4 f = *reinterpret_cast<const float4*>(p);
-  v[0] = f.x, v[1] = f.y, v[2] = f.z, v[3] = f.w;
-}
 __device__ __forceinline__ void ldq(double (&v)[2], const double* p) {
   const double2 f = *reinterpret_cast<const double2*>(p);
   v[0] = f.x, v[1] = f.y;
-}
-__device__ __forceinline__ void stq(float* p, const float (&v)[4]) {
-  *reinterpret_cast<float4*>(p) = make_float4(v[0], v[1], v[2], v[3]);
 }
 __device__ __forceinline__ void stq(double* p, const double (&v)[2]) {
   *reinterpret_cast<double2*>(p) = make_double2(v[0], v[1]);
@@ -223,42 +216,6 @@ __device__ __forceinline__ T ani_row(const SweepArgs<T>& A, T c, T xm, T xp, T y
   }
 }
 
-// The same for a quad of FP32 nodes, in packed pairs.
-template <bool ADJ>
-__device__ __forceinline__ void ani_rows(const SweepArgs<float>& A, float (&val)[4], const float (&c)[4], float xl,
-                                         float xr, const float (&ym)[4], const float (&yp)[4], const float (&zm)[4],
-                                         const float (&zp)[4], const float (&pv)[4]) {
-  const float xm[4] = {xl, c[0], c[1], c[2]}, xp[4] = {c[1], c[2], c[3], xr};
-  auto two = [](const float (&v)[4], int h) { return make_float2(v[2 * h], v[2 * h + 1]); };
-  auto both = [](float v) { return make_float2(v, v); };
-  const float2 m1 = both(-1.f);
-#pragma unroll
-  for (int h = 0; h < 2; ++h) {
-    const float2 C = two(c, h), P = two(pv, h);
-    float2 v;
-    if constexpr (ADJ) {
-      const float2 cx = both(A.c2 * A.kapt[0]), cy = both(A.c2 * A.kapt[1]), cz = both(A.c2 * A.kapt[2]);
-      v = __fmul2_rn(both(2.f + A.c2 * A.kdiag), C);
-      v = __ffma2_rn(cx, two(xm, h), v);
-      v = __ffma2_rn(cx, two(xp, h), v);
-      v = __ffma2_rn(cy, two(ym, h), v);
-      v = __ffma2_rn(cy, two(yp, h), v);
-      v = __ffma2_rn(cz, two(zm, h), v);
-      v = __ffma2_rn(cz, two(zp, h), v);
-      v = __ffma2_rn(P, m1, v);
-    } else {
-      const float2 lx = __fadd2_rn(__ffma2_rn(C, m1, two(xm, h)), __ffma2_rn(C, m1, two(xp, h)));
-      const float2 ly = __fadd2_rn(__ffma2_rn(C, m1, two(ym, h)), __ffma2_rn(C, m1, two(yp, h)));
-      const float2 lz = __fadd2_rn(__ffma2_rn(C, m1, two(zm, h)), __ffma2_rn(C, m1, two(zp, h)));
-      const float2 lap = __ffma2_rn(both(A.kapt[2]), lz,
-                                    __ffma2_rn(both(A.kapt[0]), lx, __fmul2_rn(both(A.kapt[1]), ly)));
-      v = __fadd2_rn(C, __ffma2_rn(both(A.c2), lap, __ffma2_rn(P, m1, C)));
-    }
-    val[2 * h] = v.x;
-    val[2 * h + 1] = v.y;
-  }
-}
-
 // A row with edge weights (FEM-owned node) from the differences u_nb - u^k.
 template <typename T, bool TEL>
 __device__ __forceinline__ T fem_diff_row(T c, T dxm, T dxp, T dym, T dyp, T dzm, T dzp, T pv, T wxm, T wxp, T wym,
@@ -289,13 +246,13 @@ __device__ __forceinline__ T fem_row(const SweepArgs<T>& A, T c, T xm, T xp, T y
 
 // Faces whose rows the interior items take along: absorbing in this step (and,
 // transposed, in the next one: then nothing but values at hand enters).  The
-// other faces' nodes and their neighbours are left to the face items: with FP64
-// fields the x faces among them, whose few lanes would cost every warp of a row
-// a pass of the FP64 pipe.
+// other faces' nodes and their neighbours are left to the face items, the x
+// faces among them, whose few lanes would cost every warp of a row a pass of
+// the FP64 pipe.
 template <typename T, StepMode M>
 __device__ __forceinline__ int inline_faces(const Slot<T>& S) {
   const int f = M == kAdjoint ? (S.mask_f & S.mask_c) : (M == kForward ? S.mask_f : 0);
-  return sizeof(T) == 4 ? f : f & ~3;
+  return f & ~3;
 }
 
 // Stage and phase of the ring position a side of the pipeline is at.
@@ -403,7 +360,7 @@ __device__ __forceinline__ void interior_march(const SweepArgs<T>& A, const Slot
                                                RingPos& rp, int si, const InteriorRun<T>& R) {
   constexpr int V = Quad<T>::V;
   constexpr bool ADJ = M == kAdjoint, PAIR = FEM && M != kForward;
-  constexpr bool DIF = V == 2 && !ANI;  // rows from differences: zm carries u - (u below)
+  constexpr bool DIF = !ANI;  // rows from differences: zm carries u - (u below)
   constexpr unsigned kAll = (1u << V) - 1;
   const bool valid = (int)threadIdx.x < R.n;
   const int t = R.first + (valid ? (int)threadIdx.x : R.n - 1);
@@ -482,10 +439,7 @@ __device__ __forceinline__ void interior_march(const SweepArgs<T>& A, const Slot
         ldq(wz0, W + 2 * A.wsz - wz);
         h = hidx(A, i0, j, k);
         if constexpr (TEL) ldq(sd, A.sdamp + h);
-        if (A.nref) {
-          if constexpr (V == 4) rf = *reinterpret_cast<const unsigned*>(A.rmask + h);
-          else rf = *reinterpret_cast<const unsigned short*>(A.rmask + h);
-        }
+        if (A.nref) rf = *reinterpret_cast<const unsigned short*>(A.rmask + h);
         if constexpr (PAIR) {
           pairq = S.hist_r && j - A.fl[1] < A.un[1] && k - A.fl[2] < A.un[2];
           if (pairq) {
@@ -543,15 +497,10 @@ __device__ __forceinline__ void interior_march(const SweepArgs<T>& A, const Slot
 #pragma unroll
       for (int e = 0; e < V; ++e) zm[e] = dzp[e];
     } else {
-      static_assert(ANI, "FP32 fields with equal steps take the tile kernel");
-      if constexpr (V == 4) {
-        ani_rows<ADJ>(A, val, c, xl, xr, ym, yp, zm, zp, pv);
-      } else {
 #pragma unroll
-        for (int e = 0; e < V; ++e)
-          val[e] = ani_row<T, ADJ>(A, c[e], e ? c[e - 1] : xl, e < V - 1 ? c[e + 1] : xr, ym[e], yp[e], zm[e], zp[e],
-                                   pv[e]);
-      }
+      for (int e = 0; e < V; ++e)
+        val[e] = ani_row<T, ADJ>(A, c[e], e ? c[e - 1] : xl, e < V - 1 ? c[e + 1] : xr, ym[e], yp[e], zm[e], zp[e],
+                                 pv[e]);
       if (FEM && fm) {
 #pragma unroll
         for (int e = 0; e < V; ++e) {
@@ -741,8 +690,7 @@ __device__ __forceinline__ void face_pair(const SweepArgs<T>& A, const Slot<T>& 
   } else if constexpr (ANI) {
     val = ani_row<T, ADJ>(A, c0, xm, xp, ym, yp, zm, zp, pv);
   } else {
-    const T lap = sizeof(T) == 4 ? (((xm + xp) + (ym + yp)) + (zm + zp)) - T(6) * c0
-                                 : (((xp - c0) - (c0 - xm)) + ((yp - c0) - (c0 - ym))) + ((zp - c0) - (c0 - zm));
+    const T lap = (((xp - c0) - (c0 - xm)) + ((yp - c0) - (c0 - ym))) + ((zp - c0) - (c0 - zm));
     val = c0 + ((c0 - pv) + A.c2 * lap);
   }
   const int bi = i + (ax == 0 ? sd : 0), bj = j + (ax == 1 ? sd : 0), bk = k + (ax == 2 ? sd : 0);
@@ -934,9 +882,7 @@ struct QItem {
 // 0.238 / 0.296 ms a forward / transposed level by a launch of staged tiles per
 // level, 0.132 / 0.190 ms here (the pipe's floor for the forward rows: 0.093).
 // Small lattices: the launches and their dependent chain, 33^3 9.0 / 16.7 us a
-// level then, 6.1 / 10.7 us here.  Per-axis steps in FP32: 257 x 193 x 321, eight
-// sources, 0.95 / 2.11 ms a level by a bulk and a face-shell launch per level
-// (instruction issue), 0.50 / 0.60 ms here (DRAM floor 0.23 / 0.24).
+// level then, 6.1 / 10.7 us here.
 // Two blocks of 7 row warps and a producer warp per SM leave a thread 128
 // registers, which the transposed rows with their pairing need (with three
 // blocks they spill: autograd's 97^3 FP64 49 us a transposed level against 44).
@@ -1110,23 +1056,18 @@ void launch_sweep_mode(const SweepArgs<T>& a, int block, int grid, int smem, cud
       sweep_kernel<T, M, false, true><<<grid, block + kServiceThreads, smem, st>>>(a);
       return;
     }
-  }
-  if constexpr (sizeof(T) == 8) {
-    if constexpr (M != kPaper) {
-      if (a.sdamp) {
-        sweep_kernel<T, M, true, false><<<grid, block + kServiceThreads, smem, st>>>(a);
-        return;
-      }
+    if (a.sdamp) {
+      sweep_kernel<T, M, true, false><<<grid, block + kServiceThreads, smem, st>>>(a);
+      return;
     }
-    sweep_kernel<T, M, false, false><<<grid, block + kServiceThreads, smem, st>>>(a);
   }
+  sweep_kernel<T, M, false, false><<<grid, block + kServiceThreads, smem, st>>>(a);
 }
 
-template <typename T>
-int launch_sweep(const SweepArgs<T>& a, StepMode mode, int block, int grid, int smem, cudaStream_t st) {
-  if (mode == kForward) launch_sweep_mode<T, kForward>(a, block, grid, smem, st);
-  else if (mode == kAdjoint) launch_sweep_mode<T, kAdjoint>(a, block, grid, smem, st);
-  else launch_sweep_mode<T, kPaper>(a, block, grid, smem, st);
+int launch_sweep(const SweepArgs<double>& a, StepMode mode, int block, int grid, int smem, cudaStream_t st) {
+  if (mode == kForward) launch_sweep_mode<double, kForward>(a, block, grid, smem, st);
+  else if (mode == kAdjoint) launch_sweep_mode<double, kAdjoint>(a, block, grid, smem, st);
+  else launch_sweep_mode<double, kPaper>(a, block, grid, smem, st);
   return 2;
 }
 
@@ -1143,26 +1084,16 @@ int variant_occupancy(int block, int smem) {
   return n;
 }
 
-template <typename T>
-int sweep_occupancy(int block, int smem) {
-  int n = variant_occupancy<T, kForward, false, true>(block, smem);
+int sweep_blocks_per_sm(int block, int smem) {
+  int n = variant_occupancy<double, kForward, false, false>(block, smem);
   auto least = [&n](int q) { n = q < n ? q : n; };
-  least(variant_occupancy<T, kAdjoint, false, true>(block, smem));
-  if constexpr (sizeof(T) == 8) {
-    least(variant_occupancy<T, kForward, false, false>(block, smem));
-    least(variant_occupancy<T, kAdjoint, false, false>(block, smem));
-    least(variant_occupancy<T, kPaper, false, false>(block, smem));
-    least(variant_occupancy<T, kForward, true, false>(block, smem));
-    least(variant_occupancy<T, kAdjoint, true, false>(block, smem));
-  }
+  least(variant_occupancy<double, kAdjoint, false, false>(block, smem));
+  least(variant_occupancy<double, kPaper, false, false>(block, smem));
+  least(variant_occupancy<double, kForward, true, false>(block, smem));
+  least(variant_occupancy<double, kAdjoint, true, false>(block, smem));
+  least(variant_occupancy<double, kForward, false, true>(block, smem));
+  least(variant_occupancy<double, kAdjoint, false, true>(block, smem));
   return n > 0 ? n : 1;
 }
-
-int sweep_blocks_per_sm(int precision, int block, int smem) {
-  return precision == HYB_FP32 ? sweep_occupancy<float>(block, smem) : sweep_occupancy<double>(block, smem);
-}
-
-template int launch_sweep<float>(const SweepArgs<float>&, StepMode, int, int, int, cudaStream_t);
-template int launch_sweep<double>(const SweepArgs<double>&, StepMode, int, int, int, cudaStream_t);
 
 }  // namespace hyb

@@ -1,4 +1,5 @@
-"""The sweep kernel (FP64 fields, per-axis steps) where its pieces meet:
+"""The sweep kernel (FP64 fields) and the tile kernel with per-axis steps (FP32)
+where their pieces meet:
 lattices down to 5 nodes, x extents at every remainder of the 16-byte groups,
 rows longer than an item's run (staged in three pieces), items that end inside
 a row, slabs of several planes and several launches' worth of levels, with FEM
