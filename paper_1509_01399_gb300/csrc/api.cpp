@@ -74,7 +74,8 @@ struct SweepGraph {
 
 // Work items of one level (sweep kernel) for a slot count.
 struct SweepPlan {
-  DevBuf items, need, rslab, sync;
+  DevBuf buf;                          // items, rslab, need, sync (element offsets below)
+  size_t rslab = 0, need = 0, sync = 0;
   int nitems = 0, nslab = 0, slabz = 0, block = 0, grid = 0;
   int ns = 0, smem = 0, split = 0, ccen = 0, yo = 0, ncur = 0, nstage = 0;  // ring (StepArgs)
 };
@@ -902,14 +903,19 @@ hyb_status build_plan(hyb_mesh* m, int nslots) {
     }
     for (long long f = 0; f < nq; f += block) add(0, s, f, nq, 0);
   }
-  HYB_TRY(upload(m, P.items, items));
-  HYB_TRY(upload(m, P.need, need));
-  HYB_TRY(upload(m, P.rslab, rslab));
-  HYB_TRY(upload(m, P.sync, std::vector<unsigned>(2 + (size_t)nslots * nslab, 0u)));
+  // one buffer, one copy (allocations and copies are most of what a plan costs)
+  const size_t nitems = items.size() / 4;
+  P.rslab = items.size();
+  items.insert(items.end(), rslab.begin(), rslab.end());
+  P.need = items.size();
+  items.insert(items.end(), need.begin(), need.end());
+  P.sync = (items.size() + 63) & ~(size_t)63;  // (counters on lines of their own)
+  items.resize(P.sync + 2 + (size_t)nslots * nslab, 0);
+  HYB_TRY(upload(m, P.buf, items));
   P.nslab = nslab;
   P.slabz = B;
   P.block = block;
-  P.nitems = (int)(items.size() / 4);
+  P.nitems = (int)nitems;
   P.grid = (int)std::min((double)resident, 2.0 * P.nitems * nslots);
   return HYB_OK;
 }
@@ -1009,11 +1015,12 @@ hyb_status plan_args(hyb_mesh* m, SweepArgs<T>& A, int nslots, int nsteps) {
   A.yo = P.yo;
   A.ncur = P.ncur;
   A.nstage = P.nstage;
-  A.sitems = (const int4*)P.items.p;
+  int* const base = (int*)P.buf.p;
+  A.sitems = (const int4*)base;
   A.snitems = P.nitems;
-  A.need = (const int*)P.need.p;
-  A.rslab = (const int4*)P.rslab.p;
-  A.sync = (unsigned*)P.sync.p;
+  A.need = base + P.need;
+  A.rslab = (const int4*)(base + P.rslab);
+  A.sync = (unsigned*)(base + P.sync);
   return HYB_OK;
 }
 
@@ -1893,8 +1900,7 @@ hyb_status hyb_mesh_destroy(hyb_mesh* m) {
   for (DevBuf* b : bufs) release(*b);
   for (auto& dir : m->items)
     for (DevBuf& b : dir) release(b);
-  for (SweepPlan& P : m->plans)
-    for (DevBuf* b : {&P.items, &P.need, &P.rslab, &P.sync}) release(*b);
+  for (SweepPlan& P : m->plans) release(P.buf);
   if (m->hscal) cudaFreeHost(m->hscal);
   for (SweepGraph& g : m->graphs)
     if (g.exec) cudaGraphExecDestroy(g.exec);
