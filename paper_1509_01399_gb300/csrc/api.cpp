@@ -1452,7 +1452,7 @@ hyb_status adjoint_impl(hyb_mesh* m, const T* cot, int accumulate) {
         if (paper) paper_slots<T>(m, B, cot, j - l, hq, cq);
         else adjoint_slots<T>(m, B, cot, j - l, hq, cq);
         if (!sweep) {
-          if (paper && h) HYB_TRY(paper_pair<T>(m, B, st));
+          if (paper && h && B.small) HYB_TRY(paper_pair<T>(m, B, st));  // (the tile kernel's launch pairs itself)
           HYB_TRY(launch_level<T>(m, B, !paper, st));
           continue;
         }

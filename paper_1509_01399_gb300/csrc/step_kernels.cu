@@ -872,14 +872,19 @@ __device__ __forceinline__ void adj_edge_tile(const StepArgs<T>& A, int si, int 
 
 template <typename T, bool ADJ>
 __device__ __forceinline__ void refined_rows(const StepArgs<T>& A, long long t);
+template <typename T>
+__device__ __noinline__ void paper_voxels(const StepArgs<T>& A, long long t);
 
 // One time level of every slot in one launch of kStepBlock threads per
 // block: first the edge tiles (two 128-node tiles per block, so their short
 // dependent chains start early), then the interior blocks, then the rows of
 // the refined region (gathers of short latency-bound rows, which fill the
-// slots the interior blocks free towards the end of the level).  All blocks
+// slots the interior blocks free towards the end of the level), and in the
+// paper's adjoint the pairing of the unknown voxels.  All blocks
 // read levels k, k-1 and write disjoint nodes of level k+1.
-template <typename T, bool ADJ, bool TEL, bool ANI>
+// (PAIR: the paper's adjoint with a history to pair with, a variant of its own,
+// as the forward levels lose 1 - 2 % to the mere presence of that branch.)
+template <typename T, bool ADJ, bool TEL, bool ANI, bool PAIR = false>
 __global__ void __launch_bounds__(kStepBlock, sizeof(T) == 4 ? 4 : 2) step_kernel(const __grid_constant__ StepArgs<T> A) {
   extern __shared__ __align__(128) unsigned char hyb_smem[];  // kPipe<T>::bytes
   T* sh = reinterpret_cast<T*>(hyb_smem);
@@ -901,7 +906,13 @@ __global__ void __launch_bounds__(kStepBlock, sizeof(T) == 4 ? 4 : 2) step_kerne
   b -= A.nhe;
   if (b >= A.nitems) {
     pdl_wait();
-    if constexpr (!ANI) refined_rows<T, ADJ>(A, (long long)(b - A.nitems) * kStepBlock + threadIdx.x);
+    b -= A.nitems;
+    if constexpr (PAIR)
+      if (b >= A.nhr) {
+        paper_voxels(A, (long long)(b - A.nhr) * kStepBlock + threadIdx.x);
+        return;
+      }
+    if constexpr (!ANI) refined_rows<T, ADJ>(A, (long long)b * kStepBlock + threadIdx.x);
     return;
   }
   interior_block<T, ADJ, TEL, ANI>(A, b, sh);
@@ -998,6 +1009,30 @@ __device__ __forceinline__ T refined_pair(const StepArgs<T>& A, int v, const T* 
   u[8] = chb[v];
   l[8] = clam[v];
   return refined_pair_sum(u, l, k9);
+}
+
+// Same-index pairing of the paper's adjoint, (u^j, lambda^j) of every unknown
+// voxel (threads of the trailing blocks, per slot: the voxels, then the refined
+// ones): with the step that reads lambda^j, in the slots its interior blocks
+// free, instead of launches of their own that the step waited for (66 x 49 x 57,
+// FEM block of half the lattice, 7.3 -> 5.1 us a level).
+template <typename T>
+__device__ __noinline__ void paper_voxels(const StepArgs<T>& A, long long t) {
+  const long long nv = (long long)A.un[0] * A.un[1] * A.un[2], per = nv + A.nref;
+  if (t >= per * A.nslots) return;
+  const int si = (int)(t / per);
+  const long long r = t - per * si;
+  const Slot<T>& S = A.s[si];
+  double* G = A.G + (long long)si * nv;
+  if (r >= nv) {
+    const int v = (int)(r - nv);
+    G[A.refvox_id[v]] += (double)refined_pair(A, v, S.hist_r, S.chist_r, S.cur, S.ccur, A.k9);
+  } else if (!(A.refvox && A.refvox[r])) {
+    const int x = (int)(r % A.un[0]);
+    const long long yz = r / A.un[0];
+    const int y = (int)(yz % A.un[1]), z = (int)(yz / A.un[1]);
+    G[r] += (double)voxel_pair(A, S.hist_r, S.cur, A.fl[0] + x, A.fl[1] + y, A.fl[2] + z);
+  }
 }
 
 template <typename T>
@@ -1124,7 +1159,10 @@ void launch_step(const StepArgs<T>& a, cudaStream_t st) {
   b.nhe = ((a.nedge + 1) / 2) * a.nslots;
   const long long nref_threads = (long long)(a.nrl + a.nref) * a.nslots;
   b.nhr = (int)((nref_threads + kStepBlock - 1) / kStepBlock);
-  const long long grid = (long long)b.nhe + b.nhr + a.nitems;
+  // forward rows with a history to pair with: the paper's adjoint
+  const bool pair = !ADJ && a.s[0].hist_r;
+  const long long npair = pair ? ((long long)a.un[0] * a.un[1] * a.un[2] + a.nref) * a.nslots : 0;
+  const long long grid = (long long)b.nhe + b.nhr + a.nitems + (npair + kStepBlock - 1) / kStepBlock;
   // programmatic dependent launch: this level's blocks may start while the
   // previous step launch drains (they wait for it before touching its data)
   cudaLaunchConfig_t cfg = {};
@@ -1141,6 +1179,8 @@ void launch_step(const StepArgs<T>& a, cudaStream_t st) {
     cudaLaunchKernelEx(&cfg, step_kernel<T, ADJ, false, true>, b);
   else if (a.sdamp)
     cudaLaunchKernelEx(&cfg, step_kernel<T, ADJ, true, false>, b);
+  else if (pair)
+    cudaLaunchKernelEx(&cfg, step_kernel<T, false, false, false, true>, b);
   else
     cudaLaunchKernelEx(&cfg, step_kernel<T, ADJ, false, false>, b);
 }
@@ -1153,7 +1193,8 @@ void launch_tile_step(const StepArgs<float>& a, bool adjoint, cudaStream_t st) {
 template <typename T, bool ADJ>
 int step_occupancy() {
   int n = 0;
-  for (auto kernel : {step_kernel<T, ADJ, true, false>, step_kernel<T, ADJ, false, true>, step_kernel<T, ADJ, false, false>})
+  for (auto kernel : {step_kernel<T, ADJ, true, false>, step_kernel<T, ADJ, false, true>,
+                      step_kernel<T, false, false, false, true>, step_kernel<T, ADJ, false, false>})
     if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPipe<T>::bytes) !=
             cudaSuccess ||
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kernel, kStepBlock, kPipe<T>::bytes) != cudaSuccess) {
