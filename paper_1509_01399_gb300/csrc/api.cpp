@@ -348,11 +348,11 @@ void set_wave(const hyb_mesh* m, Slot<T>& S, const hyb_source& src, int k, doubl
 }
 
 // Launch geometry of one step of the tile kernel: the interior covers nodes 1 .. n-2 on every
-// axis in 32 x 16 tiles (in x from tile_x0: FP32 tiles start at x = 0); the edge tiles cover the nodes within one node of
+// axis in 32 x 16 tiles (in x from the face node x = 0); the edge tiles cover the nodes within one node of
 // two faces.
 void step_geometry(const hyb_mesh* m, int* npb, int* ntx, int* nedge) {
   *nedge = 1 + (m->n[0] - 4 + 7) / 8 + (m->n[1] - 4 + 7) / 8 + (m->n[2] - 4 + 7) / 8;
-  *ntx = (m->n[0] - 1 - tile_x0(m->d.precision) + kTileX - 1) / kTileX;
+  *ntx = (m->n[0] - 1 + kTileX - 1) / kTileX;
   const int nty = (m->n[1] - 2 + kTileY - 1) / kTileY;
   *npb = *ntx * nty;
 }
@@ -393,8 +393,7 @@ constexpr double kZFaceLevelCost = 3.5;
 // produce the face plane and, on the source face, the trace).
 std::vector<int> build_items(const hyb_mesh* m, int nslots, bool adjoint) {
   const int nx = m->n[0], ny = m->n[1], nz = m->n[2];
-  const int x0 = tile_x0(m->d.precision);
-  const int ntx = (nx - 1 - x0 + kTileX - 1) / kTileX, nty = (ny - 2 + kTileY - 1) / kTileY;
+  const int ntx = (nx - 1 + kTileX - 1) / kTileX, nty = (ny - 2 + kTileY - 1) / kTileY;
   struct Tile {
     int si, tile;
     double base, extra;
@@ -406,7 +405,7 @@ std::vector<int> build_items(const hyb_mesh* m, int nslots, bool adjoint) {
   for (int si = 0; si < nslots; ++si)
     for (int ty = 0; ty < nty; ++ty)
       for (int tx = 0; tx < ntx; ++tx) {
-        const int i0 = x0 + tx * kTileX, j0 = 1 + ty * kTileY;
+        const int i0 = tx * kTileX, j0 = 1 + ty * kTileY;
         const bool face = i0 <= 1 || i0 + kTileX - 1 >= nx - 2 || j0 == 1 || j0 + kTileY - 1 >= ny - 2;
         const bool femt = m->fem && i0 <= m->fh[0] && i0 + kTileX - 1 >= m->fl[0] && j0 <= m->fh[1] &&
                           j0 + kTileY - 1 >= m->fl[1];
@@ -781,17 +780,15 @@ TmapEncodeFn tmap_encoder() {
 // are promoted to 64 bytes, not 128: a box's halo columns then bring in half
 // of the neighbouring tile's line, not all of it (10 % fewer DRAM bytes on
 // the 257^3 lattice with eight sources, time unchanged or lower).
-template <typename T>
 hyb_status encode_map(CUtensorMap* map, const void* base, uint64_t d0, uint64_t d1, uint64_t d2, uint64_t p0,
                       uint64_t p1, uint32_t b0, uint32_t b1) {
   const TmapEncodeFn enc = tmap_encoder();
   if (!enc) return fail(HYB_ERR_CUDA, "cuTensorMapEncodeTiled is not available");
   const cuuint64_t dims[3] = {d0, d1, d2};
-  const cuuint64_t strides[2] = {p0 * sizeof(T), p1 * sizeof(T)};
+  const cuuint64_t strides[2] = {p0 * sizeof(float), p1 * sizeof(float)};
   const cuuint32_t box[3] = {b0, b1, 1};
   const cuuint32_t estr[3] = {1, 1, 1};
-  const CUresult r = enc(map, sizeof(T) == 4 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_FLOAT64, 3,
-                         const_cast<void*>(base), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+  const CUresult r = enc(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, const_cast<void*>(base), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
                          CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_64B,
                          CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   if (r != CUDA_SUCCESS) return fail(HYB_ERR_CUDA, "cuTensorMapEncodeTiled failed (%d)", (int)r);
@@ -801,25 +798,23 @@ hyb_status encode_map(CUtensorMap* map, const void* base, uint64_t d0, uint64_t 
 // Maps of one sweep: the field buffer `field` (3 levels x nsrc slots), the
 // edge weights, and (transposed step with pairing) the history buffer of
 // `hist_levels` levels.
-template <typename T>
-hyb_status step_maps(const hyb_mesh* m, SweepArgs<T>& A, const DevBuf& field, int nsrc, int hist_levels) {
-  HYB_TRY(encode_map<T>(&A.tmf, field.p, m->n[0], m->n[1], (uint64_t)m->n[2] * 3 * nsrc, m->px,
-                        (uint64_t)m->px * m->n[1], Box<T>::BX, kBoxY));
-  HYB_TRY(encode_map<T>(&A.tmp, field.p, m->n[0], m->n[1], (uint64_t)m->n[2] * 3 * nsrc, m->px,
-                        (uint64_t)m->px * m->n[1], Box<T>::PX, kTileY));
+hyb_status step_maps(const hyb_mesh* m, SweepArgs<float>& A, const DevBuf& field, int nsrc, int hist_levels) {
+  HYB_TRY(encode_map(&A.tmf, field.p, m->n[0], m->n[1], (uint64_t)m->n[2] * 3 * nsrc, m->px,
+                        (uint64_t)m->px * m->n[1], Box::BX, kBoxY));
+  HYB_TRY(encode_map(&A.tmp, field.p, m->n[0], m->n[1], (uint64_t)m->n[2] * 3 * nsrc, m->px,
+                        (uint64_t)m->px * m->n[1], Box::PX, kTileY));
   if (m->fem && m->wsz > 0)
-    HYB_TRY(encode_map<T>(&A.tmw, m->W.p, m->wpx, m->wn[1], 3ull * m->wn[2] * (m->batch ? nsrc : 1), m->wpx,
-                          (uint64_t)m->wpx * m->wn[1], Box<T>::BX, kHBoxY));
+    HYB_TRY(encode_map(&A.tmw, m->W.p, m->wpx, m->wn[1], 3ull * m->wn[2] * (m->batch ? nsrc : 1), m->wpx,
+                          (uint64_t)m->wpx * m->wn[1], Box::BX, kHBoxY));
   if (hist_levels > 0 && m->hbox > 0)
-    HYB_TRY(encode_map<T>(&A.tmh, m->hist.p, m->hpx, m->fn[1], (uint64_t)m->fn[2] * nsrc * hist_levels, m->hpx,
-                          (uint64_t)m->hpx * m->fn[1], Box<T>::BX, kHBoxY));
+    HYB_TRY(encode_map(&A.tmh, m->hist.p, m->hpx, m->fn[1], (uint64_t)m->fn[2] * nsrc * hist_levels, m->hpx,
+                          (uint64_t)m->hpx * m->fn[1], Box::BX, kHBoxY));
   return HYB_OK;
 }
 
 // Work items of the step launches with `nslots` slots (built and uploaded the
 // first time this slot count is used, outside any captured sweep).
-template <typename T>
-hyb_status step_items(hyb_mesh* m, SweepArgs<T>& A, int nslots, bool adjoint) {
+hyb_status step_items(hyb_mesh* m, SweepArgs<float>& A, int nslots, bool adjoint) {
   const int d = adjoint ? 1 : 0;
   DevBuf& buf = m->items[d][nslots];
   if (!buf.p) {
@@ -1112,8 +1107,10 @@ hyb_status path_args(hyb_mesh* m, SweepArgs<T>& A, int nslots, int nsteps, const
     case Path::kAllNodes: return HYB_OK;
     case Path::kSweep: return plan_args<T>(m, A, nslots, nsteps);
     case Path::kTiles:
-      HYB_TRY(step_maps<T>(m, A, field, nslots, hist_levels));
-      return step_items<T>(m, A, nslots, adjoint);
+      if constexpr (sizeof(T) == 4) {
+        HYB_TRY(step_maps(m, A, field, nslots, hist_levels));
+        return step_items(m, A, nslots, adjoint);
+      }
   }
   return HYB_OK;
 }

@@ -17,29 +17,21 @@ constexpr int kTileX = 32;       // interior thread tile (x): one warp per tile 
 constexpr int kTileY = 16;       // interior tile (y): two rows per consumer thread
 constexpr int kBoxY = kTileY + 2, kHBoxY = kTileY + 1;
 
-// x geometry of the interior tiles.  FP32 tiles start at x = 32 m (tile 0
-// holds the face node x = 0, whose thread idles): with the row pitch a
-// multiple of 8, a warp's 32 nodes are one aligned 128-byte segment and its
-// stores fill whole 32-byte sectors (partly written sectors, shared by two
-// blocks, cost L2 and DRAM work).  The box then starts 4 nodes left of the
-// tile and is 40 wide.  FP64 tiles start at x = 1 + 32 m, the box at the
-// halo node x = 32 m, 36 wide (256-byte rows; a 40-wide box would cost the
-// second resident block).
-template <typename T>
+// x geometry of the interior tiles.  Tiles start at x = 32 m (tile 0 holds the
+// face node x = 0, whose thread idles): with the row pitch a multiple of 8, a
+// warp's 32 nodes are one aligned 128-byte segment and its stores fill whole
+// 32-byte sectors (partly written sectors, shared by two blocks, cost L2 and
+// DRAM work).  The box then starts 4 nodes left of the tile and is 40 wide.
 struct Box {
-  static constexpr int x0 = sizeof(T) == 4 ? 0 : 1;    // first node of tile 0
-  static constexpr int hx = sizeof(T) == 4 ? 4 : 1;    // box columns left of the tile
-  static constexpr int BX = sizeof(T) == 4 ? 40 : 36;  // box width (a multiple of 16 bytes)
-  static constexpr int C = BX * kBoxY;                 // u box
-  static constexpr int H = BX * kHBoxY;                // edge-weight / stored-u box
+  static constexpr int hx = 4;           // box columns left of the tile
+  static constexpr int BX = 40;          // box width (a multiple of 16 bytes)
+  static constexpr int C = BX * kBoxY;   // u box
+  static constexpr int H = BX * kHBoxY;  // edge-weight / stored-u box
   // u^{k-1} on tiles off the faces: only the tile's own nodes are read, so
-  // the box has no y halo and (FP32) no x halo: PX x kTileY from x = i0 - phx
-  static constexpr int phx = sizeof(T) == 4 ? 0 : 1;
-  static constexpr int PX = sizeof(T) == 4 ? 32 : 34;
+  // the box has no halo: PX x kTileY
+  static constexpr int PX = kTileX;
   static constexpr int P = PX * kTileY;
 };
-// first node (x) of interior tile 0 for a mesh of the given precision
-inline int tile_x0(int precision) { return precision == HYB_FP32 ? Box<float>::x0 : Box<double>::x0; }
 
 // ---- sweep kernel (sweep_kernels.cu: FP64 fields) ----
 constexpr int kMaxBlock = 224;   // row threads per block of the sweep kernel, at most (with the producer warp
@@ -105,10 +97,10 @@ struct alignas(16) Slot {
 // that is a multiple of 8.
 template <typename T>
 struct StepArgs {
-  CUtensorMap tmf;   // field buffer (all levels and slots): {nx, ny, planes}, box Box<T>::BX x kBoxY x 1
-  CUtensorMap tmw;   // edge weights: {wpx, wn1, 3 wn2}, box Box<T>::BX x kHBoxY x 1
-  CUtensorMap tmh;   // history: {hpx, fn1, fn2 x boxes}, box Box<T>::BX x kHBoxY x 1
-  CUtensorMap tmp;   // field buffer as tmf, box Box<T>::PX x kTileY x 1 (u^{k-1} off the faces)
+  CUtensorMap tmf;   // field buffer (all levels and slots): {nx, ny, planes}, box Box::BX x kBoxY x 1
+  CUtensorMap tmw;   // edge weights: {wpx, wn1, 3 wn2}, box Box::BX x kHBoxY x 1
+  CUtensorMap tmh;   // history: {hpx, fn1, fn2 x boxes}, box Box::BX x kHBoxY x 1
+  CUtensorMap tmp;   // field buffer as tmf, box Box::PX x kTileY x 1 (u^{k-1} off the faces)
   int* err;          // [0]: set when a bounded wait timed out
   long long wait;    // cycles such a wait may take (< 0: give up at once if not complete)
   int nx, ny, nz;

@@ -146,7 +146,7 @@ struct Col {
 // ---- shared-memory pipeline of the interior blocks ----
 // A block stages, plane by plane and kPipe<T>::D levels ahead of its z
 // march, boxes that its producer warp loads with bulk tensor copies (TMA):
-// u^k on the tile and a one-node halo (Box<T>: the box starts on a 16-byte
+// u^k on the tile and a one-node halo (Box: the box starts on a 16-byte
 // boundary, hx columns left of the tile, and is BX x 18), u^{k-1} on the
 // same box, and on tiles that meet the FEM block the three edge-weight
 // arrays and, for the transposed step, the stored u of the FEM-owned box
@@ -172,8 +172,8 @@ struct kPipe {
   static constexpr int SW = D + 2;        // edge-weight stages (k-1 .. k+D)
   static constexpr int SH = D + 2;        // stored-u stages (k .. k+1+D)
   static constexpr int NB = pow2(D + 1);  // level barriers (of each kind)
-  static constexpr int CS = round128(Box<T>::C);  // elements per u stage (128-byte aligned)
-  static constexpr int WS = round128(Box<T>::H);  // elements per edge-weight array / stored-u stage
+  static constexpr int CS = round128(Box::C);  // elements per u stage (128-byte aligned)
+  static constexpr int WS = round128(Box::H);  // elements per edge-weight array / stored-u stage
   static constexpr int elems = SC * CS + SP * CS + SW * 3 * WS + SH * WS;
   // Tiles off the FEM block stage only u^k and u^{k-1}: they spend the same
   // shared memory on deeper rings, DP levels ahead.
@@ -210,9 +210,9 @@ struct Producer {
   __device__ __forceinline__ void issue(int g, bool first) const {
     using P = kPipe<T>;
     using R = Ring<T, DEEP>;
-    constexpr uint32_t kCBytes = (uint32_t)(Box<T>::C * sizeof(T));
-    constexpr uint32_t kPBytes = (uint32_t)(Box<T>::P * sizeof(T));
-    constexpr uint32_t kWBytes = (uint32_t)(Box<T>::H * sizeof(T));
+    constexpr uint32_t kCBytes = (uint32_t)(Box::C * sizeof(T));
+    constexpr uint32_t kPBytes = (uint32_t)(Box::P * sizeof(T));
+    constexpr uint32_t kWBytes = (uint32_t)(Box::H * sizeof(T));
     uint64_t* bar = full + ((g - z0) & (R::NB - 1));
     const int wlo = A->wl[2], whi = A->wl[2] + A->wn[2] - 1, hlo = A->fl[2], hhi = A->fh[2];
     const bool c_on = g + 1 <= z1;
@@ -253,13 +253,13 @@ struct Producer {
     empty = bars + P::NBX;
     z0 = zlo;
     z1 = zhi;
-    xf = i0 - Box<T>::hx;
+    xf = i0 - Box::hx;
     yf = j0 - 1;
-    xw = i0 - Box<T>::hx - a.wx0;
+    xw = i0 - Box::hx - a.wx0;
     yw = j0 - 1 - a.wl[1];
-    xh = i0 - Box<T>::hx - a.hx0;
+    xh = i0 - Box::hx - a.hx0;
     yh = j0 - a.fl[1];
-    xp = i0 - Box<T>::phx;
+    xp = i0;
     yp = j0;
     pface = face;
     fem_tile = !DEEP;
@@ -287,7 +287,7 @@ __device__ __forceinline__ void interior_node(const StepArgs<T>& A, const Slot<T
                                               const T* Cp, const T* Pk, const T* Wk, const T* Wm, const T* Hk,
                                               const T* Hp, int rf, T sd) {
   using P = kPipe<T>;
-  constexpr int kBoxX = Box<T>::BX;
+  constexpr int kBoxX = Box::BX;
   if (ZF && FACE && (C.dxs != 0 || C.dys != 0)) return;  // near two faces: edge tiles
   const T c2 = A.c2;
   const T c0 = Ck[0], cm = Cm[0], cp = Cp[0], pv = Pk[0];
@@ -314,10 +314,8 @@ __device__ __forceinline__ void interior_node(const StepArgs<T>& A, const Slot<T
   } else if constexpr (ANI) {
     val = c0 + ((c0 - pv) + c2 * ((k0 * ((xm - c0) + (xp - c0)) + k1 * ((ym - c0) + (yp - c0))) +
                                   k2 * ((cm - c0) + (cp - c0))));
-  } else if constexpr (sizeof(T) == 4) {  // unit weights: the neighbour sum minus 6 u^k
+  } else {  // unit weights: the neighbour sum minus 6 u^k
     val = c0 + ((c0 - pv) + c2 * ((((xm + xp) + (ym + yp)) + (cm + cp)) - T(6) * c0));
-  } else {  // FP64 sums the six differences
-    val = c0 + ((c0 - pv) + c2 * lap7(xm, xp, ym, yp, cm, cp, c0));
   }
   if constexpr (ZF) {  // the z face node next to this node (the rows of the x / y faces below)
     const int f = dzs > 0 ? 5 : 4;
@@ -447,8 +445,8 @@ __device__ __forceinline__ void xface_levels(const StepArgs<T>& A, const Slot<T>
   const bool row_on = j >= 2 && j <= A.ny - 3;
   const int f = X.sd > 0 ? 1 : 0;
   const int sd = X.sd;
-  constexpr int kBoxX = Box<T>::BX;
-  const int o = (r + 1) * kBoxX + (X.mi - X.i0 + Box<T>::hx);  // m in a u box
+  constexpr int kBoxX = Box::BX;
+  const int o = (r + 1) * kBoxX + (X.mi - X.i0 + Box::hx);  // m in a u box
   const T c2 = A.c2, rf = ANI ? A.ra[0] : A.r;
   const T k0 = ANI ? A.kapt[0] : T(1), k1 = ANI ? A.kapt[1] : T(1), k2 = ANI ? A.kapt[2] : T(1);
   const bool abc = (S.mask_f >> f) & 1;
@@ -473,10 +471,8 @@ __device__ __forceinline__ void xface_levels(const StepArgs<T>& A, const Slot<T>
       if constexpr (ANI)
         val = c0 + ((c0 - pv) + c2 * ((k0 * ((xm - c0) + (xp - c0)) + k1 * ((ym - c0) + (yp - c0))) +
                                       k2 * ((cm - c0) + (cp - c0))));
-      else if constexpr (sizeof(T) == 4)
-        val = c0 + ((c0 - pv) + c2 * ((((xm + xp) + (ym + yp)) + (cm + cp)) - T(6) * c0));
       else
-        val = c0 + ((c0 - pv) + c2 * lap7(xm, xp, ym, yp, cm, cp, c0));
+        val = c0 + ((c0 - pv) + c2 * ((((xm + xp) + (ym + yp)) + (cm + cp)) - T(6) * c0));
       const T ub = Ck[sd];
       const int offb = off + sd;
       if constexpr (!ADJ) {
@@ -559,14 +555,14 @@ __device__ __forceinline__ void interior_levels(const StepArgs<T>& A, const Slot
   const int tx = t & 31, ty = t >> 5;
   const int nz = A.nz;
   const int pl = A.px * A.ny;
-  constexpr int kBoxX = Box<T>::BX;
-  const int o0 = (ty + 1) * kBoxX + (tx + Box<T>::hx);  // row 0 in a u box / edge-weight array
+  constexpr int kBoxX = Box::BX;
+  const int o0 = (ty + 1) * kBoxX + (tx + Box::hx);  // row 0 in a u box / edge-weight array
   const int o1 = o0 + (kTileY / 2) * kBoxX;             // row 1
-  const int h0 = ty * kBoxX + (tx + Box<T>::hx);        // row 0 in a stored-u box
+  const int h0 = ty * kBoxX + (tx + Box::hx);        // row 0 in a stored-u box
   const int h1 = h0 + (kTileY / 2) * kBoxX;
   // u^{k-1}: the u box layout on face tiles, else the halo-free box
-  const int p0 = FACE ? o0 : ty * Box<T>::PX + (tx + Box<T>::phx);
-  const int p1 = FACE ? o1 : p0 + (kTileY / 2) * Box<T>::PX;
+  const int p0 = FACE ? o0 : ty * Box::PX + tx;
+  const int p1 = FACE ? o1 : p0 + (kTileY / 2) * Box::PX;
   const bool act0 = !FACE || active[0], act1 = !FACE || active[1];  // every row of a tile off the faces is active
   T* __restrict__ gnext = S.next;
   int off0 = C[0].i + A.px * C[0].j + pl * z0;       // field offsets of the two nodes
@@ -687,7 +683,7 @@ __device__ __forceinline__ void interior_block(const StepArgs<T>& A, int b, T* s
   if (z0 >= z1) return;  // whole block
   const int t = (int)threadIdx.x;
   const int tx = t & 31, ty = t >> 5;
-  const int i0 = Box<T>::x0 + txx * kTileX, j0 = 1 + tyy * kTileY;
+  const int i0 = txx * kTileX, j0 = 1 + tyy * kTileY;
   const Slot<T>& S = A.s[si];
   const bool has_fem = A.fl[0] <= A.fh[0];
   const bool pairing = ADJ && S.hist_r != nullptr;
@@ -885,7 +881,7 @@ __device__ __noinline__ void paper_voxels(const StepArgs<T>& A, long long t);
 // (PAIR: the paper's adjoint with a history to pair with, a variant of its own,
 // as the forward levels lose 1 - 2 % to the mere presence of that branch.)
 template <typename T, bool ADJ, bool TEL, bool ANI, bool PAIR = false>
-__global__ void __launch_bounds__(kStepBlock, sizeof(T) == 4 ? 4 : 2) step_kernel(const __grid_constant__ StepArgs<T> A) {
+__global__ void __launch_bounds__(kStepBlock, 4) step_kernel(const __grid_constant__ StepArgs<T> A) {
   extern __shared__ __align__(128) unsigned char hyb_smem[];  // kPipe<T>::bytes
   T* sh = reinterpret_cast<T*>(hyb_smem);
   pdl_trigger();  // the next level's launch may start its blocks
