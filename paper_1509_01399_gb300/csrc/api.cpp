@@ -335,16 +335,26 @@ void set_wave(const hyb_mesh* m, Slot<T>& S, const hyb_source& src, int k, doubl
   phase_of(m, src, k, dt, &mask, &sm);
   S.mask_f = mask;
   S.src_mask = sm;
-  S.st = k * dt;
   const double h = m->d.h;
-  for (int f = 0; f < 6; ++f) S.sf[f] = dt * dt * 2.0 / (m->ani ? m->hv[f >> 1] : h) * src.amp * w.fac[f];
+  double sd[3];
+  for (int f = 0; f < 6; ++f) S.sf[f] = (T)(dt * dt * 2.0 / (m->ani ? m->hv[f >> 1] : h) * src.amp * w.fac[f]);
   for (int a = 0; a < 3; ++a) {
-    S.sd[a] = m->ani ? w.d[a] * m->hv[a] : w.d[a];  // per-axis steps: the delay d . (x - x0) axis by axis
+    sd[a] = w.d[a] * (m->ani ? m->hv[a] : h);  // the delay d . (x - x0) axis by axis
     S.si0[a] = w.i0[a];
   }
-  S.sh = m->ani ? 1.0 : h;
-  S.somega = src.omega;
-  S.st1 = 2.0 * M_PI / src.omega;
+  const double t1 = 2.0 * M_PI / src.omega;
+  if constexpr (sizeof(T) == 8) {
+    S.pulse = {k * dt, {sd[0], sd[1], sd[2]}, src.omega, t1};
+  } else {
+    auto split = [](float (&f)[2], double v) {
+      f[0] = (float)v;
+      f[1] = (float)(v - (double)f[0]);
+    };
+    split(S.pulse.st, k * dt);
+    for (int a = 0; a < 3; ++a) split(S.pulse.sd[a], sd[a]);
+    split(S.pulse.omega, src.omega);
+    split(S.pulse.t1, t1);
+  }
 }
 
 // Launch geometry of one step of the tile kernel: the interior covers nodes 1 .. n-2 on every

@@ -46,6 +46,17 @@ constexpr int kReduceBlocks = 512;
 constexpr double kGradPairScale = 6.0;
 constexpr int kReduceThreads = 256;
 
+// A slot's pulse at t_k: its time t_k, the delay per index step h d, omega and
+// the end t1; for FP32 fields as unevaluated sums of two FP32 numbers.
+template <typename T>
+struct Pulse {
+  double st, sd[3], omega, t1;
+};
+template <>
+struct Pulse<float> {
+  float st[2], sd[3][2], omega[2], t1[2];
+};
+
 // One problem (one source of one mesh) at one time level.  A sweep launch gets
 // the slots of its first level and advances them from level to level itself.
 template <typename T>
@@ -64,12 +75,9 @@ struct alignas(16) Slot {
   int obs_face;      // face recorded in the trace / receiving the cotangent
   // Plane wave of the slot's source: the flux term of node (i, j, k) on face f
   // is sf[f] p(t_k - h (d . ((i, j, k) - si0))), p(s) = sin(omega s) on [0, t1].
-  double st;         // t_k
-  double sf[6];      // tau^2 (2 / h) amp (-(d . n_f)) on the entry faces, 0 elsewhere
-  double sd[3];      // unit direction d
-  double sh;         // lattice spacing h
+  T sf[6];           // tau^2 (2 / h) amp (-(d . n_f)) on the entry faces, 0 elsewhere
   int si0[3];        // entry corner (node index)
-  double somega, st1;
+  Pulse<T> pulse;
   // paper-mode adjoint (forward rows on lambda): the cotangent row entering on
   // the observation face as inj_scale 2^b c_j, b the node's boundary axes
   const T* inj;

@@ -823,7 +823,7 @@ __global__ void slots_kernel(const __grid_constant__ SweepArgs<T> A) {
   S->chist_r = hist && S->chist_r ? S->chist_r + l * A.chist_step : nullptr;
   if constexpr (M == kForward) {
     S->mask_f = phase(A, si, step, &S->src_mask);
-    S->st = __dmul_rn((double)step, A.dt);
+    S->pulse.st = __dmul_rn((double)step, A.dt);
   } else if constexpr (M == kAdjoint) {
     S->mask_f = phase(A, si, step, (int*)nullptr);
     S->mask_e = phase(A, si, step - 1, (int*)nullptr);
