@@ -1098,7 +1098,7 @@ hyb_status launch_piece(hyb_mesh* m, const SweepArgs<T>& A, StepMode mode, cudaS
 // and history that FP32 rows would wait for: 257^3, eight sources, refined,
 // 0.47 / 0.51 ms a level against 0.66 / 0.92 ms by the sweep kernel (without a FEM
 // block 0.40 against 0.32); per-axis steps, 257 x 193 x 321 with eight sources,
-// 0.38 / 0.41 ms against 0.52 / 0.71, and faster at every size down to 21 x 18 x
+// 0.37 / 0.43 ms against 0.52 / 0.71, and faster at every size down to 21 x 18 x
 // 26 (10.3 against 11.1 us a step pair).  FP64 rows wait for the FP64 pipe, and
 // gain 1.5 - 1.7 times from the sweep kernel at every size measured (its comment).
 enum class Path { kAllNodes, kTiles, kSweep };

@@ -44,7 +44,7 @@
 // Lattices whose steps differ per axis (ANI) weigh the axis terms by kap and take
 // the faces' own absorbing coefficients, by variants of the same kernel without
 // refinement (those weights are operands from the argument block and cost no
-// registers): 257 x 193 x 321, eight sources, 0.38 / 0.41 ms a level (forward /
+// registers): 257 x 193 x 321, eight sources, 0.37 / 0.43 ms a level (forward /
 // transposed), 0.95 / 2.11 ms by two kernels over the nodes and 0.52 / 0.71 ms by
 // the sweep kernel before.
 //
@@ -274,6 +274,23 @@ struct Producer {
   }
 };
 
+// Transposed row with per-axis steps in the gathered order of adj_rhs (diag: the
+// coefficient of the node itself).  Its rounding of the diagonal, the same at
+// every level, dominates the gradient's FP32 error and is kept: rows from
+// differences round better but end up as far from these as both are from FP64.
+template <typename T>
+__device__ __forceinline__ T gathered_row(T c2, T diag, T wxm, T wxp, T wym, T wyp, T wzm, T wzp, T c, T xm, T xp, T ym,
+                                          T yp, T zm, T zp, T pv) {
+  T rhs = diag * c;
+  rhs += c2 * wxm * xm;
+  rhs += c2 * wxp * xp;
+  rhs += c2 * wym * ym;
+  rhs += c2 * wyp * yp;
+  rhs += c2 * wzm * zm;
+  rhs += c2 * wzp * zp;
+  return rhs - pv;
+}
+
 // One node (i, j, k) of an interior block from the staged planes: Ck, Cm, Cp
 // are this node in the u^k boxes of planes k, k-1, k+1, Pk in the u^{k-1}
 // box, Wk / Wm in the edge-weight arrays of planes k / k-1, Hk / Hp in the
@@ -307,10 +324,15 @@ __device__ __forceinline__ void interior_node(const StepArgs<T>& A, const Slot<T
     wzm = Wm[2 * P::WS];
     const T lap =
         wxp * (xp - c0) + wxm * (xm - c0) + wyp * (yp - c0) + wym * (ym - c0) + wzp * (cp - c0) + wzm * (cm - c0);
-    if constexpr (TEL)  // damped row (sd: the node's damping ratio)
+    if constexpr (ADJ && ANI)
+      val = gathered_row(c2, T(2) + c2 * -(wxp + wxm + wyp + wym + wzp + wzm), wxm, wxp, wym, wyp, wzm, wzp, c0, xm, xp,
+                         ym, yp, cm, cp, pv);
+    else if constexpr (TEL)  // damped row (sd: the node's damping ratio)
       val = c0 + ((c0 - pv) * (T(1) - sd) + c2 * lap) / (T(1) + sd);
     else
       val = c0 + ((c0 - pv) + c2 * lap);
+  } else if constexpr (ADJ && ANI) {
+    val = gathered_row(c2, T(2) + c2 * A.kdiag, k0, k0, k1, k1, k2, k2, c0, xm, xp, ym, yp, cm, cp, pv);
   } else if constexpr (ANI) {
     val = c0 + ((c0 - pv) + c2 * ((k0 * ((xm - c0) + (xp - c0)) + k1 * ((ym - c0) + (yp - c0))) +
                                   k2 * ((cm - c0) + (cp - c0))));
@@ -468,7 +490,9 @@ __device__ __forceinline__ void xface_levels(const StepArgs<T>& A, const Slot<T>
       const T c0 = Ck[0], xm = Ck[-1], xp = Ck[1], ym = Ck[-kBoxX], yp = Ck[kBoxX];
       const T cm = Cm[0], cp = Cp[0], pv = Pk[0];
       T val;
-      if constexpr (ANI)
+      if constexpr (ADJ && ANI)
+        val = gathered_row(c2, T(2) + c2 * A.kdiag, k0, k0, k1, k1, k2, k2, c0, xm, xp, ym, yp, cm, cp, pv);
+      else if constexpr (ANI)
         val = c0 + ((c0 - pv) + c2 * ((k0 * ((xm - c0) + (xp - c0)) + k1 * ((ym - c0) + (yp - c0))) +
                                       k2 * ((cm - c0) + (cp - c0))));
       else
