@@ -1125,13 +1125,14 @@ hyb_status path_args(hyb_mesh* m, SweepArgs<T>& A, int nslots, int nsteps, const
   return HYB_OK;
 }
 
-// One level of every slot (not the sweep kernel).
+// One level of every slot (not the sweep kernel; `pair`: the tile kernel's
+// launch pairs too).
 template <typename T>
-hyb_status launch_level(hyb_mesh* m, const SweepArgs<T>& A, bool adjoint, cudaStream_t st) {
+hyb_status launch_level(hyb_mesh* m, const SweepArgs<T>& A, bool adjoint, bool pair, cudaStream_t st) {
   if (A.small) {
     launch_all_nodes<T>(A, adjoint, st);
   } else if constexpr (sizeof(T) == 4) {
-    launch_tile_step(A, adjoint, st);
+    launch_tile_step(A, adjoint, pair, st);
   }
   HYB_LAUNCHED(m);
   return HYB_OK;
@@ -1150,7 +1151,7 @@ hyb_status forward_levels(hyb_mesh* m, SweepArgs<T>& A, const hyb_source* src, i
     const bool h = hl && l < nh;
     forward_slots<T>(m, A, src, nsrc, nsteps, dt, k + l, trace, h ? hl + l * lvl : nullptr, h ? chl + l * clvl : nullptr);
     if (!sweep) {
-      HYB_TRY(launch_level<T>(m, A, false, st));
+      HYB_TRY(launch_level<T>(m, A, false, false, st));
       continue;
     }
     A.nlev = q;
@@ -1386,6 +1387,22 @@ hyb_status paper_pair(hyb_mesh* m, SweepArgs<T>& A, cudaStream_t st) {
   return HYB_OK;
 }
 
+// Whether the tile kernel's launch takes the paper's pairing along (paper_voxels)
+// or launches of its own do it first.  In the step's launch it saves those
+// launches, but its sixteen loads a voxel run in blocks that hold the step's
+// shared memory, four to an SM; a refined voxel there weighs about ninety others
+// (its 81 table entries are FP64).  Gradients in ms, in the step / on their own:
+// full block of 105^3 (0.94 M voxels) 4.76 / 4.82, 113^3 (1.19 M) 5.48 / 5.50, 121^3
+// (1.48 M) 6.67 / 6.42, 257^3 30.0 / 25.0, four slots of 193^3 48.6 / 41.4; block of half
+// the lattice, 1 % and 5 % refined, 97^3 4.89 / 5.87 and 6.03 / 6.32, 129^3 6.05 /
+// 6.90 and 7.35 / 7.13.
+constexpr double kPairVoxelsInStep = 1.2e6, kRefinedVoxelWeight = 90.0;
+
+template <typename T>
+bool pairs_in_step(const hyb_mesh* m, const SweepArgs<T>& A) {
+  return path_of(A) == Path::kTiles && (double)m->nu + kRefinedVoxelWeight * m->nc <= kPairVoxelsInStep;
+}
+
 // Gradient pairing of level 0: (u^0, lambda^1) on every unknown voxel.
 template <typename T>
 hyb_status pair_first(hyb_mesh* m, SweepArgs<T>& A, const T* level0, const T* clevel0, cudaStream_t st) {
@@ -1459,8 +1476,9 @@ hyb_status adjoint_impl(hyb_mesh* m, const T* cot, int accumulate) {
         if (paper) paper_slots<T>(m, B, cot, j - l, hq, cq);
         else adjoint_slots<T>(m, B, cot, j - l, hq, cq);
         if (!sweep) {
-          if (paper && h && B.small) HYB_TRY(paper_pair<T>(m, B, st));  // (the tile kernel's launch pairs itself)
-          HYB_TRY(launch_level<T>(m, B, !paper, st));
+          const bool in_step = paper && h && pairs_in_step(m, B);
+          if (paper && h && !in_step) HYB_TRY(paper_pair<T>(m, B, st));
+          HYB_TRY(launch_level<T>(m, B, !paper, in_step, st));
           continue;
         }
         B.nlev = q;

@@ -222,8 +222,9 @@ enum StepMode { kForward = 0, kAdjoint = 1, kPaper = 2 };
 // bytes of ring each).  Returns the kernels launched.
 int launch_sweep(const SweepArgs<double>& a, StepMode mode, int block, int grid, int smem, cudaStream_t st);
 // One level of every slot by the tile kernel (edge tiles, interior tiles and
-// refined rows in one launch).
-void launch_tile_step(const StepArgs<float>& a, bool adjoint, cudaStream_t st);
+// refined rows in one launch; `pair`: forward rows with the paper's adjoint's
+// pairing of A.s's history in it).
+void launch_tile_step(const StepArgs<float>& a, bool adjoint, bool pair, cudaStream_t st);
 // Resident blocks per SM of the tile kernel, at least 1.
 int tile_blocks_per_sm(bool adjoint);
 // One level by the generic all-node kernel (A.small), from A.s as it stands.

@@ -1035,7 +1035,8 @@ __device__ __forceinline__ T refined_pair(const StepArgs<T>& A, int v, const T* 
 // voxel (threads of the trailing blocks, per slot: the voxels, then the refined
 // ones): with the step that reads lambda^j, in the slots its interior blocks
 // free, instead of launches of their own that the step waited for (66 x 49 x 57,
-// FEM block of half the lattice, 7.3 -> 5.1 us a level).
+// FEM block of half the lattice, 7.3 -> 5.1 us a level).  Large blocks keep those
+// launches (the host's pairs_in_step).
 template <typename T>
 __device__ __noinline__ void paper_voxels(const StepArgs<T>& A, long long t) {
   const long long nv = (long long)A.un[0] * A.un[1] * A.un[2], per = nv + A.nref;
@@ -1174,13 +1175,11 @@ void launch_all_nodes(const StepArgs<T>& a, bool adjoint, cudaStream_t st) {
 }
 
 template <typename T, bool ADJ>
-void launch_step(const StepArgs<T>& a, cudaStream_t st) {
+void launch_step(const StepArgs<T>& a, bool pair, cudaStream_t st) {
   StepArgs<T> b = a;
   b.nhe = ((a.nedge + 1) / 2) * a.nslots;
   const long long nref_threads = (long long)(a.nrl + a.nref) * a.nslots;
   b.nhr = (int)((nref_threads + kStepBlock - 1) / kStepBlock);
-  // forward rows with a history to pair with: the paper's adjoint
-  const bool pair = !ADJ && a.s[0].hist_r;
   const long long npair = pair ? ((long long)a.un[0] * a.un[1] * a.un[2] + a.nref) * a.nslots : 0;
   const long long grid = (long long)b.nhe + b.nhr + a.nitems + (npair + kStepBlock - 1) / kStepBlock;
   // programmatic dependent launch: this level's blocks may start while the
@@ -1205,9 +1204,9 @@ void launch_step(const StepArgs<T>& a, cudaStream_t st) {
     cudaLaunchKernelEx(&cfg, step_kernel<T, ADJ, false, false>, b);
 }
 
-void launch_tile_step(const StepArgs<float>& a, bool adjoint, cudaStream_t st) {
-  if (adjoint) launch_step<float, true>(a, st);
-  else launch_step<float, false>(a, st);
+void launch_tile_step(const StepArgs<float>& a, bool adjoint, bool pair, cudaStream_t st) {
+  if (adjoint) launch_step<float, true>(a, false, st);
+  else launch_step<float, false>(a, pair, st);
 }
 
 template <typename T, bool ADJ>
