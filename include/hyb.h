@@ -71,7 +71,10 @@ typedef struct {
   int32_t bc[6];       /* HYB_BC_* per face: d_n u = 0, or d_n u = -d_t u
                           discretised by Eq. (eq:abs2) */
   int32_t precision;   /* HYB_FP64, or HYB_FP32 (FP32 fields and stencils,
-                          FP64 gradient accumulation and CG reductions) */
+                          FP64 gradient accumulation and CG reductions).
+                          HYB_FP32 with refinement or the telegraph model
+                          needs planes of fewer than 2^30 padded nodes and a
+                          FEM block of fewer than 2^31 (HYB_ERR_ARG) */
   int32_t ckpt_every;  /* 0: the forward keeps u on the FEM-owned nodes at
                           every level for the gradient; C > 0: it keeps full
                           fields every C steps and the adjoint recomputes each

@@ -357,6 +357,21 @@ void set_wave(const hyb_mesh* m, Slot<T>& S, const hyb_source& src, int k, doubl
   }
 }
 
+// Rows start on 32-byte boundaries (whole sectors per warp row).
+int row_pitch(int nx) {
+  return (nx + 7) & ~7;
+}
+
+// Lattices beyond the tile kernel's 32-bit offsets: within two planes, and
+// within the FEM-owned box.
+bool beyond_tiles(const hyb_mesh_desc& d) {
+  if ((long long)row_pitch(d.n[0]) * d.n[1] >= 1LL << 30) return true;
+  if (d.fem_lo[0] < 0) return false;
+  const int hx0 = (d.fem_lo[0] + 1) & ~7;
+  return (long long)((d.fem_hi[0] - hx0 + 7) & ~7) * (d.fem_hi[1] - d.fem_lo[1] - 1) >=
+         (1LL << 31) / (d.fem_hi[2] - d.fem_lo[2] - 1);
+}
+
 // Launch geometry of one step of the tile kernel: the interior covers nodes 1 .. n-2 on every
 // axis in 32 x 16 tiles (in x from the face node x = 0); the edge tiles cover the nodes within one node of
 // two faces.
@@ -427,13 +442,15 @@ std::vector<int> build_items(const hyb_mesh* m, int nslots, bool adjoint) {
   const double resident = (double)std::max(m->nsm, 1) * std::max(m->bps, 1);
   const double levels_per_block = (double)tiles.size() * (nz - 2) / resident;
   const double target = total / (resident * step_waves(levels_per_block, nslots));
+  // planes of an item and the ones next to it: 32-bit offsets (beyond_tiles leaves at least one)
+  const long long most = ((1LL << 31) - 1) / ((long long)m->px * ny) - 1;
   std::vector<std::pair<double, std::array<int, 4>>> items;
   for (const Tile& t : tiles) {
     double acc = 0.0;
     int z0 = 1;
     for (int k = 1; k <= nz - 2; ++k) {
       acc += t.base + ((k >= zf0 && k <= zf1) ? t.extra : 0.0) + ((k == 1 || k == nz - 2) ? kZFaceLevelCost : 0.0);
-      if (acc >= target || k == nz - 2) {
+      if (acc >= target || k - z0 + 1 >= most || k == nz - 2) {
         items.push_back({acc, {t.si, t.tile, z0, k + 1}});
         z0 = k + 1;
         acc = 0.0;
@@ -955,13 +972,12 @@ void base_args(const hyb_mesh* m, SweepArgs<T>& A, double dt, int nslots) {
   A.c2 = (T)(dt * dt / (h * h));
   A.r = (T)((h - dt) / (h + dt));
   // the generic kernel: lattices without an interior, and beyond the sweep
-  // kernel's 32-bit item indices or, with per-axis steps, the tile kernel's
-  // 32-bit node offsets
+  // kernel's 32-bit item indices or the tile kernel's 32-bit offsets
   A.small = (m->n[0] < 5 || m->n[1] < 5 || m->n[2] < 5) ? 1 : 0;
   if (m->d.precision == HYB_FP64 && m->nc == 0 &&
       ((long long)m->n[0] * m->n[1] + (m->n[0] + (long long)m->n[1]) * kMaxMarch >= 1LL << 30 || m->n[2] >= 1 << 23))
     A.small = 1;
-  if (m->d.precision == HYB_FP32 && m->ani && (long long)m->px * m->n[1] * m->n[2] >= 1LL << 31) A.small = 1;
+  if (m->d.precision == HYB_FP32 && beyond_tiles(m->d)) A.small = 1;
   if (m->ani) {  // axis terms weighed by kap
     A.ani = 1;
     for (int a = 0; a < 3; ++a) {
@@ -1813,6 +1829,8 @@ hyb_status hyb_mesh_create(const hyb_mesh_desc* d, void* stream, hyb_mesh** out)
         return fail(HYB_ERR_ARG, "FEM block axis %d: need 0 <= lo, hi <= n-1, hi - lo >= 2", a);
     }
   }
+  if (d->precision == HYB_FP32 && beyond_tiles(*d) && (d->refine_mask || d->model == HYB_MODEL_TELEGRAPH))
+    return fail(HYB_ERR_ARG, "lattice plane or FEM block too large for FP32 fields with refinement or the telegraph model");
   hyb_mesh* m = new (std::nothrow) hyb_mesh();
   if (!m) return fail(HYB_ERR_OOM, "host allocation failed");
   m->d = *d;
@@ -1822,7 +1840,7 @@ hyb_status hyb_mesh_create(const hyb_mesh_desc* d, void* stream, hyb_mesh** out)
   m->st = (cudaStream_t)stream;
   for (int a = 0; a < 3; ++a) m->n[a] = d->n[a];
   m->N = (long long)d->n[0] * d->n[1] * d->n[2];
-  m->px = (d->n[0] + 7) & ~7;  // rows start on 32-byte boundaries (whole sectors per warp row)
+  m->px = row_pitch(d->n[0]);
   m->Np = (long long)m->px * d->n[1] * d->n[2];
   m->fem = fem;
   for (int a = 0; a < 3; ++a) {

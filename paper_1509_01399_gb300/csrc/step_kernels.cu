@@ -345,6 +345,7 @@ __device__ __forceinline__ void interior_node(const StepArgs<T>& A, const Slot<T
     const T ub = Cb[0];
     const bool abc = (S.mask_f >> f) & 1;
     const int offb = off + dzs * A.px * A.ny;
+    const long long gb = (gnext - S.next) + offb;  // (fields hold 2^31 nodes and more; an item's offsets fit 32 bits)
     const T rf = ANI ? A.ra[2] : A.r;
     if constexpr (!ADJ) {
       T vb;
@@ -354,7 +355,7 @@ __device__ __forceinline__ void interior_node(const StepArgs<T>& A, const Slot<T
         T lb = T(2) * k2 * (c0 - ub);
         lb += k0 * ((Cb[-1] - ub) + (Cb[1] - ub));
         lb += k1 * ((Cb[-kBoxX] - ub) + (Cb[kBoxX] - ub));
-        vb = ub + ((ub - S.prev[offb]) + c2 * lb);  // (u^{k-1} of the face plane is not staged)
+        vb = ub + ((ub - S.prev[gb]) + c2 * lb);  // (u^{k-1} of the face plane is not staged)
         if ((S.src_mask >> f) & 1) vb += src_term(S, f, C.i, C.j, k + dzs);
         if (S.inj && S.obs_face == f) vb += S.inj_scale * T(2) * S.inj[face_index(f, C.i, C.j, k + dzs, A.nx, A.ny)];
       }
@@ -368,7 +369,7 @@ __device__ __forceinline__ void interior_node(const StepArgs<T>& A, const Slot<T
         lb += c2 * k0 * (Cb[-1] + Cb[1]);
         lb += c2 * k1 * (Cb[-kBoxX] + Cb[kBoxX]);
       }
-      if (!((S.mask_c >> f) & 1)) lb -= S.prev[offb];
+      if (!((S.mask_c >> f) & 1)) lb -= S.prev[gb];
       if (S.obs_r && S.obs_face == f) lb += S.obs_r[face_index(f, C.i, C.j, k + dzs, A.nx, A.ny)];
       val += (abc ? ub : T(2) * c2 * k2 * ub) - c2 * coef_mb * ub;
       if ((S.mask_e >> f) & 1) val -= rf * lb;
@@ -472,9 +473,9 @@ __device__ __forceinline__ void xface_levels(const StepArgs<T>& A, const Slot<T>
   const T c2 = A.c2, rf = ANI ? A.ra[0] : A.r;
   const T k0 = ANI ? A.kapt[0] : T(1), k1 = ANI ? A.kapt[1] : T(1), k2 = ANI ? A.kapt[2] : T(1);
   const bool abc = (S.mask_f >> f) & 1;
-  T* __restrict__ gnext = S.next;
   const int pl = A.px * A.ny;
-  int off = X.mi + A.px * j + pl * z0;
+  T* __restrict__ gnext = S.next + (long long)pl * z0;
+  int off = X.mi + A.px * j;
   for (int k = z0; k < z1; ++k, off += pl) {
     const int q = k - z0;
     const bool ok = mbar_wait(pr.full + (q & (R::NB - 1)), (uint32_t)((q / R::NB) & 1), budget, A.err);
@@ -588,8 +589,8 @@ __device__ __forceinline__ void interior_levels(const StepArgs<T>& A, const Slot
   const int p0 = FACE ? o0 : ty * Box::PX + tx;
   const int p1 = FACE ? o1 : p0 + (kTileY / 2) * Box::PX;
   const bool act0 = !FACE || active[0], act1 = !FACE || active[1];  // every row of a tile off the faces is active
-  T* __restrict__ gnext = S.next;
-  int off0 = C[0].i + A.px * C[0].j + pl * z0;       // field offsets of the two nodes
+  T* __restrict__ gnext = S.next + (long long)pl * z0;
+  int off0 = C[0].i + A.px * C[0].j;                 // field offsets of the two nodes from plane z0
   int off1 = off0 + (kTileY / 2) * A.px;
   // refinement flags of the two nodes, loaded one level ahead (their
   // latency then overlaps the wait for the level's planes)

@@ -1,0 +1,26 @@
+"""Sizes that no kernel takes are refused when the mesh is described, before
+anything is allocated (so this needs no GPU)."""
+import numpy as np
+import pytest
+
+CASES = {  # lattice, FEM block: planes of 2^30 padded nodes, blocks of 2^31 nodes
+    "telegraph_plane": ((7, 140_000_000, 7), (2, 2, 2), (4, 4, 4)),
+    "telegraph_block": ((1400, 1400, 1400), (2, 2, 2), (1397, 1397, 1397)),
+    "refined_plane": ((40_000, 30_000, 9), (2, 2, 2), (5, 5, 5)),
+}
+
+
+@pytest.mark.parametrize("name", sorted(CASES))
+def test_fp32_beyond_the_tile_kernel(name):
+    hyb = pytest.importorskip("paper_1509_01399_gb300.hyb")
+    d = hyb.hyb_mesh_desc()
+    for a in range(3):
+        d.n[a], d.fem_lo[a], d.fem_hi[a] = (v[a] for v in CASES[name])
+    d.h, d.a_max, d.precision = 0.1, 1.0, hyb.HYB_FP32
+    mask = np.ones(1, np.uint8)
+    if name.startswith("telegraph"):
+        d.model = hyb.HYB_MODEL_TELEGRAPH
+    else:
+        d.refine_mask = mask.ctypes.data
+    with pytest.raises(hyb.HybError, match="too large for FP32"):
+        hyb.hyb_mesh_create(d, 0)
