@@ -895,13 +895,14 @@ hyb_status build_plan(hyb_mesh* m, int nslots) {
   const int B = (int)std::min((double)kMaxMarch, std::max(1.0, std::floor(work / block / (kItemsPerBlock * resident))));
   const int nslab = (nz - 2 + B - 1) / B;
   std::vector<int> items, need(nslab, 0), rslab(4 * (size_t)nslab, 0);
-  auto add = [&](int kind, int slab, long long first, long long end, int w) {
-    items.insert(items.end(), {kind | slab << 8, (int)first, (int)end, w});
+  // (first and end are read as unsigned: the entries of two z faces of nearly 2^31 nodes)
+  auto add = [&](int kind, int slab, long long first, long long end, int z_end) {
+    items.insert(items.end(), {slab, (int)(unsigned)first, (int)(unsigned)end, kind | z_end << 8});
     ++need[slab];
   };
   const int mx = nx - 4, my = ny - 4, per = block / 128;
   // entries of a face or refined item: up to kGatherRounds per thread
-  const double gathered = nslots * (2.0 * mx * my + 2.0 * (mx + my) * (nz - 4) + m->nrl + m->nc);
+  const double gathered = nslots * (2.0 * mx * my + 2.0 * ((double)mx + my) * (nz - 4) + m->nrl + m->nc);
   const int gather = block * (int)std::min((double)kGatherRounds, std::max(1.0, std::floor(gathered / block / resident)));
   for (int s = 0; s < nslab; ++s) {
     const int c0 = 1 + s * B, c1 = std::min(c0 + B, nz - 1);          // planes
@@ -913,7 +914,8 @@ hyb_status build_plan(hyb_mesh* m, int nslots) {
         for (int e = 0; e < xy; e += per) add(3, s, e, std::min(e + per, xy), end);
     const int ez = (mz + 7) / 8;
     for (int e = 0; e < ez; e += per) add(2, s, e, std::min(e + per, ez), 0);
-    const long long nf = ((s == 0 ? 1LL : 0) + (s == nslab - 1 ? 1LL : 0)) * mx * my + 2LL * (mx + my) * mz;
+    const long long nf = ((s == 0 ? 1LL : 0) + (s == nslab - 1 ? 1LL : 0)) * mx * my + 2LL * (mx + (long long)my) * mz;
+    if (nf + gather >= 1LL << 32) return fail(HYB_ERR_ARG, "lattice face too large");
     for (long long f = 0; f < nf; f += gather) add(1, s, f, std::min(f + gather, nf), 0);
     if (m->nc > 0) {
       int* r = &rslab[4 * (size_t)s];
@@ -971,12 +973,8 @@ void base_args(const hyb_mesh* m, SweepArgs<T>& A, double dt, int nslots) {
   const double h = m->ani ? m->hv[0] : m->d.h;
   A.c2 = (T)(dt * dt / (h * h));
   A.r = (T)((h - dt) / (h + dt));
-  // the generic kernel: lattices without an interior, and beyond the sweep
-  // kernel's 32-bit item indices or the tile kernel's 32-bit offsets
+  // the generic kernel: lattices without an interior, or beyond the tile kernel's offsets
   A.small = (m->n[0] < 5 || m->n[1] < 5 || m->n[2] < 5) ? 1 : 0;
-  if (m->d.precision == HYB_FP64 && m->nc == 0 &&
-      ((long long)m->n[0] * m->n[1] + (m->n[0] + (long long)m->n[1]) * kMaxMarch >= 1LL << 30 || m->n[2] >= 1 << 23))
-    A.small = 1;
   if (m->d.precision == HYB_FP32 && beyond_tiles(m->d)) A.small = 1;
   if (m->ani) {  // axis terms weighed by kap
     A.ani = 1;

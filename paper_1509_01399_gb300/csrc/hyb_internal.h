@@ -204,7 +204,7 @@ struct SweepArgs : StepArgs<T> {
   int split;         // a stage's rows above, at and below the item's are copied apart (wide rows) or as one run
   int ccen, yo, ncur, nstage;  // elements: first quad in a u^k stage, from row to row, of the u^k part, of a stage
   int nqx;           // x quads (16 bytes) holding nodes 1 .. nx - 2
-  const int4* sitems;  // (kind | slab << 8, first, end, z end)
+  const int4* sitems;  // (slab, first, end (both unsigned), kind | z end << 8)
   int snitems;
   const int* need;   // per slab: items that signal it at each level
   const int4* rslab; // per slab: first corner row, corner rows, first centre row, centre rows of the refined region

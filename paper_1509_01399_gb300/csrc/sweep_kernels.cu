@@ -730,11 +730,11 @@ __device__ __forceinline__ void face_pair(const SweepArgs<T>& A, const Slot<T>& 
 // One entry of a slab's list of nodes one step inside exactly one face, in
 // the order z faces (first and last slab), y faces, x faces.
 template <typename T, StepMode M, bool ANI>
-__device__ __forceinline__ void face_entry(const SweepArgs<T>& A, const Slot<T>& S, int si, int slab, int t) {
-  const int mx = A.nx - 4, my = A.ny - 4;
+__device__ __forceinline__ void face_entry(const SweepArgs<T>& A, const Slot<T>& S, int si, int slab, unsigned t) {
+  const unsigned mx = A.nx - 4, my = A.ny - 4;
   const int k0 = max(1 + slab * A.slabz, 2), k1 = min(1 + (slab + 1) * A.slabz, A.nz - 2);
-  const int mz = max(k1 - k0, 0);
-  const int nlo = slab == 0 ? mx * my : 0, nhi = slab == A.nslab - 1 ? mx * my : 0;
+  const unsigned mz = max(k1 - k0, 0);
+  const unsigned nlo = slab == 0 ? mx * my : 0, nhi = slab == A.nslab - 1 ? mx * my : 0;
   if (t < nlo + nhi) {
     const bool hi = t >= nlo;
     if (hi) t -= nlo;
@@ -874,7 +874,9 @@ __device__ __forceinline__ void refined_item(const SweepArgs<T>& A, const Slot<T
 // Queue entry of an item for the row threads.
 struct QItem {
   int si;  // -1: no more work
-  int kind, slab, first, end, zend;
+  int slab;
+  unsigned first, end;
+  int kind, zend;
 };
 
 // What bounds it and why it is built so.  FP64: the FP64 pipe (two lanes per SM
@@ -959,13 +961,13 @@ __global__ void __launch_bounds__(kMaxBlock + kServiceThreads, kSweepBlocksPerSm
       const int4 nq = entry(nit);  // (the next item's entry and the claim after it are on their way meanwhile)
       unsigned nnit = 0;
       if (lane == 0) nnit = atomicAdd(A.sync, 1u);
-      const int kind = q.x & 255, slab = q.x >> 8;
+      const int kind = q.w & 255, slab = q.x;
       if (l > 0 && !wait_level(A, need, si, slab, l)) {
         if (lane == 0) atomicExch(A.err, 1);
         ok = false;
       }
       if (lane == 0) {
-        Q2[b] = {si, kind, slab, q.y, q.z, q.w};
+        Q2[b] = {si, slab, (unsigned)q.y, (unsigned)q.z, kind, q.w >> 8};
         mbar_arrive(B.qfull + b);
         if (kind == kInterior && ok) {
           fence_proxy_async_global();  // (other blocks' stores to the planes, acquired above, before the copies)
@@ -995,13 +997,13 @@ __global__ void __launch_bounds__(kMaxBlock + kServiceThreads, kSweepBlocksPerSm
       if (q.kind == kInterior) {
         interior_item<T, M, TEL, ANI>(A, S, &B, ring, rp, q.si, q.slab, q.first);
       } else if (q.kind == kFace) {
-        for (int r = q.first + t; r < q.end; r += rows) face_entry<T, M, ANI>(A, S, q.si, q.slab, r);
+        for (unsigned r = q.first + t; r < q.end; r += rows) face_entry<T, M, ANI>(A, S, q.si, q.slab, r);
       } else if (q.kind == kRefined) {
         if constexpr (!TEL && !ANI) refined_item<T, M != kForward>(A, S, q.si, q.slab, q.first, q.end);
       } else {
-        const int e = q.first + (t >> 7);  // one tile per 128 threads
+        const int e = (int)q.first + (t >> 7);  // one tile per 128 threads
         EdgeTile E = {-2, 0, 0, 0};
-        if (e < q.end) {
+        if (e < (int)q.end) {
           const int by = (A.ny - 4 + 15) / 16, p = e - 1;
           if (q.kind == kEdgeZ) {
             const int k0 = max(1 + q.slab * A.slabz, 2), k1 = min(1 + (q.slab + 1) * A.slabz, A.nz - 2);
