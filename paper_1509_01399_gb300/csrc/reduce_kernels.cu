@@ -68,12 +68,14 @@ __device__ __forceinline__ double widen(double x) { return x; }
 // w (a - b) rounded to FP32, w = wh + wl and d = a - b: the difference as s + e
 // and the leading product as p + q exactly, the small terms summed before they
 // meet p (within 2^-46 of the rounded FP64 product); the FP64 product where the
-// error terms would not be exact.
+// error terms would not be exact.  The roundings are written out, as a fused
+// last sum would count q twice.
 __device__ __forceinline__ float product(float a, float b, float wh, float wl, double w, double d) {
-  const float s = a - b, v = s - a, e = (a - (s - v)) + (-b - v);
-  const float p = wh * s;
-  if (!(fabsf(p) > 1e-30f && fabsf(p) < 1e30f && fabsf(s) < 1e30f) && s != 0.f) return product_any(w, d);
-  return p + (fmaf(wh, s, -p) + (wl * s + wh * e));
+  const float s = __fsub_rn(a, b), v = __fsub_rn(s, a);
+  const float e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, v)), __fsub_rn(-b, v));
+  const float p = __fmul_rn(wh, s);
+  if (!(fabsf(p) > 1e-30f && fabsf(p) < 1e30f && fabsf(s) < 1e30f)) return s == 0.f ? 0.f : product_any(w, d);
+  return __fadd_rn(p, fmaf(wh, s, -p) + (wl * s + wh * e));
 }
 __device__ __forceinline__ double product(double, double, float, float, double w, double d) { return w * d; }
 
@@ -109,7 +111,8 @@ __global__ void __launch_bounds__(kReduceThreads) misfit_kernel(const MisfitGeom
       if (cq == 0 || cq == g.nq[s] - 1) m *= 0.5;
     }
     w[q] = g.wt * m;
-    wh[q] = (float)w[q];
+    // (weights whose low part would be rounded or overflow take the FP64 product: product() of a NaN)
+    wh[q] = w[q] > 1e-30 && w[q] < 1e30 ? (float)w[q] : nanf("");
     wl[q] = (float)(w[q] - (double)wh[q]);
     sq[q] = 0.0;
   }
