@@ -342,18 +342,15 @@ void set_wave(const hyb_mesh* m, Slot<T>& S, const hyb_source& src, int k, doubl
     sd[a] = w.d[a] * (m->ani ? m->hv[a] : h);  // the delay d . (x - x0) axis by axis
     S.si0[a] = w.i0[a];
   }
-  const double t1 = 2.0 * M_PI / src.omega;
   if constexpr (sizeof(T) == 8) {
-    S.pulse = {k * dt, {sd[0], sd[1], sd[2]}, src.omega, t1};
+    S.pulse = {k * dt, {sd[0], sd[1], sd[2]}, src.omega, 2.0 * M_PI / src.omega};
   } else {
     auto split = [](float (&f)[2], double v) {
       f[0] = (float)v;
       f[1] = (float)(v - (double)f[0]);
     };
-    split(S.pulse.st, k * dt);
-    for (int a = 0; a < 3; ++a) split(S.pulse.sd[a], sd[a]);
-    split(S.pulse.omega, src.omega);
-    split(S.pulse.t1, t1);
+    split(S.pulse.ph, src.omega * (k * dt));
+    for (int a = 0; a < 3; ++a) split(S.pulse.pd[a], src.omega * sd[a]);
   }
 }
 

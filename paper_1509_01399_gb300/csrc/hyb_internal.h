@@ -47,14 +47,16 @@ constexpr double kGradPairScale = 6.0;
 constexpr int kReduceThreads = 256;
 
 // A slot's pulse at t_k: its time t_k, the delay per index step h d, omega and
-// the end t1; for FP32 fields as unevaluated sums of two FP32 numbers.
+// the end t1; for FP32 fields the phases omega t_k and omega h d (which no unit
+// of length or time takes out of FP32's range) as unevaluated sums of two FP32
+// numbers.
 template <typename T>
 struct Pulse {
   double st, sd[3], omega, t1;
 };
 template <>
 struct Pulse<float> {
-  float st[2], sd[3][2], omega[2], t1[2];
+  float ph[2], pd[3][2];
 };
 
 // One problem (one source of one mesh) at one time level.  A sweep launch gets

@@ -40,29 +40,29 @@ __device__ __forceinline__ double src_term(const Slot<double>& S, int f, int i, 
   return S.sf[f] * sin(p.omega * s);
 }
 
-// FP32 fields: the delay and omega times it in pairs of FP32 numbers (Dekker's and
-// Knuth's exact product and sum), to about 2^-45 of the delay's terms before the one
-// rounding of the pulse's argument.  In FP64 they are a dependent chain of a dozen
-// operations on a pipe of two lanes per SM and clock, in the warps next to the
+// FP32 fields: the phase omega (t_k - d . (x - x0)) in pairs of FP32 numbers
+// (Dekker's and Knuth's exact product and sum), to about 2^-45 of its terms before
+// the one rounding of the pulse's argument.  In FP64 the delay is a dependent chain of a
+// dozen operations on a pipe of two lanes per SM and clock, in the warps next to the
 // flux faces, for which a whole level then waits: 250 x 171 x 215, a diagonal
 // wave through three faces, 41.8 -> 35.4 us a forward level; 193^3, four sources,
-// 107.6 -> 101.2; 129^3 through z, 9.37 -> 9.01 (arguments against 64 bits: the same
-// largest error, 2.4e-7, as FP64 rounded once).
+// 107.6 -> 101.2; 129^3 through z, 9.37 -> 9.01.
 __device__ __forceinline__ float src_term(const Slot<float>& S, int f, int i, int j, int k) {
+  constexpr float kEnd[2] = {6.28318548f, -1.74845553e-7f};  // 2 pi
   const Pulse<float>& p = S.pulse;
   const int q[3] = {i, j, k};
-  float s = p.st[0], lo = p.st[1];
+  float s = p.ph[0], lo = p.ph[1];
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
     const float n = (float)(q[a] - S.si0[a]);
-    const float m = __fmul_rn(p.sd[a][0], n), e = fmaf(p.sd[a][1], n, fmaf(p.sd[a][0], n, -m));
+    const float m = __fmul_rn(p.pd[a][0], n), e = fmaf(p.pd[a][1], n, fmaf(p.pd[a][0], n, -m));
     const float t = __fsub_rn(s, m), b = __fsub_rn(t, s);
     lo += __fsub_rn(__fsub_rn(s, __fsub_rn(t, b)), __fadd_rn(m, b)) - e;
     s = t;
   }
   const float v = __fadd_rn(s, lo), r = __fadd_rn(__fsub_rn(s, v), lo);
-  if (!(v >= 0.f && __fsub_rn(v, p.t1[0]) + (r - p.t1[1]) <= 0.f)) return 0.f;
-  return S.sf[f] * sinf(fmaf(p.omega[0], v, fmaf(p.omega[0], r, p.omega[1] * v)));
+  if (!(v >= 0.f && __fsub_rn(v, kEnd[0]) + (r - kEnd[1]) <= 0.f)) return 0.f;
+  return S.sf[f] * sinf(v);
 }
 
 // Sum of the flux terms of the faces in `faces` (bits) that carry the flux.
