@@ -483,10 +483,12 @@ constexpr size_t kFieldPad = 64;
 // others (131 x 118 x 143 FP64, two sources, forward / transposed level:
 // 0.175 / 0.341 ms with one item a block, 0.144 / 0.262 with three, 0.132 /
 // 0.197 with six, 0.133 / 0.189 with ten).
-// Entries a thread of a face or refined item takes at most.
-constexpr int kGatherRounds = 4;
 constexpr int kMaxMarch = 16;
 constexpr double kItemsPerBlock = 8.0;
+// Entries a thread of a face or refined item takes at most.
+constexpr int kGatherRounds = 4;
+// Items of a level per SM up to which a sweep gets one block per SM.
+constexpr double kLoneItemsPerSm = 3.6;
 
 // P1 element of a tetrahedron (vertex coordinates X[4][3]): volume and
 // stiffness K_ij = |K| grad phi_i . grad phi_j (Sec. 7.2), a = 1.
@@ -938,6 +940,14 @@ hyb_status build_plan(hyb_mesh* m, int nslots) {
   P.block = block;
   P.nitems = (int)nitems;
   P.grid = (int)std::min((double)resident, 2.0 * P.nitems * nslots);
+  // Small levels of one or two slots (their items are a chain of short waits) get one
+  // block per SM: faster alone, and other streams' sweeps find room beside them.  A
+  // gradient in ms with all resident blocks / one per SM, alone and four at once on
+  // streams of their own: 33^3 (206 items a level) 6.66 / 6.26 and 4.94 / 3.05, 49^3 (406)
+  // 3.69 / 3.15 and 3.61 / 2.50, 57^3 (535) 4.22 / 3.91; 150 forward levels of 57^3 1.90 /
+  // 1.95, of 65^3 (802) 1.70 / 2.13; three slots of 37^3 1.87 / 2.04, four of 25^3 2.87 /
+  // 3.30.
+  if (nslots <= 2 && P.nitems * (double)nslots <= kLoneItemsPerSm * m->nsm) P.grid = std::min(P.grid, m->nsm);
   return HYB_OK;
 }
 
