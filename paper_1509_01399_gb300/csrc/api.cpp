@@ -127,10 +127,10 @@ struct hyb_mesh {
   SweepPlan plans[kMaxSlots + 1];
   int nsm = 0;                  // SMs of the device
   DevBuf table;                 // the sweep launch's slots at every level
-  // tile kernel: interior work items of the forward / transposed step per slot
-  // count; built once and kept
-  DevBuf items[2][kMaxSlots + 1];
-  int nitems[2][kMaxSlots + 1] = {};
+  // tile kernel: interior work items of the forward / transposed step (the same of
+  // batches) per slot count; built once and kept
+  DevBuf items[4][kMaxSlots + 1];
+  int nitems[4][kMaxSlots + 1] = {};
   int bps = 0;                  // its resident blocks per SM
   std::vector<int> rcorner, rcentre;  // refined corner rows / centres below each plane (prefix counts)
   SweepGraph graphs[3];
@@ -381,26 +381,33 @@ void step_geometry(const hyb_mesh* m, int* npb, int* ntx, int* nedge) {
 
 // Waves of resident interior blocks the work items are cut for, by the tile
 // levels of work there are per resident block (measured: us a forward /
-// transposed level).
+// transposed level; ms a gradient).
 //  * up to 40: one for a single slot (a block's first level waits for its planes,
 //    so long items pay off: 129^3 9.6 / 10.1 against 10.7 / 10.5 with two; 161^3
 //    15.3 / 17.7 against 16.6 / 17.7), and for several up to 6 (81^3, three, 11.0 /
-//    13.4 against 11.8 / 13.5); two for several slots from there (the edge tiles'
+//    13.4 against 11.8 / 13.5); two for several sources from there (the edge tiles'
 //    blocks, slot by slot, and the last slot's items leave a single wave uneven:
-//    65^3, eight, 17.9 / 17.6 -> 15.3 / 16.2; 97^3, six, 30.6 / 38.5 -> 28.1 / 33.9;
-//    161^3, two, 38.0 / 41.5 -> 33.5 / 34.5);
+//    97^3, six, 30.6 / 38.5 -> 28.1 / 33.9; 161^3, two, 38.0 / 41.5 -> 33.5 / 34.5);
+//    one for batches, which the serving engine's workers run side by side on streams
+//    of their own, where the planes read twice and the second fill of the pipelines cost
+//    more than the evenness gives (four at once, ms a batch, one / two waves: eight of
+//    65^3 4.45 / 4.97, six of 97^3 5.16 / 5.43, two of 129^3 2.72 / 3.05; alone 6.23 / 5.73,
+//    6.84 / 6.33, 3.77 / 3.48);
 //  * up to 60: three (257^3 refined, one source, 66 / 69 against 70 / 73 with five);
 //  * beyond: five, or items of about 35 levels if those are shorter, so that the
 //    items running together stay within one slab and find each other's halos in
 //    L2 (against three: 193^3 telegraph, four sources, 119 / 116 -> 110 / 110;
 //    257^3 refined, three sources, 183 / 199 -> 178 / 196; eight, 493 / 551 ->
-//    452 / 502).
-double step_waves(double levels_per_block, int nslots) {
-  if (levels_per_block <= 40.0) return nslots > 1 && levels_per_block > 6.0 ? 2.0 : 1.0;
+//    452 / 502; four at once on streams of their own 1 - 2 % faster too).
+constexpr double kFewLevels = 6.0, kSmallLevels = 40.0;
+double step_waves(double levels_per_block, int nslots, bool batch) {
+  if (levels_per_block <= kSmallLevels) return nslots > 1 && !batch && levels_per_block > kFewLevels ? 2.0 : 1.0;
   if (levels_per_block <= 60.0) return 3.0;
   return std::max(5.0, levels_per_block / 35.0);
 }
 
+// Cost of a block of edge tiles (build_items), in levels of a plain tile.
+constexpr double kEdgeBlockCost = 3.3;
 constexpr double kZFaceLevelCost = 3.5;
 
 // Interior work items of one step launch, one per block: (slot, tile, z0,
@@ -438,21 +445,45 @@ std::vector<int> build_items(const hyb_mesh* m, int nslots, bool adjoint) {
       }
   const double resident = (double)std::max(m->nsm, 1) * std::max(m->bps, 1);
   const double levels_per_block = (double)tiles.size() * (nz - 2) / resident;
-  const double target = total / (resident * step_waves(levels_per_block, nslots));
+  const double target = total / (resident * step_waves(levels_per_block, nslots, m->batch));
   // planes of an item and the ones next to it: 32-bit offsets (beyond_tiles leaves at least one)
   const long long most = ((1LL << 31) - 1) / ((long long)m->px * ny) - 1;
-  std::vector<std::pair<double, std::array<int, 4>>> items;
-  for (const Tile& t : tiles) {
-    double acc = 0.0;
-    int z0 = 1;
-    for (int k = 1; k <= nz - 2; ++k) {
-      acc += t.base + ((k >= zf0 && k <= zf1) ? t.extra : 0.0) + ((k == 1 || k == nz - 2) ? kZFaceLevelCost : 0.0);
-      if (acc >= target || k - z0 + 1 >= most || k == nz - 2) {
-        items.push_back({acc, {t.si, t.tile, z0, k + 1}});
-        z0 = k + 1;
-        acc = 0.0;
+  using Items = std::vector<std::pair<double, std::array<int, 4>>>;
+  auto cut = [&](double target) {
+    Items items;
+    for (const Tile& t : tiles) {
+      double acc = 0.0;
+      int z0 = 1;
+      for (int k = 1; k <= nz - 2; ++k) {
+        acc += t.base + ((k >= zf0 && k <= zf1) ? t.extra : 0.0) + ((k == 1 || k == nz - 2) ? kZFaceLevelCost : 0.0);
+        if (acc >= target || k - z0 + 1 >= most || k == nz - 2) {
+          items.push_back({acc, {t.si, t.tile, z0, k + 1}});
+          z0 = k + 1;
+          acc = 0.0;
+        }
       }
     }
+    return items;
+  };
+  Items items = cut(target);
+  if (m->batch && nslots > 1 && levels_per_block > kFewLevels && levels_per_block <= kSmallLevels) {
+    // the edge tiles' blocks come first, and items that find no room beside them wait
+    // for their end: longer items that leave them room, where that lengthens them by less
+    // than such a block costs (ms a batch, alone and four at once: eight of 65^3 6.23 ->
+    // 5.63 and 4.45 -> 4.52, two of 129^3 3.77 -> 3.60 and 2.72 -> 2.70; where it lengthens
+    // them by more: six of 97^3 6.84 -> 6.87 and 5.16 -> 5.70, sixteen of 65^3 5.56 -> 6.59 and
+    // 4.32 -> 4.44)
+    int npb, ntx_, nedge;
+    step_geometry(m, &npb, &ntx_, &nedge);
+    const double room = resident - (nedge + 1) / 2 * nslots;
+    auto longest = [](const Items& q) {
+      double l = 0.0;
+      for (const auto& it : q) l = std::max(l, it.first);
+      return l;
+    };
+    Items fit = items;
+    for (double t = target; fit.size() > room && t < 2.0 * target;) fit = cut(t *= 1.01);
+    if (fit.size() <= room && longest(fit) - longest(items) <= kEdgeBlockCost) items = fit;
   }
   // by source, then by z slab, then by tile: the items of one source run
   // together, and the blocks resident at one time cover one slab of
@@ -841,7 +872,7 @@ hyb_status step_maps(const hyb_mesh* m, SweepArgs<float>& A, const DevBuf& field
 // Work items of the step launches with `nslots` slots (built and uploaded the
 // first time this slot count is used, outside any captured sweep).
 hyb_status step_items(hyb_mesh* m, SweepArgs<float>& A, int nslots, bool adjoint) {
-  const int d = adjoint ? 1 : 0;
+  const int d = (adjoint ? 1 : 0) + (m->batch ? 2 : 0);
   DevBuf& buf = m->items[d][nslots];
   if (!buf.p) {
     const std::vector<int> host = build_items(m, nslots, adjoint);
