@@ -77,7 +77,7 @@ struct SweepPlan {
   DevBuf buf;                          // items, rslab, need, sync (element offsets below)
   size_t rslab = 0, need = 0, sync = 0;
   int nitems = 0, nslab = 0, slabz = 0, block = 0, grid = 0;
-  int ns = 0, smem = 0, split = 0, ccen = 0, yo = 0, ncur = 0, nstage = 0;  // ring (StepArgs)
+  int ns = 0, smem = 0, split = 0, ccen = 0, yo = 0, ncur = 0, nstage = 0;  // ring (SweepArgs)
 };
 
 }  // namespace

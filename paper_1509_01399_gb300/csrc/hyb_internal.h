@@ -191,7 +191,7 @@ struct SweepArgs : StepArgs<T> {
   // items, one block at a time each; `sitems` lists the items of one level of
   // one slot in slab order (the same for every slot).
   int nlev;
-  int k0, dir;       // time index of the first step (as in Slot::st), +1 / -1 per level
+  int k0, dir;       // time index of the first step (as in Slot::pulse), +1 / -1 per level
   int ring0;         // ring slot (level mod 3) of `cur` at the first level
   int abc_mask;      // absorbing faces of the mesh
   double dt;

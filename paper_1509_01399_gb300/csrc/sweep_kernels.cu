@@ -353,8 +353,7 @@ __device__ __forceinline__ T inline_face(const Slot<T>& S, T rf, T c2, int f, T 
 // The rows of one warp through an interior item's planes.  FEM: the warp has
 // FEM-owned nodes in the item (edge weights, history, pairing); the other
 // warps run the short loop.  Every lane computes all of its quad's nodes and
-// stores those that are the item's; with both x faces inline that is the whole
-// quad of a row (its x face node too), so that no lane leaves the common path.
+// stores those that are the item's.
 template <typename T, StepMode M, bool TEL, bool ANI, bool FEM>
 __device__ __forceinline__ void interior_march(const SweepArgs<T>& A, const Slot<T>& S, Bars* B, const T* ring,
                                                RingPos& rp, int si, const InteriorRun<T>& R) {
@@ -370,8 +369,6 @@ __device__ __forceinline__ void interior_march(const SweepArgs<T>& A, const Slot
   const int px = A.px, yo = A.yo, nstage = A.nstage, ns = A.ns;
   const long long pl = (long long)px * A.ny;
   const int inl = inline_faces<T, M>(S);
-  const bool xin = (inl & 3) == 3;  // both x faces inline
-  const int em = A.nx - 2 - i0;     // element next to the high x face (on quads that hold it)
   // elements: off the x faces' neighbours, FEM-owned
   unsigned mid = 0, fem = 0;
 #pragma unroll
@@ -383,15 +380,12 @@ __device__ __forceinline__ void interior_march(const SweepArgs<T>& A, const Slot
   const int fy = j == 1 ? 2 : (j == A.ny - 2 ? 3 : -1);  // the y face next to the row
   if (!valid) mid = 0;
   const bool anyfy = __any_sync(0xffffffffu, fy >= 0);
-  const bool xlo = valid && fy < 0 && i0 == 0 && (inl & 1), xhi = valid && fy < 0 && em < V && (inl & 2);
   // elements written on the planes off the z faces
-  unsigned wr0 = fy >= 0 ? ((inl >> fy) & 1 ? mid : 0) : mid | (xlo ? 2u : 0u) | (xhi ? 1u << em : 0u);
-  if (valid && fy < 0 && xin) wr0 = kAll;
+  const unsigned wr0 = fy < 0 || ((inl >> fy) & 1) ? mid : 0;
   const int so = (int)(i0 + (long long)px * j - R.a0);  // this quad in the item's run
   const T* const base = ring + A.ccen + so;
   const int pvo = A.ncur - A.ccen;
-  const T c2 = A.c2, rx = ANI ? A.ra[0] : A.r;
-  const bool obs_x = S.obs_face < 2 && (ADJ ? S.obs_r != nullptr : S.obs_w != nullptr);
+  const T c2 = A.c2;
   T* o = S.next + (i0 + (long long)px * j + pl * R.za);
   const int last = A.fl[0] + A.un[0] - 1;  // x of the last voxel origin
   const bool over = PAIR && i0 + V - 1 <= last;
@@ -461,9 +455,6 @@ __device__ __forceinline__ void interior_march(const SweepArgs<T>& A, const Slot
         }
       }
     }
-    T oxl = T(0), oxh = T(0);  // cotangent on the x faces
-    if (ADJ && obs_x && xlo && S.obs_face == 0) oxl = S.obs_r[j + A.ny * k];
-    if (ADJ && obs_x && xhi && S.obs_face == 1) oxh = S.obs_r[j + A.ny * k];
     T ym[V], yp[V];
     ldq(ym, C - yo);
     ldq(yp, C + yo);
@@ -582,40 +573,6 @@ __device__ __forceinline__ void interior_march(const SweepArgs<T>& A, const Slot
                                            ADJ && obs && S.obs_r ? S.obs_r[idx + e] : T(0));
           ob[e] = vb;
           if (!ADJ && obs && S.obs_w) S.obs_w[idx + e] = vb;
-        }
-      }
-    }
-    if (inl & 3) {  // (uniform) the x face nodes
-      if (fz < 0) {
-        const T kx = ANI ? A.kapt[0] : T(1);
-        T v1 = val[1], blo = inline_face<T, ADJ>(S, rx, c2, 0, c[0], c[1], v1,
-                                                 FEM && ADJ && (fm & 2) ? wx[0] : kx, oxl);
-        T vm = val[0], cm = c[0], ub = c[1], wm = wx[0];  // the high side's m and b
-#pragma unroll
-        for (int e = 1; e < V; ++e)
-          if (em == e) {
-            vm = val[e];
-            cm = c[e];
-            ub = e < V - 1 ? c[e < V - 1 ? e + 1 : e] : xr;
-            wm = wx[e];
-          }
-        const T bhi = inline_face<T, ADJ>(S, rx, c2, 1, ub, cm, vm, FEM && ADJ && ((fm >> (em & 7)) & 1) ? wm : kx, oxh);
-        if (xlo) {
-          val[0] = blo;
-          val[1] = v1;
-        }
-        if (xhi) {
-#pragma unroll
-          for (int e = 0; e < V; ++e) {
-            if (em == e) val[e] = vm;
-            if (em + 1 == e) val[e] = bhi;
-          }
-          if (em == V - 1 || !xin) o[em + 1] = bhi;
-        }
-        if (xlo && !xin) o[0] = blo;
-        if (!ADJ && obs_x) {
-          if (xlo && S.obs_face == 0) S.obs_w[j + A.ny * k] = blo;
-          if (xhi && S.obs_face == 1) S.obs_w[j + A.ny * k] = bhi;
         }
       }
     }
