@@ -77,6 +77,7 @@ struct SweepPlan {
   DevBuf buf;                          // items, rslab, need, sync (element offsets below)
   size_t rslab = 0, need = 0, sync = 0;
   int nitems = 0, nslab = 0, slabz = 0, block = 0, grid = 0;
+  int levels = 0;                      // of one launch
   int ns = 0, smem = 0, split = 0, ccen = 0, yo = 0, ncur = 0, nstage = 0;  // ring (SweepArgs)
 };
 
@@ -884,13 +885,22 @@ hyb_status step_items(hyb_mesh* m, SweepArgs<float>& A, int nslots, bool adjoint
   return HYB_OK;
 }
 
-// Levels of one sweep launch at most: about this many node-steps, so that
-// sweeps on other streams get their turn.
-constexpr double kLaunchNodeSteps = 5e9;
+// Levels whose slots are made at once (the table's size): about this many node-steps.
+constexpr double kTableNodeSteps = 5e9;
 
-int launch_levels(const hyb_mesh* m, int nsrc) {
-  return (int)std::min(1e6, std::max(1.0, kLaunchNodeSteps / ((double)m->Np * nsrc)));
+int table_levels(const hyb_mesh* m, int nsrc) {
+  return (int)std::min(1e6, std::max(1.0, kTableNodeSteps / ((double)m->Np * nsrc)));
 }
+
+// Levels of one sweep launch, which holds every SM while it runs: about this many
+// node-steps, so that other streams get their turn, but enough levels that its first
+// and last ones, which leave blocks idle (0.3 to 0.7 of a level's time), cost 1 to 2 %.
+// A 33^3 FP32 gradient of 100 steps (1.05 ms alone) beside an FP64 inversion on another
+// stream, in ms, with launches of 5e9 / 5e7 / 1e7 node-steps: 65^3 212 / 43 / 10.8, 131 x
+// 118 x 143, two sources, 188 / 19 / 4.6; the inversions' own time 0 / 2.5 / 12 % (the
+// latter's; ten and two levels a launch) longer.
+constexpr double kLaunchNodeSteps = 1.5e7;
+constexpr int kLaunchLevels = 24;
 
 // The plan for `nslots` slots (built and uploaded the first time this slot
 // count is used, outside any captured sweep): the ring of plane stages, the
@@ -978,7 +988,13 @@ hyb_status build_plan(hyb_mesh* m, int nslots) {
   // 3.69 / 3.15 and 3.61 / 2.50, 57^3 (535) 4.22 / 3.91; 150 forward levels of 57^3 1.90 /
   // 1.95, of 65^3 (802) 1.70 / 2.13; three slots of 37^3 1.87 / 2.04, four of 25^3 2.87 /
   // 3.30.
-  if (nslots <= 2 && P.nitems * (double)nslots <= kLoneItemsPerSm * m->nsm) P.grid = std::min(P.grid, m->nsm);
+  // (and one launch for all levels, as they leave that room)
+  if (nslots <= 2 && P.nitems * (double)nslots <= kLoneItemsPerSm * m->nsm) {
+    P.grid = std::min(P.grid, m->nsm);
+    P.levels = 1 << 30;
+  } else {
+    P.levels = std::max(kLaunchLevels, (int)std::min(1e9, kLaunchNodeSteps / ((double)m->Np * nslots)));
+  }
   return HYB_OK;
 }
 
@@ -1061,7 +1077,7 @@ void base_args(const hyb_mesh* m, SweepArgs<T>& A, double dt, int nslots) {
 template <typename T>
 hyb_status plan_args(hyb_mesh* m, SweepArgs<T>& A, int nslots, int nsteps) {
   HYB_TRY(build_plan(m, nslots));
-  HYB_TRY(ensure(m, m->table, (size_t)std::min(nsteps, launch_levels(m, nslots)) * nslots * sizeof(Slot<T>)));
+  HYB_TRY(ensure(m, m->table, (size_t)std::min(nsteps, table_levels(m, nslots)) * nslots * sizeof(Slot<T>)));
   A.table = (Slot<T>*)m->table.p;
   const SweepPlan& P = m->plans[nslots];
   A.nslab = P.nslab;
@@ -1138,7 +1154,7 @@ template <typename T>
 hyb_status launch_piece(hyb_mesh* m, const SweepArgs<T>& A, StepMode mode, cudaStream_t st) {
   if constexpr (sizeof(T) == 8) {
     const SweepPlan& P = m->plans[A.nslots];
-    m->launches += launch_sweep(A, mode, P.block, P.grid, P.smem, st) - 1;
+    m->launches += launch_sweep(A, mode, P.block, P.grid, P.smem, P.levels, st) - 1;
     HYB_LAUNCHED(m);
   }
   return HYB_OK;
@@ -1197,7 +1213,7 @@ hyb_status forward_levels(hyb_mesh* m, SweepArgs<T>& A, const hyb_source* src, i
                           int n, T* trace, T* hl, T* chl, int nh, cudaStream_t st) {
   const long long lvl = (long long)nsrc * m->hbox, clvl = (long long)nsrc * m->nc;
   const bool sweep = path_of(A) == Path::kSweep;
-  const int most = sweep ? launch_levels(m, nsrc) : 1;
+  const int most = sweep ? table_levels(m, nsrc) : 1;
   for (int l = 0; l < n; l += most) {
     const int q = std::min(most, n - l);
     const bool h = hl && l < nh;
@@ -1519,7 +1535,7 @@ hyb_status adjoint_impl(hyb_mesh* m, const T* cot, int accumulate) {
     auto adj_steps = [&](int j, int n, const T* hl, const T* chl, int l0) -> hyb_status {
       SweepArgs<T>& B = paper ? Pp : A;
       const bool sweep = path_of(B) == Path::kSweep;
-      const int most = sweep ? launch_levels(m, nsrc) : 1;
+      const int most = sweep ? table_levels(m, nsrc) : 1;
       for (int l = 0; l < n; l += most) {
         const int q = std::min(most, n - l);
         const bool h = hl && l + q > l0;

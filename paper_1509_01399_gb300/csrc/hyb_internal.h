@@ -219,10 +219,10 @@ struct SweepArgs : StepArgs<T> {
 // pairing, and the paper's adjoint (forward rows on lambda with the pairing).
 enum StepMode { kForward = 0, kAdjoint = 1, kPaper = 2 };
 
-// A.nlev consecutive levels of every slot: fills A.table, then one launch of
-// the sweep kernel (blocks of `block` row threads and a producer warp, `smem`
-// bytes of ring each).  Returns the kernels launched.
-int launch_sweep(const SweepArgs<double>& a, StepMode mode, int block, int grid, int smem, cudaStream_t st);
+// A.nlev consecutive levels of every slot: fills A.table, then launches of the
+// sweep kernel of about `levels` each (blocks of `block` row threads and a producer
+// warp, `smem` bytes of ring each).  Returns the kernels launched.
+int launch_sweep(const SweepArgs<double>& a, StepMode mode, int block, int grid, int smem, int levels, cudaStream_t st);
 // One level of every slot by the tile kernel (edge tiles, interior tiles and
 // refined rows in one launch; `pair`: forward rows with the paper's adjoint's
 // pairing of A.s's history in it).

@@ -1008,8 +1008,7 @@ __global__ void __launch_bounds__(kMaxBlock + kServiceThreads, kSweepBlocksPerSm
 }  // namespace
 
 template <typename T, StepMode M>
-void launch_sweep_mode(const SweepArgs<T>& a, int block, int grid, int smem, cudaStream_t st) {
-  slots_kernel<T, M><<<(a.nlev * a.nslots + 127) / 128, 128, 0, st>>>(a);
+void launch_levels(const SweepArgs<T>& a, int block, int grid, int smem, cudaStream_t st) {
   if constexpr (M != kPaper) {
     if (a.ani) {
       sweep_kernel<T, M, false, true><<<grid, block + kServiceThreads, smem, st>>>(a);
@@ -1023,11 +1022,27 @@ void launch_sweep_mode(const SweepArgs<T>& a, int block, int grid, int smem, cud
   sweep_kernel<T, M, false, false><<<grid, block + kServiceThreads, smem, st>>>(a);
 }
 
-int launch_sweep(const SweepArgs<double>& a, StepMode mode, int block, int grid, int smem, cudaStream_t st) {
-  if (mode == kForward) launch_sweep_mode<double, kForward>(a, block, grid, smem, st);
-  else if (mode == kAdjoint) launch_sweep_mode<double, kAdjoint>(a, block, grid, smem, st);
-  else launch_sweep_mode<double, kPaper>(a, block, grid, smem, st);
-  return 2;
+template <typename T, StepMode M>
+int launch_sweep_mode(const SweepArgs<T>& a, int block, int grid, int smem, int levels, cudaStream_t st) {
+  slots_kernel<T, M><<<(a.nlev * a.nslots + 127) / 128, 128, 0, st>>>(a);
+  int n = 1;
+  const int parts = a.nlev / levels > 1 ? a.nlev / levels : 1;  // (even ones: short launches cost most)
+  levels = (a.nlev + parts - 1) / parts;
+  SweepArgs<T> b = a;
+  for (int l = 0; l < a.nlev; l += b.nlev, ++n) {
+    b.table = a.table + (size_t)l * a.nslots;
+    b.ring0 = (a.ring0 + a.dir * (l % 3) + 3) % 3;
+    b.nlev = a.nlev - l < levels ? a.nlev - l : levels;
+    launch_levels<T, M>(b, block, grid, smem, st);
+  }
+  return n;
+}
+
+int launch_sweep(const SweepArgs<double>& a, StepMode mode, int block, int grid, int smem, int levels,
+                 cudaStream_t st) {
+  if (mode == kForward) return launch_sweep_mode<double, kForward>(a, block, grid, smem, levels, st);
+  if (mode == kAdjoint) return launch_sweep_mode<double, kAdjoint>(a, block, grid, smem, levels, st);
+  return launch_sweep_mode<double, kPaper>(a, block, grid, smem, levels, st);
 }
 
 template <typename T, StepMode M, bool TEL, bool ANI>

@@ -102,3 +102,55 @@ def test_small_sweeps_share_the_gpu(H):
     three = min(max(at_once([sweep] * 3)) for _ in range(2))
     print("one sweep %.2f ms, three at once %.2f ms" % (one * 1e3, three * 1e3))
     assert three < 2.0 * one
+
+
+def test_small_pass_beside_an_fp64_inversion(H):
+    """A short FP32 gradient beside an FP64 inversion that fills the GPU takes less than
+    half of the inversion's time: the sweep's launches end often enough for it."""
+    import torch
+
+    def gradient(w, m, a, cot):
+        m.forward(a, w.sources, w.nsteps, w.dt)
+        m.adjoint(cot)
+        m.sync()
+
+    def ready(n, precision, nsteps):
+        w = synth.small_problem(n=n, fem=(tuple(v // 4 for v in n), tuple(3 * v // 4 for v in n)), nsteps=nsteps,
+                                omega=14.0, courant=0.8)
+        m = H.HybMesh.from_workload(w, precision=precision)
+        args = w, m, torch.full((w.n_unknown,), 1.5, device="cuda", dtype=torch.float64), m.new_trace(1, nsteps)
+        for _ in range(3):  # (the first calls allocate and capture)
+            gradient(*args)
+        return args
+
+    def timed(args):
+        t0 = time.perf_counter()
+        gradient(*args)
+        return time.perf_counter() - t0
+
+    big, small = [], []
+    loaded, done = threading.Event(), threading.Event()
+
+    def inversion():
+        with torch.cuda.stream(torch.cuda.Stream()):
+            args = ready((65, 65, 65), "fp64", 2000)
+            big.append(min(timed(args) for _ in range(3)))
+            loaded.set()
+            while not done.is_set():
+                gradient(*args)
+            args[1].close()
+
+    with torch.cuda.stream(torch.cuda.Stream()):
+        args = ready((33, 33, 33), "fp32", 100)
+        t = threading.Thread(target=inversion)
+        t.start()
+        try:
+            assert loaded.wait(60)
+            time.sleep(0.05)
+            small = sorted(timed(args) for _ in range(7))
+        finally:
+            done.set()
+            t.join()
+        args[1].close()
+    print("inversion alone %.1f ms, small pass beside it %.1f ms" % (big[0] * 1e3, small[3] * 1e3))
+    assert small[3] < 0.5 * big[0]
