@@ -88,7 +88,8 @@ typedef struct {
                           tetrahedra are bisected along their refinement edge,
                           the voxel diagonal, at a new centre node.  Marked
                           voxels need every corner at least 2 nodes from the
-                          outer faces. */
+                          outer faces, and the block fewer than 2^31 unknown
+                          voxels. */
   int64_t wait_cycles; /* limit, in SM clock cycles, of each bounded wait of
                           the step kernels for their staged planes and for
                           the earlier levels' work they build on (0: the

@@ -1883,6 +1883,9 @@ hyb_status hyb_mesh_create(const hyb_mesh_desc* d, void* stream, hyb_mesh** out)
   }
   if (d->precision == HYB_FP32 && beyond_tiles(*d) && (d->refine_mask || d->model == HYB_MODEL_TELEGRAPH))
     return fail(HYB_ERR_ARG, "lattice plane or FEM block too large for FP32 fields with refinement or the telegraph model");
+  if (fem && d->refine_mask && (double)(d->fem_hi[0] - d->fem_lo[0] - 2) * (d->fem_hi[1] - d->fem_lo[1] - 2) *
+                                       (d->fem_hi[2] - d->fem_lo[2] - 2) >= (double)(1LL << 31))
+    return fail(HYB_ERR_ARG, "refinement needs fewer than 2^31 unknown voxels");
   hyb_mesh* m = new (std::nothrow) hyb_mesh();
   if (!m) return fail(HYB_ERR_OOM, "host allocation failed");
   m->d = *d;
